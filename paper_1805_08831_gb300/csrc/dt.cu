@@ -906,6 +906,7 @@ struct dt_handle {
   uint64_t out_cap = 0;        // rows
   bool use_subdet = false;
   uint64_t cap_tets = 0;
+  uint64_t cap_lock = 0;     // owner words (a batch grows the store without them)
   uint32_t* freelist = nullptr;
   uint32_t* pending = nullptr;
   uint64_t cap_free = 0;
@@ -1007,7 +1008,7 @@ struct dt_handle {
   cudaEvent_t bev[4] = {nullptr, nullptr, nullptr, nullptr};
   cudaGraph_t bgraph = nullptr;             // the captured steady-state batch
   cudaGraphExec_t bexec = nullptr;
-  uint64_t bgraph_key[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+  std::vector<uint64_t> bgraph_key;         // what the captured graph was made for
   uint64_t bgraph_kernels = 0;              // kernels in the captured graph
   bool bgraph_used = false;                 // the last batch replayed the graph
   // learned scheduler
@@ -1138,16 +1139,21 @@ int reserve_tets(dt_handle* h, uint64_t total_pts) {
   double f = h->cfg.tet_capacity_factor > 0 ? h->cfg.tet_capacity_factor : 8.0;
   uint64_t need = (uint64_t)(f * (double)total_pts) + 4096;
   if (need > kMaxSlots) need = kMaxSlots;
-  if (need <= h->cap_tets) return DT_OK;
+  // after a batch the store may be large enough while it has no owner words and a shorter free
+  // list than this engine's
+  if (need <= h->cap_tets && h->cap_lock >= h->cap_tets) return DT_OK;
   unsigned long long bump = h->has_mesh ? h->st_host->bump : 0;
-  if (grow(h->tets, bump, need, h->stream) != cudaSuccess) return DT_ENOMEM;
-  // slots not yet handed out read as dead (v.x == v.y == 0): the asynchronous engine may read
-  // a slot through a freshly written pointer before its record arrives, and must never find an
-  // old, self-consistent mesh there
-  cudaMemsetAsync(h->tets + bump, 0, (need - bump) * sizeof(Tet), h->stream);
-  if (grow(h->claim, 2 * bump, 2 * need, h->stream) != cudaSuccess) return DT_ENOMEM;
-  // claim words of slots not yet handed out start at zero (below every priority)
-  cudaMemsetAsync(h->claim + 2 * bump, 0, 2 * (need - bump) * sizeof(unsigned long long), h->stream);
+  need = std::max(need, h->cap_tets);
+  if (need > h->cap_tets) {
+    if (grow(h->tets, bump, need, h->stream) != cudaSuccess) return DT_ENOMEM;
+    // slots not yet handed out read as dead (v.x == v.y == 0): the asynchronous engine may read
+    // a slot through a freshly written pointer before its record arrives, and must never find an
+    // old, self-consistent mesh there
+    cudaMemsetAsync(h->tets + bump, 0, (need - bump) * sizeof(Tet), h->stream);
+    if (grow(h->claim, 2 * bump, 2 * need, h->stream) != cudaSuccess) return DT_ENOMEM;
+    // claim words of slots not yet handed out start at zero (below every priority)
+    cudaMemsetAsync(h->claim + 2 * bump, 0, 2 * (need - bump) * sizeof(unsigned long long), h->stream);
+  }
   if (h->use_subdet) {
     // cache entries of slots not yet handed out read as invalid
     if (grow(h->subdet, 2 * bump, 2 * need, h->stream) != cudaSuccess) return DT_ENOMEM;
@@ -1157,11 +1163,13 @@ int reserve_tets(dt_handle* h, uint64_t total_pts) {
   cudaStreamSynchronize(h->stream);
   cudaFree(h->lock);
   h->lock = nullptr;
+  h->cap_lock = 0;
   if (cudaMalloc(&h->lock, need * sizeof(uint32_t)) != cudaSuccess) return DT_ENOMEM;
+  h->cap_lock = need;
   cudaMemsetAsync(h->lock, 0, need * sizeof(uint32_t), h->stream);
   // free list: the slots a round frees, plus every warp's private slots that the asynchronous
   // engine hands back when its launch ends
-  uint64_t nf = need / 4 + 4096 + (uint64_t)async_max_warps() * 160;
+  uint64_t nf = std::max<uint64_t>(need / 4 + 4096 + (uint64_t)async_max_warps() * 160, h->cap_free);
   uint64_t fold = h->has_mesh ? h->st_host->free_avail : 0;
   if (grow(h->freelist, fold, nf, h->stream) != cudaSuccess) return DT_ENOMEM;
   cudaFree(h->pending);
@@ -1962,11 +1970,18 @@ int batch_impl(dt_handle* h, const double* xyz, const uint64_t* off, uint32_t nc
   }
   // the steady state: sort, records, reset and the persistent launch, replayed from a CUDA graph
   // while the batch keeps its shape (same input buffer, cloud sizes, block shape and round size)
-  const uint64_t key[8] = {(uint64_t)(uintptr_t)xyz, N, nc, hash, (uint64_t)h->batch_W,
-                           (uint64_t)(h->batch_alpha * 1e6f), h->cfg.seed, (uint64_t)(h->gamma * 1e9)};
+  // (every buffer the graph names is part of the key: an insert in between may have moved some)
+  const void* const named[] = {xyz, h->pts, h->ptf, h->vflag, h->point_hint, h->tets, h->claim, h->freelist, h->pending,
+                               h->ows.keys, h->ows.k0, h->ows.k1, h->ows.v0, h->ows.v1, h->ows.rounds, h->ows.dup,
+                               h->ows.perm, h->ows.rank, h->ows.hist, h->ows.bad, h->bcid, h->bdup, h->blist_a,
+                               h->blist_b, h->blist_big, h->boff_dev, h->bclouds, h->border, h->bhint_f, h->bhint_c,
+                               h->bcbox, h->bstates, h->bws, h->bstats, h->bnext, h->beta};
+  std::vector<uint64_t> key = {N, nc, hash, h->cap_tets, h->cap_pts, h->cap_free, (uint64_t)h->batch_W, (uint64_t)(h->batch_alpha * 1e6f), h->cfg.seed,
+                               (uint64_t)(h->gamma * 1e9)};
+  for (const void* p : named) key.push_back((uint64_t)(uintptr_t)p);
   const bool use_graph = !std::getenv("DT_BATCH_NO_GRAPH");
   h->bgraph_used = false;
-  if (use_graph && !(h->bexec && std::equal(key, key + 8, h->bgraph_key))) {
+  if (use_graph && !(h->bexec && key == h->bgraph_key)) {
     if (h->bexec) cudaGraphExecDestroy(h->bexec);
     if (h->bgraph) cudaGraphDestroy(h->bgraph);
     h->bexec = nullptr;
@@ -1984,7 +1999,7 @@ int batch_impl(dt_handle* h, const double* xyz, const uint64_t* off, uint32_t nc
     }
     if (ok) ok = cudaGraphInstantiate(&h->bexec, h->bgraph, 0) == cudaSuccess;
     if (ok) {
-      std::copy(key, key + 8, h->bgraph_key);
+      h->bgraph_key = key;
       h->bgraph_kernels = g_kernel_launches - k0;
     } else {
       cudaGetLastError();  // capture unsupported here: run the same sequence eagerly

@@ -165,3 +165,20 @@ def test_repeated_batch_replays_its_graph_on_new_data():
         assert t.stats()["batch_graph"] == 1
     clouds = split(xyz2 * 3.0 - 1.0, off)
     assert_clouds_match(clouds, [new[int(c3[c]):int(c3[c + 1])] for c in range(30)])
+
+
+def test_insert_after_a_larger_batch_on_the_same_handle():
+    """A batch grows the tetrahedron store without the asynchronous engine's owner words: an
+    insert that follows on the handle has to bring them."""
+    xyz, off = synth.batched_clouds(12, 5, lo=50, hi=3000)
+    x = synth.uniform_cube(900, 6)
+    ref, _ = oracle.delaunay(x)
+    with dt.Triangulation(seed=0) as t:
+        t.batch(torch.from_numpy(xyz).cuda(), off)
+        t.clear()
+        t.insert(torch.from_numpy(x).cuda())
+        assert np.array_equal(t.tets_numpy(), ref)
+        t.batch(torch.from_numpy(xyz).cuda(), off)
+        t.clear()
+        t.insert(torch.from_numpy(x).cuda())
+        assert np.array_equal(t.tets_numpy(), ref)
