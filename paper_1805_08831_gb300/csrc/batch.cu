@@ -20,11 +20,6 @@ namespace dtg {
 
 namespace {
 
-unsigned grid_for(uint64_t n, int threads) {
-  uint64_t b = (n + threads - 1) / threads;
-  return (unsigned)std::max<uint64_t>(1, std::min<uint64_t>(b, 152ull * 16));
-}
-
 // Per-warp workspace: cavities up to kBatchCN tetrahedra and kBatchFN boundary facets.
 constexpr uint32_t kBatchHashN = 2048, kBatchCN = 512, kBatchFN = 512, kBatchEdgeN = 2048;
 constexpr uint32_t kBatchLongWalk = 1u << 14;  // walk limit of short retry lists
@@ -425,26 +420,6 @@ __global__ void k_batch_collect(const BatchCloud* clouds, uint32_t n_clouds, con
   }
 }
 
-// Key of a collected tetrahedron for the canonical order of a batch: (cloud, tetrahedron).
-__global__ void k_batch_tet_keys(const uint4* tets, uint64_t T, const unsigned long long* out_off, uint32_t n_clouds,
-                                 uint64_t* khi, uint64_t* klo, uint64_t* kcl, uint32_t* idx) {
-  for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < T;
-       i += (uint64_t)gridDim.x * blockDim.x) {
-    uint4 t = tets[i];
-    khi[i] = ((uint64_t)t.x << 32) | t.y;
-    klo[i] = ((uint64_t)t.z << 32) | t.w;
-    uint32_t lo = 0, hi = n_clouds;  // cloud: last c with out_off[c] <= i
-    while (hi - lo > 1) {
-      uint32_t mid = (lo + hi) / 2;
-      if (out_off[mid] <= i) lo = mid;
-      else hi = mid;
-    }
-    kcl[i] = lo;
-    idx[i] = (uint32_t)i;
-  }
-}
-
-
 // Hint grid of every cloud (8 cells per axis over its box) and the batch's FP32 error term
 // eta = 2^-44 max|x| (+ the spacing of FP32 subnormals), as the single-cloud engine sets it.
 __global__ void k_batch_prepare(BatchCloud* clouds, const double* __restrict__ cbox, uint32_t n_clouds,
@@ -550,12 +525,6 @@ void batch_collect(const BatchCloud* clouds, uint32_t n_clouds, const Tet* tets,
                    int canonical, cudaStream_t s) {
   k_batch_collect<<<std::min<uint32_t>(n_clouds, 152u * 8), 256, 0, s>>>(clouds, n_clouds, tets, pts, in_off, pass,
                                                                         counts, out_off, out, canonical);
-  ++g_kernel_launches;
-}
-
-void batch_tet_keys(const uint32_t* tets, uint64_t T, const unsigned long long* out_off, uint32_t n_clouds,
-                    uint64_t* khi, uint64_t* klo, uint64_t* kcl, uint32_t* idx, cudaStream_t s) {
-  k_batch_tet_keys<<<grid_for(T, 256), 256, 0, s>>>((const uint4*)tets, T, out_off, n_clouds, khi, klo, kcl, idx);
   ++g_kernel_launches;
 }
 

@@ -673,28 +673,6 @@ __global__ void k_count_seen(const uint8_t* seen, uint64_t n, unsigned long long
   if (m) atomicAdd(out, m);
 }
 
-__global__ void k_split_keys(const uint4* tets, uint64_t T, uint64_t* khi, uint64_t* klo, uint32_t* idx) {
-  for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < T;
-       i += (uint64_t)gridDim.x * blockDim.x) {
-    uint4 t = tets[i];
-    khi[i] = ((uint64_t)t.x << 32) | t.y;
-    klo[i] = ((uint64_t)t.z << 32) | t.w;
-    idx[i] = (uint32_t)i;
-  }
-}
-
-__global__ void k_gather_keys(const uint64_t* src, const uint32_t* idx, uint64_t T, uint64_t* dst) {
-  for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < T;
-       i += (uint64_t)gridDim.x * blockDim.x)
-    dst[i] = src[idx[i]];
-}
-
-__global__ void k_gather_tets(const uint4* src, const uint32_t* idx, uint64_t T, uint4* dst) {
-  for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < T;
-       i += (uint64_t)gridDim.x * blockDim.x)
-    dst[i] = src[idx[i]];
-}
-
 __global__ void k_eval_predicates(int kind, const double* pts, const int64_t* ids, int8_t* out, uint64_t n,
                                   DevState* st) {
   for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n;
@@ -904,6 +882,8 @@ struct dt_handle {
   uint64_t in_cap = 0;         // rows
   uint32_t* out_buf = nullptr; // dt_get_tets_host: the tetrahedra on the device before the copy out
   uint64_t out_cap = 0;        // rows
+  CanonWS canon;               // the canonical list's workspace
+  uint64_t mesh_pts = 0;       // vertices the mesh may hold (points whose records were built)
   bool use_subdet = false;
   uint64_t cap_tets = 0;
   uint64_t cap_lock = 0;     // owner words (a batch grows the store without them)
@@ -1093,6 +1073,7 @@ uint64_t device_bytes(const dt_handle* h) {
   b += h->cap_tets * (sizeof(Tet) + 16 + 4);                         // records, claim pair, owner word
   if (h->subdet) b += h->cap_tets * 2 * sizeof(float4);              // sub-determinant cache
   b += h->in_cap * 24 + h->out_cap * 16;                             // host entry points' buffers
+  b += canon_ws_bytes(h->canon);                                     // the canonical list's workspace
   b += h->cap_free * 8;                                              // free list and pending
   if (h->cell_hint_cb > 0) {
     const int cb = h->cell_hint_cb, cbc = cb > 3 ? cb - 3 : 1;
@@ -1657,6 +1638,7 @@ int insert_impl(dt_handle* h, const double* xyz, uint64_t n, bool allow_async = 
   k_build_pts<<<grid_for(n, 256), 256, 0, s>>>(xyz, h->ows.perm, h->ows.dup, n, base, h->pts, h->ptf,
                                                 h->vflag, h->point_hint);
   ++g_kernel_launches;
+  h->mesh_pts = base + n;
   h->last_base = base;
   h->risky_ready = false;
   h->prank_ready = false;
@@ -2069,6 +2051,28 @@ int batch_impl(dt_handle* h, const double* xyz, const uint64_t* off, uint32_t nc
   return degenerate == nc ? DT_EDEGENERATE : DT_OK;
 }
 
+// The rows of the handle's own device buffer for tetrahedra (grown on demand, kept).
+int reserve_out(dt_handle* h, uint64_t rows) {
+  if (rows <= h->out_cap) return DT_OK;
+  cudaStreamSynchronize(h->stream);
+  cudaFree(h->out_buf);
+  h->out_buf = nullptr;
+  h->out_cap = 0;
+  if (cudaMalloc(&h->out_buf, rows * 16) != cudaSuccess) return DT_ENOMEM;
+  h->out_cap = rows;
+  return DT_OK;
+}
+
+// Memory of the mesh that holds nothing while no insertion runs: the claim words (16 bytes per
+// slot; zero is below every priority), the owner words (4 bytes per slot, zero between
+// launches) and the list of freed slots (a quarter of the slots, empty between launches). A batch
+// has no owner words; its lists of freed and free slots hold an entry per slot and start empty.
+CanonScratch canon_scratch(dt_handle* h) {
+  uint4* rows = reinterpret_cast<uint4*>(h->claim);
+  if (h->batch_mode) return CanonScratch{rows, h->pending, reinterpret_cast<uint2*>(h->freelist)};
+  return CanonScratch{rows, h->lock, reinterpret_cast<uint2*>(h->pending)};
+}
+
 // Finite tetrahedra of a batch, grouped by cloud (cloud-local ids).
 int batch_get_tets(dt_handle* h, uint32_t* tets_dev, uint64_t cap, uint64_t* n_tets, uint64_t* cloud_offsets,
                    int canonical) {
@@ -2080,68 +2084,44 @@ int batch_get_tets(dt_handle* h, uint32_t* tets_dev, uint64_t cap, uint64_t* n_t
     cudaFree(counts);
     return DT_ENOMEM;
   }
-  cudaMemsetAsync(counts, 0, nc * 8ull, s);
-  batch_collect(h->bclouds, nc, h->tets, h->pts, h->boff_dev, 0, counts, nullptr, nullptr, canonical, s);
-  std::vector<unsigned long long> cnt(nc), oo(nc + 1, 0);
-  cudaMemcpyAsync(cnt.data(), counts, nc * 8ull, cudaMemcpyDeviceToHost, s);
-  int rc = cudaStreamSynchronize(s) == cudaSuccess ? DT_OK : DT_ECUDA;
-  for (uint32_t c = 0; c < nc; ++c) oo[c + 1] = oo[c] + cnt[c];
-  const uint64_t T = oo[nc];
-  *n_tets = T;
-  h->stats.n_tets = T;
-  if (cloud_offsets)
-    for (uint32_t c = 0; c <= nc; ++c) cloud_offsets[c] = oo[c];
-  if (rc == DT_OK && T > cap) rc = DT_ETOOSMALL;
-  // the sorted list needs the unsorted one first; otherwise the rows go straight to the output
-  const bool sort = canonical && !(h->cfg.flags & DT_FLAG_NO_CANONICAL_SORT) && T > 1;
-  uint32_t* tmp = nullptr;
-  if (rc == DT_OK && sort && cudaMalloc(&tmp, T * 16) != cudaSuccess) rc = DT_ENOMEM;
-  if (rc == DT_OK && T > 0) {
-    cudaMemcpyAsync(ooff, oo.data(), (nc + 1) * 8ull, cudaMemcpyHostToDevice, s);
-    batch_collect(h->bclouds, nc, h->tets, h->pts, h->boff_dev, 1, counts, ooff, sort ? tmp : tets_dev, canonical, s);
-    if (sort) {
-      // lexicographic by (cloud, a, b, c, d): LSD passes on (c, d), then (a, b), then the cloud
-      uint64_t *khi = nullptr, *klo = nullptr, *kcl = nullptr, *ka = nullptr;
-      uint32_t *idx = nullptr, *ia = nullptr, *hist = nullptr;
-      bool ok = cudaMalloc(&khi, T * 8) == cudaSuccess && cudaMalloc(&klo, T * 8) == cudaSuccess &&
-                cudaMalloc(&kcl, T * 8) == cudaSuccess && cudaMalloc(&ka, T * 8) == cudaSuccess &&
-                cudaMalloc(&idx, T * 4) == cudaSuccess && cudaMalloc(&ia, T * 4) == cudaSuccess &&
-                cudaMalloc(&hist, radix_hist_entries(T) * 4) == cudaSuccess;
-      if (ok) {
-        int cbits = 8;
-        while (cbits < 32 && (1ull << cbits) < nc) cbits += 8;
-        batch_tet_keys(tmp, T, ooff, nc, khi, klo, kcl, idx, s);
-        bool alt = radix_sort_pairs(klo, idx, ka, ia, T, 64, hist, s);
-        uint32_t* order = alt ? ia : idx;
-        uint32_t* other = alt ? idx : ia;
-        k_gather_keys<<<grid_for(T, 256), 256, 0, s>>>(khi, order, T, ka);
-        ++g_kernel_launches;
-        bool alt2 = radix_sort_pairs(ka, order, klo, other, T, 64, hist, s);
-        uint32_t* order2 = alt2 ? other : order;
-        uint32_t* other2 = alt2 ? order : other;
-        k_gather_keys<<<grid_for(T, 256), 256, 0, s>>>(kcl, order2, T, ka);
-        ++g_kernel_launches;
-        bool alt3 = radix_sort_pairs_bits(ka, order2, klo, other2, T, 0, cbits, hist, s);
-        k_gather_tets<<<grid_for(T, 256), 256, 0, s>>>((const uint4*)tmp, alt3 ? other2 : order2, T,
-                                                       (uint4*)tets_dev);
-        ++g_kernel_launches;
-      } else {
-        rc = DT_ENOMEM;
-      }
-      cudaFree(khi);
-      cudaFree(klo);
-      cudaFree(kcl);
-      cudaFree(ka);
-      cudaFree(idx);
-      cudaFree(ia);
-      cudaFree(hist);
-    }
+  std::vector<unsigned long long> oo(nc + 1, 0);
+  int rc = DT_OK;
+  if (cap > 0 && canonical && !(h->cfg.flags & DT_FLAG_NO_CANONICAL_SORT)) {
+    // clouds hold ascending ranges of the input: rows sorted by input ids are sorted by (cloud,
+    // row), and each cloud's rows start at its first point's bucket
+    const BatchCloud& last = h->bclouds_host[nc - 1];
+    const uint64_t slots = (uint64_t)last.tb + last.used;
+    const CanonIn in{h->tets, slots, h->pts, h->n_pts, h->bclouds, nc, h->bcid, h->boff_dev};
+    uint64_t T = 0;
+    rc = reserve_out(h, std::min<uint64_t>(cap, slots));
+    if (rc == DT_OK)
+      rc = canon_rows(in, h->canon, canon_scratch(h), cap, reinterpret_cast<uint4*>(h->out_buf),
+                      reinterpret_cast<uint4*>(tets_dev), &T, ooff, s);
+    if (rc == DT_OK &&
+        cudaMemcpyAsync(oo.data(), ooff, (nc + 1) * 8ull, cudaMemcpyDeviceToHost, s) != cudaSuccess)
+      rc = DT_ECUDA;
     if (cudaStreamSynchronize(s) != cudaSuccess) rc = DT_ECUDA;
+  } else {
+    cudaMemsetAsync(counts, 0, nc * 8ull, s);
+    batch_collect(h->bclouds, nc, h->tets, h->pts, h->boff_dev, 0, counts, nullptr, nullptr, canonical, s);
+    std::vector<unsigned long long> cnt(nc);
+    cudaMemcpyAsync(cnt.data(), counts, nc * 8ull, cudaMemcpyDeviceToHost, s);
+    rc = cudaStreamSynchronize(s) == cudaSuccess ? DT_OK : DT_ECUDA;
+    for (uint32_t c = 0; c < nc; ++c) oo[c + 1] = oo[c] + cnt[c];
+    if (rc == DT_OK && oo[nc] > 0 && oo[nc] <= cap) {
+      cudaMemcpyAsync(ooff, oo.data(), (nc + 1) * 8ull, cudaMemcpyHostToDevice, s);
+      batch_collect(h->bclouds, nc, h->tets, h->pts, h->boff_dev, 1, counts, ooff, tets_dev, canonical, s);
+      if (cudaStreamSynchronize(s) != cudaSuccess) rc = DT_ECUDA;
+    }
   }
-  cudaFree(tmp);
   cudaFree(counts);
   cudaFree(ooff);
-  return rc;
+  if (rc != DT_OK) return rc;
+  *n_tets = oo[nc];
+  h->stats.n_tets = oo[nc];
+  if (cloud_offsets)
+    for (uint32_t c = 0; c <= nc; ++c) cloud_offsets[c] = oo[c];
+  return oo[nc] > cap ? DT_ETOOSMALL : DT_OK;
 }
 
 
@@ -2509,6 +2489,7 @@ int dt_get_tets(dt_handle* h, uint32_t* tets_dev, uint64_t cap, uint64_t* n_tets
                 int canonical) {
   if (!h || !n_tets || (cap > 0 && !tets_dev)) return DT_EINVAL;
   *n_tets = 0;
+  bool mapped = false;
   if (cap > 0) {
     // page-locked host memory is accepted too, through its mapped device address
     cudaPointerAttributes at{};
@@ -2517,6 +2498,7 @@ int dt_get_tets(dt_handle* h, uint32_t* tets_dev, uint64_t cap, uint64_t* n_tets
       if (at.type == cudaMemoryTypeHost) {
         if (!at.devicePointer) return DT_EINVAL;
         tets_dev = static_cast<uint32_t*>(at.devicePointer);
+        mapped = true;
       }
     }
     cudaGetLastError();  // an unknown pointer leaves an error behind; it is not one
@@ -2526,65 +2508,39 @@ int dt_get_tets(dt_handle* h, uint32_t* tets_dev, uint64_t cap, uint64_t* n_tets
   cudaStream_t s = h->stream;
   int rc = sync_state(h);
   if (rc != DT_OK) return rc;
-  uint64_t slots = h->st_host->bump;
-  unsigned long long* cnt = nullptr;
-  uint32_t* tmp = nullptr;
-  if (cudaMalloc(&cnt, 8) != cudaSuccess) return DT_ENOMEM;
-  // the sorted list needs the unsorted one first; otherwise the tetrahedra go straight to the
-  // caller's buffer (a count alone when it has none)
-  const bool sort = canonical && !(h->cfg.flags & DT_FLAG_NO_CANONICAL_SORT) && cap > 0;
-  if (sort && cudaMalloc(&tmp, std::max<uint64_t>(slots, 1) * 16) != cudaSuccess) {
+  const uint64_t slots = h->st_host->bump;
+  const CanonIn in{h->tets, slots, h->pts, h->mesh_pts, nullptr, 0, nullptr, nullptr};
+  uint64_t T = 0;
+  if (cap == 0) {  // a count alone
+    if ((rc = canon_count(in, h->canon, &T, s)) != DT_OK) return rc;
+  } else if (canonical && !(h->cfg.flags & DT_FLAG_NO_CANONICAL_SORT)) {
+    // mapped host memory is written once, in order: its rows are put into their buckets in a
+    // device buffer first
+    uint4* staged = reinterpret_cast<uint4*>(tets_dev);
+    if (mapped) {
+      if ((rc = reserve_out(h, std::min<uint64_t>(cap, slots))) != DT_OK) return rc;
+      staged = reinterpret_cast<uint4*>(h->out_buf);
+    }
+    if ((rc = canon_rows(in, h->canon, canon_scratch(h), cap, staged, reinterpret_cast<uint4*>(tets_dev), &T, nullptr,
+                         s)) != DT_OK)
+      return rc;
+    if (cudaStreamSynchronize(s) != cudaSuccess) return DT_ECUDA;
+  } else {
+    unsigned long long* cnt = nullptr;
+    if (cudaMalloc(&cnt, 8) != cudaSuccess) return DT_ENOMEM;
+    cudaMemsetAsync(cnt, 0, 8, s);
+    k_collect<<<grid_for(slots, 256), 256, 0, s>>>(h->tets, slots, h->pts, h->mesh_pts, tets_dev, cnt, cap, canonical);
+    ++g_kernel_launches;
+    unsigned long long c = 0;
+    cudaMemcpyAsync(&c, cnt, 8, cudaMemcpyDeviceToHost, s);
+    const bool ok = cudaStreamSynchronize(s) == cudaSuccess;
     cudaFree(cnt);
-    return DT_ENOMEM;
+    if (!ok) return DT_ECUDA;
+    T = c;
   }
-  cudaMemsetAsync(cnt, 0, 8, s);
-  k_collect<<<grid_for(slots, 256), 256, 0, s>>>(h->tets, slots, h->pts, h->cap_pts, sort ? tmp : tets_dev, cnt,
-                                                 sort ? slots : cap, canonical);
-  ++g_kernel_launches;
-  unsigned long long T = 0;
-  cudaMemcpyAsync(&T, cnt, 8, cudaMemcpyDeviceToHost, s);
-  cudaStreamSynchronize(s);
   *n_tets = T;
   h->stats.n_tets = T;
-  if (T > cap) {
-    cudaFree(cnt);
-    cudaFree(tmp);
-    return DT_ETOOSMALL;
-  }
-  if (sort && T > 1) {
-    uint64_t *khi = nullptr, *klo = nullptr, *ka = nullptr;
-    uint32_t *idx = nullptr, *ia = nullptr, *hist = nullptr;
-    bool ok = cudaMalloc(&khi, T * 8) == cudaSuccess && cudaMalloc(&klo, T * 8) == cudaSuccess &&
-              cudaMalloc(&ka, T * 8) == cudaSuccess && cudaMalloc(&idx, T * 4) == cudaSuccess &&
-              cudaMalloc(&ia, T * 4) == cudaSuccess &&
-              cudaMalloc(&hist, radix_hist_entries(T) * 4) == cudaSuccess;
-    if (ok) {
-      k_split_keys<<<grid_for(T, 256), 256, 0, s>>>((const uint4*)tmp, T, khi, klo, idx);
-      ++g_kernel_launches;
-      bool alt = radix_sort_pairs(klo, idx, ka, ia, T, 64, hist, s);
-      uint32_t* order = alt ? ia : idx;
-      uint32_t* other = alt ? idx : ia;
-      k_gather_keys<<<grid_for(T, 256), 256, 0, s>>>(khi, order, T, ka);
-      ++g_kernel_launches;
-      bool alt2 = radix_sort_pairs(ka, order, klo, other, T, 64, hist, s);
-      k_gather_tets<<<grid_for(T, 256), 256, 0, s>>>((const uint4*)tmp, alt2 ? other : order, T, (uint4*)tets_dev);
-      ++g_kernel_launches;
-    } else {
-      rc = DT_ENOMEM;
-    }
-    cudaFree(khi);
-    cudaFree(klo);
-    cudaFree(ka);
-    cudaFree(idx);
-    cudaFree(ia);
-    cudaFree(hist);
-  } else if (sort && T) {
-    cudaMemcpyAsync(tets_dev, tmp, T * 16, cudaMemcpyDeviceToDevice, s);
-  }
-  if (cudaStreamSynchronize(s) != cudaSuccess) rc = DT_ECUDA;
-  cudaFree(cnt);
-  cudaFree(tmp);
-  return rc;
+  return T > cap ? DT_ETOOSMALL : DT_OK;
 }
 
 int dt_get_tets_host(dt_handle* h, uint32_t* tets_host, uint64_t cap, uint64_t* n_tets, int canonical) {
@@ -2605,15 +2561,10 @@ int dt_get_tets_host(dt_handle* h, uint32_t* tets_host, uint64_t cap, uint64_t* 
   cudaGetLastError();  // a pointer the runtime does not know leaves an error behind; it is not one
   // one collection into a device buffer kept by the handle, then one copy out (fast from
   // page-locked memory)
-  if (cap > h->out_cap) {
-    cudaFree(h->out_buf);
-    h->out_buf = nullptr;
-    h->out_cap = 0;
-    if (cudaMalloc(&h->out_buf, cap * 16) != cudaSuccess) return DT_ENOMEM;
-    h->out_cap = cap;
-  }
+  int rc = reserve_out(h, cap);
+  if (rc != DT_OK) return rc;
   uint64_t T = 0;
-  int rc = dt_get_tets(h, h->out_buf, cap, &T, nullptr, canonical);
+  rc = dt_get_tets(h, h->out_buf, cap, &T, nullptr, canonical);
   *n_tets = T;
   if (rc != DT_OK) return rc;
   if (T && cudaMemcpyAsync(tets_host, h->out_buf, T * 16, cudaMemcpyDeviceToHost, h->stream) != cudaSuccess)
@@ -2713,6 +2664,7 @@ void dt_destroy(dt_handle* h) {
   cudaFree(h->subdet);
   cudaFree(h->in_buf);
   cudaFree(h->out_buf);
+  canon_ws_free(h->canon);
   cudaFree(h->async_big_ws);
   cudaFree(h->async_borrow_ws);
   cudaFree(h->async_borrow_busy);

@@ -117,6 +117,7 @@ bool radix_sort_pairs_bits(uint64_t* k, uint32_t* v, uint64_t* ka, uint32_t* va,
 uint64_t radix_hist_entries(uint64_t n);
 // In-place exclusive prefix sum of data[0, len) (device); scratch holds radix_hist_entries(len).
 void prefix_sum_exclusive(uint32_t* data, uint64_t len, uint32_t* scratch, cudaStream_t s);
+uint64_t prefix_scratch_entries(uint64_t len);  // entries that scan needs of scratch
 
 // Cumulative end of BRIO round r (Section 2.3 / Table 2): 2048 * 7^r.
 uint64_t brio_round_end(int r);
@@ -188,9 +189,46 @@ void batch_reset(const BatchCloud* clouds, const uint32_t* list, uint32_t n_list
 void batch_collect(const BatchCloud* clouds, uint32_t n_clouds, const Tet* tets, const Pt* pts, const uint64_t* in_off,
                    int pass, unsigned long long* counts, const unsigned long long* out_off, uint32_t* out,
                    int canonical, cudaStream_t s);
-// Sort keys of collected tetrahedra: (a, b), (c, d) and the cloud.
-void batch_tet_keys(const uint32_t* tets, uint64_t T, const unsigned long long* out_off, uint32_t n_clouds,
-                    uint64_t* khi, uint64_t* klo, uint64_t* kcl, uint32_t* idx, cudaStream_t s);
+
+// ---------------------------------------------------------------- canonical.cu (dt_get_tets)
+// Device workspace of the canonical list, kept by the handle: 8 bytes per vertex.
+struct CanonWS {
+  uint32_t* ids = nullptr;    // input index of every vertex
+  uint32_t* first = nullptr;  // per input index: its bucket's size, then where it starts
+  uint32_t* scan = nullptr;   // prefix sum scratch
+  unsigned long long* count = nullptr;  // rows; 1 when a bucket is larger than a block orders
+  uint64_t cap = 0, scan_cap = 0;
+};
+// The mesh a list is made of: slots [0, nslots), vertices [0, npts). For a batch also its
+// clouds, the cloud of every input index and the clouds' first input indices (device).
+struct CanonIn {
+  const Tet* tets;
+  uint64_t nslots;
+  const Pt* pts;
+  uint64_t npts;
+  const BatchCloud* clouds;
+  uint32_t n_clouds;
+  const uint32_t* cid;
+  const uint64_t* in_off;
+};
+// Scratch that is idle while no point is being inserted: 16 and 4 bytes per slot, zeroed again
+// before the call ends, and 8 bytes per 1024 slots of any content.
+struct CanonScratch {
+  uint4* rows;
+  uint32_t* place;
+  uint2* bounds;
+};
+void canon_ws_free(CanonWS& w);
+uint64_t canon_ws_bytes(const CanonWS& w);
+// Counts the live finite tetrahedra. Synchronises s.
+int canon_count(const CanonIn& in, CanonWS& w, uint64_t* T, cudaStream_t s);
+// Writes them to out as canonical rows in lexicographic order (of the cloud, then the row, with
+// a cloud's own ids, for a batch) when there are at most cap; *T is their number in any case.
+// staged: device memory for the rows in bucket order; may be out itself, except for a batch or
+// when out is host memory. cloud_starts (device, n_clouds + 1, or null): where each cloud's rows
+// start. Synchronises s once, before the rows are placed.
+int canon_rows(const CanonIn& in, CanonWS& w, const CanonScratch& t, uint64_t cap, uint4* staged, uint4* out, uint64_t* T,
+               unsigned long long* cloud_starts, cudaStream_t s);
 // ---------------------------------------------------------------- mlp.cu (learned scheduler)
 // ---------------------------------------------------------------- refinement (refine.cu)
 // Parameters of one refinement iteration (Section 4): thresholds (ratio h)^2 and (spacing h)^2,

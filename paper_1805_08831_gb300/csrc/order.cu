@@ -642,6 +642,15 @@ constexpr uint64_t radix_hist_entries_for(uint64_t n) {
 
 uint64_t radix_hist_entries(uint64_t n) { return radix_hist_entries_for(n); }
 
+uint64_t prefix_scratch_entries(uint64_t len) {
+  uint64_t all = 64;
+  for (uint64_t l = len; l > 1;) {
+    l = (l + kScanTile - 1) / kScanTile;
+    all += l;
+  }
+  return all;
+}
+
 void prefix_sum_exclusive(uint32_t* data, uint64_t len, uint32_t* scratch, cudaStream_t s) {
   if (len) scan_exclusive(data, len, scratch, s);
 }
