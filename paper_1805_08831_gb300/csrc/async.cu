@@ -47,7 +47,9 @@ constexpr int kADefer = 16;       // aborted points waiting for a retry
 constexpr int kARetry = 3;        // immediate restarts after a failed re-read
 constexpr uint32_t kAChunk = 32;  // slots taken from the allocator at a time
 
-enum AStatus : int { kAInserted = 0, kALost = 1, kARestart = 2, kABig = 3, kAWalkLimit = 4, kADup = 5, kAExact = 6 };
+enum AStatus : int {
+  kAInserted = 0, kALost = 1, kARestart = 2, kABig = 3, kAWalkLimit = 4, kADup = 5, kAExact = 6, kANoSeed = 7
+};
 
 // Ball adjacency (Section 2.5): the n x n edge table for balls of at most 32 boundary vertices
 // (the shared-memory workspaces), an edge hash for larger ones (the global-memory workspaces).
@@ -130,12 +132,9 @@ __device__ __forceinline__ bool same_v(const uint4& a, const uint4& b) {
 // A record that references only allocated vertices and slots (a record being rewritten may be
 // read half old, half new; such a read is never followed).
 __device__ __forceinline__ bool rec_ok(const Tet& T, uint32_t ntets, uint32_t npts) {
-  bool ok = true;
-  for (int k = 0; k < 4; ++k) {
-    uint32_t v = get4(T.v, k), n = get4(T.n, k);
-    ok = ok && (v == kGhost || v < npts) && n < ntets;
-  }
-  return ok;
+  // v + 1 wraps the ghost vertex to 0
+  return max(max(T.v.x + 1u, T.v.y + 1u), max(T.v.z + 1u, T.v.w + 1u)) <= npts &&
+         max(max(T.n.x, T.n.y), max(T.n.z, T.n.w)) < ntets;
 }
 
 // The predicates' FP32 stage on the double-float point copy (predicates.cuh: rigorous error
@@ -238,14 +237,55 @@ __device__ __forceinline__ int inside_maybe_cached(const Ctx& c, uint32_t u, con
   return insphere_cached(q0, q1, load_ptf(c.ptf, v.x), FP, c.eta);
 }
 
+// The exact signs behind the FP32 stage, for the kernels built with kExact (inputs the FP32 stage
+// often cannot decide: lattices, co-spherical and coplanar sets). Out of line: their code and
+// registers stay out of the common path.
+
+// orient3d of the finite tetrahedron v with vertex i replaced by p: the FP64 filter, then exact.
+static __device__ __noinline__ int orient_exact_at(const Pt* pts, DevState* st, uint4 v, int i, uint32_t p) {
+  const Pt a = load_pt(pts, i == 0 ? p : v.x), b = load_pt(pts, i == 1 ? p : v.y), d = load_pt(pts, i == 2 ? p : v.z),
+           e = load_pt(pts, i == 3 ? p : v.w);
+  return orient3d(a, b, d, e, st);
+}
+
+// Whether p lies inside the perturbed sphere of the finite tetrahedron v.
+static __device__ __noinline__ bool inside_exact_at(const Pt* pts, DevState* st, uint4 v, uint32_t p) {
+  return insphere_sos(load_pt(pts, v.x), load_pt(pts, v.y), load_pt(pts, v.z), load_pt(pts, v.w), load_pt(pts, p),
+                      st) < 0;
+}
+
+// Conflict of the ghost v (ghost vertex at position g, finite neighbour r) with p: p strictly
+// beyond the hull facet, or on its plane and inside the finite neighbour's sphere (Section 2.6).
+// The neighbour is read without a lock and need not be verified later: p on the facet's plane is
+// inside the sphere of whatever tetrahedron is built on the facet from inside exactly when it is
+// inside the facet's circle, and on the circle the perturbation decides by orient3d's with the
+// apex among their four points, whose signs depend on the apex's side alone (the one without it
+// is zero). So any live tetrahedron that holds the three vertices gives the same answer. Returns
+// 1, 0, or -1 when r does not hold them (a record read mid-change).
+static __device__ __noinline__ int ghost_exact_at(const Pt* pts, DevState* st, const Tet* tets, uint32_t npts, uint4 v,
+                                                  int g, uint32_t r, uint32_t p) {
+  const int o = orient_exact_at(pts, st, v, g, p);
+  if (o != 0) return o > 0 ? 1 : 0;
+  const uint4 R = __ldcg(reinterpret_cast<const uint4*>(tets + r));
+  bool ok = !tet_dead(R) && R.x < npts && R.y < npts && R.z < npts && R.w < npts;
+  for (int k = 0; k < 4; ++k) {
+    const uint32_t q = get4(v, k);
+    ok = ok && (k == g || R.x == q || R.y == q || R.z == q || R.w == q);
+  }
+  if (!ok) return -1;
+  return inside_exact_at(pts, st, R, p) ? 1 : 0;
+}
+
 // Visibility walk (Section 2.1, ghost rules of Section 2.6) on unlocked reads. Lanes 0-3 test
 // the four facets of the current tetrahedron at once (lane i: p against the facet opposite
 // vertex i), and the walk leaves through the first facet p sees, in an order that turns with
 // the steps. A record that is being rewritten may be read half old, half new: such reads end
 // the walk with kARestart (or it runs into its step bound); nothing is trusted before step 4
-// re-reads it under a lock. Called by the whole warp; the result is uniform.
+// re-reads it under a lock. Called by the whole warp; the result is uniform. *n_out: the
+// neighbours of the tetrahedron reached.
+template <bool kExact>
 __device__ __forceinline__ int walk_async(const Ctx& c, uint32_t p, const PtF& FP, uint32_t start, uint32_t salt,
-                                          uint32_t max_steps, uint32_t* t_out, uint32_t* steps_out) {
+                                          uint32_t max_steps, uint32_t* t_out, uint4* n_out, uint32_t* steps_out) {
   const int lane = threadIdx.x & 31;
   uint32_t t = start;
   Tet T;
@@ -272,15 +312,20 @@ __device__ __forceinline__ int walk_async(const Ctx& c, uint32_t p, const PtF& F
     if (ghost_pos(T.v) >= 0) break;
     // lane i < 4: orientation of p against the facet opposite vertex i (0: undecided)
     int o = 1;
-    if (lane < 4) {
+    const bool mine = lane < 4 && get4(T.n, lane) != prev;  // p is on this side of the facet just crossed
+    if (mine) {
       const PtF F0 = load_ptf(c.ptf, T.v.x), F1 = load_ptf(c.ptf, T.v.y), F2 = load_ptf(c.ptf, T.v.z),
                 F3 = load_ptf(c.ptf, T.v.w);
-      o = get4(T.n, lane) == prev ? 1 : orient_with_p(c, lane, FP, F0, F1, F2, F3);
+      o = orient_with_p(c, lane, FP, F0, F1, F2, F3);
     }
-    const unsigned sees = __ballot_sync(kFull, lane < 4 && o < 0) & 0xFu;
+    unsigned sees = __ballot_sync(kFull, o < 0);
     // a facet the FP32 stage cannot decide matters only when no other facet is certainly seen:
     // any facet p sees is a valid exit of the visibility walk
-    if (sees == 0 && (__ballot_sync(kFull, lane < 4 && o == 0) & 0xFu)) return kAExact;
+    if (sees == 0 && __any_sync(kFull, o == 0)) {
+      if constexpr (!kExact) return kAExact;
+      if (o == 0) o = orient_exact_at(c.pts, c.st, T.v, lane, p);
+      sees = __ballot_sync(kFull, o < 0);
+    }
     if (sees == 0) {
       // p is inside (or on) this tetrahedron: a vertex equal to p would be a duplicate
       bool dup = false;
@@ -292,6 +337,7 @@ __device__ __forceinline__ int walk_async(const Ctx& c, uint32_t p, const PtF& F
         }
       }
       *t_out = t;
+      *n_out = T.n;
       *steps_out = steps;
       return __any_sync(kFull, dup) ? kADup : kAInserted;
     }
@@ -314,151 +360,158 @@ __device__ __forceinline__ int walk_async(const Ctx& c, uint32_t p, const PtF& F
     }
   }
   *t_out = t;
+  *n_out = T.n;
   *steps_out = steps;
   return kAInserted;
 }
 
-// Conflict of a record U (already read) with p: 1 in the cavity, 0 outside, -2 undecided by the
-// FP32 stage. For a ghost whose hull facet's plane holds p the finite neighbour across the facet
-// decides (Section 2.6): that case is left to the round-based engine (-2).
-template <bool kCache>
-__device__ __forceinline__ int conflict_async(const Ctx& c, uint32_t u, const Tet& U, const PtF& FP) {
-  const int g = ghost_pos(U.v);
-  if (g < 0) {
+// Conflict of a record U (already read) with p: 1 in the cavity, 2 outside, 4 undecided by the
+// FP32 stage, 8 not a consistent live record.
+template <bool kCache, bool kExact>
+__device__ __forceinline__ int conflict_async(const Ctx& c, uint32_t u, const Tet& U, uint32_t p, const PtF& FP) {
+  const uint32_t vm = max(max(U.v.x, U.v.y), max(U.v.z, U.v.w)), nm = max(max(U.n.x, U.n.y), max(U.n.z, U.n.w));
+  if (tet_dead(U.v) || nm >= c.ntets) return 8;
+  if (vm < c.npts) {
     const int s = kCache ? inside_maybe_cached(c, u, U.v, FP) : inside_async(c, U.v, FP);
-    return s < 0 ? 1 : (s > 0 ? 0 : -2);
+    if (s != 0) return s < 0 ? 1 : 2;
+    if constexpr (!kExact) return 4;
+    else return inside_exact_at(c.pts, c.st, U.v, p) ? 1 : 2;
   }
-  // orientation of the hull facet's three vertices and p in the ghost's place
+  const int g = ghost_pos(U.v);
+  // the hull facet's three vertices
   const uint32_t a = g == 0 ? U.v.y : U.v.x, b = g <= 1 ? U.v.z : U.v.y, d = g <= 2 ? U.v.w : U.v.z;
+  if (g < 0 || a >= c.npts || b >= c.npts || d >= c.npts) return 8;
+  // orientation of the hull facet and p in the ghost's place
   int o = orient3d_f(load_ptf(c.ptf, a), load_ptf(c.ptf, b), load_ptf(c.ptf, d), FP, c.eta);
   o = (g & 1) ? o : -o;
-  if (o != 0) return o > 0 ? 1 : 0;
-  // p on the facet's plane as far as the FP32 stage can tell: the exact rule needs the
-  // round-based engine (the plane test and the neighbour's perturbed sphere)
-  return -2;
+  if (o != 0) return o > 0 ? 1 : 2;
+  // p on the facet's plane as far as the FP32 stage can tell
+  if constexpr (!kExact) return 4;
+  const int s = ghost_exact_at(c.pts, c.st, c.tets, c.npts, U.v, g, get4(U.n, g), p);
+  return s < 0 ? 8 : (s ? 1 : 2);
 }
 
+// The visited set's entry of key (its index), claimed for the caller when *mine comes back true.
+// The table is never full: it has more entries than the lists have room for, plus one per lane.
 template <class W>
-__device__ __forceinline__ int hfind(const W& w, uint32_t key) {
+__device__ __forceinline__ uint32_t hclaim(W& w, uint32_t key, bool* mine) {
+  static_assert(W::kHash > W::kCMax + W::kAMax + 32, "room for every visited tetrahedron");
   uint32_t h = (hash32(key) >> 8) & (W::kHash - 1);
+  *mine = false;
 #pragma unroll 1
   for (int probe = 0; probe < W::kHash; ++probe) {
-    uint32_t k = vld(&w.hkey[h]);
-    if (k == key) return vld(&w.hval[h]);
-    if (k == kNone) return 0;
+    const uint32_t old = atomicCAS(&w.hkey[h], kNone, key);
+    if (old == kNone) *mine = true;
+    if (old == kNone || old == key) break;
     h = (h + 1) & (W::kHash - 1);
   }
-  return 0;
+  return h;
 }
 
-template <class W>
-__device__ __forceinline__ bool hinsert(W& w, uint32_t key, uint8_t val) {
-  uint32_t h = (hash32(key) >> 8) & (W::kHash - 1);
-#pragma unroll 1
-  for (int probe = 0; probe < W::kHash; ++probe) {
-    uint32_t old = atomicCAS(&w.hkey[h], kNone, key);
-    if (old == kNone || old == key) {
-      w.hval[h] = val;
-      return true;
-    }
-    h = (h + 1) & (W::kHash - 1);
-  }
-  return false;
-}
-
-// Step 2: the cavity of p from t0 on unlocked reads. Returns kAInserted (lists filled),
-// kARestart (an inconsistent read), kABig (the workspace is too small) or kAExact. The first
-// pass of the loop tests t0 itself (one lane), so the conflict test's code exists once.
-template <class W>
-__device__ __forceinline__ int cavity_async(const Ctx& c, W& w, uint32_t t0, uint32_t p, const PtF& FP) {
+// Step 2: the cavity of p on unlocked reads. The search starts from every tetrahedron of the
+// first pass that is in conflict with p: with ball > 0 the ball last inserted by this warp
+// (w.slot[0, ball)), else the walk's end t0 (which has to be in conflict) and its neighbours
+// tn. The conflict region is connected, so the cavity found does not depend on where the search
+// starts; starting from all of them at once takes the breadth-first levels from about seven to
+// four (each level is a chain of dependent loads: record, points, test), and the test's code
+// exists once. Returns kAInserted (lists filled), kANoSeed (no tetrahedron of the ball is in
+// conflict), kARestart (an inconsistent read), kABig (the workspace is too small) or kAExact.
+template <bool kExact, class W>
+__device__ __forceinline__ int cavity_async(const Ctx& c, W& w, int ball, uint32_t t0, const uint4& tn, uint32_t p,
+                                            const PtF& FP) {
   const int lane = threadIdx.x & 31;
-  for (int i = lane; i < W::kHash; i += 32) w.hkey[i] = kNone;
+  static_assert(W::kHash % 128 == 0, "cleared by 16 bytes a lane");
+  for (int i = lane; i < W::kHash / 4; i += 32)
+    reinterpret_cast<uint4*>(w.hkey)[i] = make_uint4(kNone, kNone, kNone, kNone);
   __syncwarp();
-  int flag = 0;  // 1 restart, 2 big, 4 a predicate the FP32 stage cannot decide
-  int nc = 0, na = 0, nb = 0, head = 0;
-  bool seed = true;
-  while (flag == 0 && (seed || head < nc)) {
-    const int k = lane >> 2, f = lane & 3;
-    bool active;
-    int ci;
+  int nc = 0, na = 0, nb = 0;
+  {
     uint32_t u = kNone;
-    if (seed) {
-      active = lane == 0;
-      ci = -1;
-      u = t0;
-    } else {
-      const int batch = min(8, nc - head);
-      active = k < batch;
-      ci = head + k;
-      if (active) {
-        u = get4(w.cr[ci].n, f);
-        if (u >= c.ntets) {
-          flag = 1;
-          active = false;
+    if (ball > 0) {
+      if (lane < ball) u = w.slot[lane];
+    } else if (lane < 5) {
+      u = lane == 0 ? t0 : get4(tn, lane - 1);
+    }
+    int res = 0;
+    Tet U;
+    if (u < c.ntets) {
+      U = ld_tet(c.tets, u);
+      res = conflict_async<W::kCache, kExact>(c, u, U, p, FP);
+    }
+    const unsigned m = __ballot_sync(kFull, res == 1);
+    if (ball > 0) {
+      if (m == 0) return kANoSeed;
+    } else if (!(m & 1u)) {  // the walk's tetrahedron: undecided, or read mid-rewrite
+      return __shfl_sync(kFull, res, 0) == 4 ? kAExact : kARestart;
+    }
+    if (res == 1) {
+      bool mine;
+      w.hval[hclaim(w, u, &mine)] = 1;
+      const int pos = __popc(m & lanemask_lt());
+      w.cl[pos] = u;
+      w.cr[pos] = U;
+    }
+    nc = __popc(m);
+    __syncwarp();
+  }
+  int flag = 0, head = 0;
+  while (head < nc) {
+    const int k = lane >> 2, f = lane & 3, ci = head + k;
+    const bool active = ci < nc;
+    head = min(head + 8, nc);
+    uint32_t u = 0, h = 0;
+    bool first = false;  // this lane is the first to reach u
+    if (active) {
+      u = reinterpret_cast<const uint32_t*>(&w.cr[ci].n)[f];
+      h = hclaim(w, u, &first);
+    }
+    int res = 0;
+    Tet U;
+    if (first) {
+      U = ld_tet(c.tets, u);  // u < ntets: the record that names it was checked
+      res = conflict_async<W::kCache, kExact>(c, u, U, p, FP);
+      w.hval[h] = (uint8_t)res;
+    }
+    __syncwarp();
+    if (active && !first) res = vld(&w.hval[h]);
+    const unsigned mX = __ballot_sync(kFull, res >= 4);
+    const unsigned mC = __ballot_sync(kFull, first && res == 1);
+    const unsigned mA = __ballot_sync(kFull, first && res == 2);
+    const unsigned mB = __ballot_sync(kFull, res == 2);
+    if (mX) {
+      flag = __any_sync(kFull, res == 4) ? 4 : 1;
+      break;
+    }
+    if (first) {
+      if (res == 1) {
+        const int pos = nc + __popc(mC & lanemask_lt());
+        if (pos < W::kCMax) {
+          w.cl[pos] = u;
+          w.cr[pos] = U;
+        }
+      } else {  // outside tetrahedra (locked and verified)
+        const int pos = na + __popc(mA & lanemask_lt());
+        if (pos < W::kAMax) {
+          w.al[pos] = u;
+          w.av[pos] = U.v;
         }
       }
-      flag = __reduce_or_sync(kFull, flag);
-      if (flag) break;
-      head += batch;
     }
-    const int known = active ? hfind(w, u) : 0;
-    const bool need = active && known == 0;
-    const unsigned peers = __match_any_sync(kFull, need ? u : 0xFFFFFFFFu);
-    const int leader = __ffs(peers) - 1;
-    const bool is_leader = need && lane == leader;
-    int res = 0, myflag = 0;
-    Tet U;
-    if (is_leader) {
-      U = ld_tet(c.tets, u);
-      const int in = (tet_dead(U.v) || !rec_ok(U, c.ntets, c.npts)) ? -1 : conflict_async<W::kCache>(c, u, U, FP);
-      if (in == -2) {
-        myflag |= 4;
-      } else if (in < 0) {
-        myflag |= 1;
-      } else {
-        res = in ? 1 : 2;
-        if (seed && res != 1) myflag |= 1;  // the walk's tetrahedron was read mid-rewrite
-        else if (!hinsert(w, u, (uint8_t)res)) myflag |= 2;
-      }
-    }
-    const int lres = __shfl_sync(kFull, res, leader);
-    res = need ? lres : known;
-    flag = __reduce_or_sync(kFull, myflag);
-    if (flag) break;
-    const bool addC = is_leader && res == 1;
-    const unsigned mC = __ballot_sync(kFull, addC);
-    if (addC) {
-      const int pos = nc + __popc(mC & lanemask_lt());
-      if (pos < W::kCMax) {
-        w.cl[pos] = u;
-        w.cr[pos] = U;
-      }
-    }
-    nc += __popc(mC);
-    // outside tetrahedra (locked and verified)
-    const bool addA = is_leader && res == 2;
-    const unsigned mA = __ballot_sync(kFull, addA);
-    if (addA) {
-      const int pos = na + __popc(mA & lanemask_lt());
-      if (pos < W::kAMax) {
-        w.al[pos] = u;
-        w.av[pos] = U.v;
-      }
-    }
-    na += __popc(mA);
-    const bool addB = active && ci >= 0 && res == 2;
-    const unsigned mB = __ballot_sync(kFull, addB);
-    if (addB) {
+    if (res == 2) {
       const int pos = nb + __popc(mB & lanemask_lt());
       if (pos < W::kFMax) {
         w.bl_ci[pos] = (typename W::CI)ci;
         w.bl_f[pos] = (uint8_t)f;
       }
     }
+    nc += __popc(mC);
+    na += __popc(mA);
     nb += __popc(mB);
-    if (nc > W::kCMax || na > W::kAMax || nb > W::kFMax) flag |= 2;
-    seed = false;
     __syncwarp();
+    if (nc > W::kCMax || na > W::kAMax || nb > W::kFMax) {
+      flag = 2;
+      break;
+    }
   }
   if (lane == 0) {
     w.nc = nc;
@@ -466,10 +519,7 @@ __device__ __forceinline__ int cavity_async(const Ctx& c, W& w, uint32_t t0, uin
     w.nb = nb;
   }
   __syncwarp();
-  if (flag & 4) return kAExact;
-  if (flag & 1) return kARestart;
-  if (flag & 2) return kABig;
-  return kAInserted;
+  return flag == 0 ? kAInserted : flag == 4 ? kAExact : flag == 2 ? kABig : kARestart;
 }
 
 // Slot of lock-list entry i: cavity slots, then the outside slots, then the ball's extra slots.
@@ -540,29 +590,22 @@ __device__ __forceinline__ void pool_give(const Ctx& c, W& w, const uint32_t* s,
 }
 
 // One attempt at inserting p (steps 1-5). w.hint is the warp's last ball, updated on success.
-template <class W>
+template <bool kExact, class W>
 __device__ __forceinline__ int try_insert(const Ctx& c, W& w, uint32_t* lock, uint32_t me, uint32_t p,
-                                          const InsertLog& lg, bool io_balltest = true) {
+                                          const InsertLog& lg, bool ball_start) {
   const int lane = threadIdx.x & 31;
   const PtF FP = load_ptf(c.ptf, p);
-  for (int attempt = 0; attempt <= kARetry; ++attempt) {
-    // 1. a start in conflict with p. Consecutive points of a segment are close, so p is often
-    //    inside the circumsphere of a tetrahedron of the previous ball (it will be joined to the
-    //    previous point): one insphere test per lane finds it without a walk. Otherwise walk.
-    int ws = kAInserted;
+  // 1. a start in conflict with p. Consecutive points of a segment are close, so p is often
+  //    inside the circumsphere of a tetrahedron of the previous ball (it will be joined to the
+  //    previous point): the search's first pass tests them all, without a walk. Otherwise walk.
+  int ball = ball_start ? w.bn : 0;
+  uint32_t start = w.hint;
+  __syncwarp();
+  if (lane == 0) w.bn = 0;  // used once
+  for (int attempt = 0; attempt <= kARetry;) {
     uint32_t t0 = kNone;
-    if (attempt == 0 && w.bn > 0 && io_balltest) {
-      bool in = false;
-      if (lane < w.bn) {
-        const uint4 v = __ldcg(reinterpret_cast<const uint4*>(c.tets + w.slot[lane]));
-        in = !tet_dead(v) && ghost_pos(v) < 0 && v.x < c.npts && v.y < c.npts && v.z < c.npts && v.w < c.npts &&
-             inside_async(c, v, FP) < 0;
-      }
-      const unsigned m = __ballot_sync(kFull, in);
-      if (m) t0 = w.slot[__ffs(m) - 1];
-    }
-    if (t0 == kNone) {
-      uint32_t start = attempt == 0 ? w.hint : kNone;
+    uint4 tn = make_uint4(kNone, kNone, kNone, kNone);
+    if (ball == 0) {
       if (start == kNone) start = c.point_hint[p];
       if (start == kNone) {
         uint32_t f, g;
@@ -572,21 +615,26 @@ __device__ __forceinline__ int try_insert(const Ctx& c, W& w, uint32_t* lock, ui
       }
       start = __shfl_sync(kFull, start, 0);
       uint32_t steps = 0;
-      ws = walk_async(c, p, FP, start, p * 0x9E3779B1u >> 30, c.max_walk, &t0, &steps);
+      const int ws = walk_async<kExact>(c, p, FP, start, p * 0x9E3779B1u >> 30, c.max_walk, &t0, &tn, &steps);
       if (lane == 0) {
         if (t0 != kNone && t0 < c.ntets) c.point_hint[p] = t0;
         w.cnt[5] += steps;
       }
-    }
-    if (lane == 0) w.bn = 0;  // used once
-    if (ws == kADup || ws == kAWalkLimit || ws == kAExact) return ws;
-    if (ws == kARestart) {
-      if (lane == 0) w.cnt[6] += 1;
-      continue;
+      if (ws == kADup || ws == kAWalkLimit || ws == kAExact) return ws;
+      if (ws == kARestart) {
+        if (lane == 0) w.cnt[6] += 1;
+        start = kNone;
+        ++attempt;
+        continue;
+      }
     }
     // 2. cavity on unlocked reads
-    const int r = cavity_async(c, w, t0, p, FP);
+    const int r = cavity_async<kExact>(c, w, ball, t0, tn, p, FP);
+    ball = 0;
+    if (r == kANoSeed) continue;  // walk from the warp's last ball
     if (r == kABig || r == kAExact) return r;
+    start = kNone;  // a further attempt starts from the grid
+    ++attempt;
     if (r == kARestart) {
       if (lane == 0) w.cnt[6] += 1;
       continue;
@@ -747,6 +795,9 @@ __device__ __forceinline__ int try_insert(const Ctx& c, W& w, uint32_t* lock, ui
         __stcg(c.subdet + 2 * (size_t)s, q0);
         __stcg(c.subdet + 2 * (size_t)s + 1, q1);
       }
+      if constexpr (kExact) {  // this kernel keeps no cache: the entry it replaces is void
+        if (c.subdet) __stcg(c.subdet + 2 * (size_t)s + 1, make_float4(0.f, 0.f, 0.f, 0.f));
+      }
       __stcg(reinterpret_cast<uint32_t*>(&c.tets[out].n) + back, s);
     }
     if (__any_sync(kFull, bad)) {
@@ -804,7 +855,7 @@ __device__ __forceinline__ void to_queue(const AsyncIO& io, const Ctx& c, int q,
 // for). Returns kABig when none is free or the cavity exceeds it too. The borrowed workspace's
 // counters, spare slots and ball hint come back to the warp's own. Out of line: it runs for
 // about one point in 1500, and inlined it would double the kernel's instruction footprint.
-template <class W>
+template <bool kExact, class W>
 __device__ __noinline__ int try_insert_large(const Ctx& c, const AsyncIO& io, W& w, uint32_t* lock, uint32_t me,
                                              uint32_t p, const InsertLog& lg) {
   if (!io.big_ws || io.big_n == 0) return kABig;
@@ -827,7 +878,7 @@ __device__ __noinline__ int try_insert_large(const Ctx& c, const AsyncIO& io, W&
     for (int q = 0; q < 8; ++q) L.cnt[q] = 0;
   }
   __syncwarp();
-  const int r = try_insert(c, L, lock, me, p, lg);
+  const int r = try_insert<kExact>(c, L, lock, me, p, lg, false);
   pool_give(c, w, L.pool, L.np);
   if (lane == 0) {
     w.cnt[0] += L.cnt[0];
@@ -846,7 +897,7 @@ __device__ __noinline__ int try_insert_large(const Ctx& c, const AsyncIO& io, W&
 
 // One warp's work: segment [b0, e0) of io's list in order, deferred points retried after later
 // insertions, then what is left handed on, unused slots returned and counters flushed.
-template <class W>
+template <bool kExact, class W>
 __device__ __forceinline__ void run_segment(const Ctx& c, const AsyncIO& io, W& w, uint32_t* lock, uint32_t me,
                                             uint64_t b0, uint64_t e0, const uint8_t* vflag, const InsertLog& lg) {
   const int lane = threadIdx.x & 31;
@@ -880,9 +931,9 @@ __device__ __forceinline__ void run_segment(const Ctx& c, const AsyncIO& io, W& 
       break;
     }
     if (lane == 0) w.cnt[2] += 1;
-    int r = try_insert(c, w, lock, me, p, lg, io.ball_start != 0);
+    int r = try_insert<kExact>(c, w, lock, me, p, lg, io.ball_start != 0);
     if constexpr (W::kTable) {
-      if (r == kABig) r = try_insert_large(c, io, w, lock, me, p, lg);
+      if (r == kABig) r = try_insert_large<kExact>(c, io, w, lock, me, p, lg);
     }
     // a raised error stops the launch; read every 16 points for the same reason as the anchor
     unsigned err = 0;
@@ -933,7 +984,7 @@ __device__ __forceinline__ void run_segment(const Ctx& c, const AsyncIO& io, W& 
   }
 }
 
-template <int kMinBlocks, bool kCache = false>
+template <int kMinBlocks, bool kCache = false, bool kExact = false>
 __global__ void __launch_bounds__(kAW * 32, kMinBlocks) k_async(Ctx c, AsyncIO io, uint32_t* lock,
                                                                const uint8_t* __restrict__ vflag, InsertLog lg) {
   __shared__ SmallWST<kCache> s_ws[kAW];
@@ -948,20 +999,20 @@ __global__ void __launch_bounds__(kAW * 32, kMinBlocks) k_async(Ctx c, AsyncIO i
     b0 = (uint64_t)seg * io.L;
     e0 = b0 + io.L < io.m ? b0 + io.L : io.m;
   }
-  run_segment(c, io, s_ws[wid], lock, seg + 1, b0, e0, vflag, lg);
+  run_segment<kExact>(c, io, s_ws[wid], lock, seg + 1, b0, e0, vflag, lg);
 }
 
 // Large cavities (beyond the shared-memory workspaces): the same insertion with each warp's
 // workspace in global memory. Owner words are per warp of the launch, and this kernel never
 // runs beside k_async, so warp numbers may repeat across the two.
-template <bool kCache>
+template <bool kCache, bool kExact>
 __global__ void __launch_bounds__(128) k_async_big(Ctx c, AsyncIO io, uint32_t* lock, const uint8_t* __restrict__ vflag,
                                                   InsertLog lg, LargeWST<kCache>* ws) {
   const uint32_t seg = blockIdx.x * 4 + (threadIdx.x >> 5);
   if (seg >= io.W) return;
   const uint64_t b0 = (uint64_t)seg * io.L;
   const uint64_t e0 = b0 + io.L < io.m ? b0 + io.L : io.m;
-  run_segment(c, io, ws[seg], lock, seg + 1, b0, e0, vflag, lg);
+  run_segment<kExact>(c, io, ws[seg], lock, seg + 1, b0, e0, vflag, lg);
 }
 
 // Folds the allocator of the launch into the free list, as a round close does
@@ -1041,9 +1092,9 @@ int async_launch_big(const Ctx& c, const AsyncIO& io, uint32_t* lock, const uint
   cc.coherent = 1;
   cc.max_walk = io.max_walk;
   if (c.subdet)
-    k_async_big<true><<<(io.W + 3) / 4, 128, 0, s>>>(cc, io, lock, vflag, lg, static_cast<LargeWST<true>*>(ws));
+    k_async_big<true, false><<<(io.W + 3) / 4, 128, 0, s>>>(cc, io, lock, vflag, lg, static_cast<LargeWST<true>*>(ws));
   else
-    k_async_big<false><<<(io.W + 3) / 4, 128, 0, s>>>(cc, io, lock, vflag, lg, static_cast<LargeWS*>(ws));
+    k_async_big<false, false><<<(io.W + 3) / 4, 128, 0, s>>>(cc, io, lock, vflag, lg, static_cast<LargeWS*>(ws));
   k_async_close_copy<<<152, 256, 0, s>>>(cc);
   k_async_close_state<<<1, 1, 0, s>>>(cc);
   g_kernel_launches += 3;
