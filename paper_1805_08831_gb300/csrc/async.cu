@@ -53,10 +53,18 @@ enum AStatus : int {
 
 // Ball adjacency (Section 2.5): the n x n edge table for balls of at most 32 boundary vertices
 // (the shared-memory workspaces), an edge hash for larger ones (the global-memory workspaces).
-template <bool kTable, int kHashN, int kFMaxN>
-struct AWSTail;
+template <int kHashN, int kFMaxN, int kEdgeSlots>
+struct AWSTail {
+  static constexpr uint32_t kEdgeN = kEdgeSlots;
+  uint32_t hkey[kHashN];
+  uint8_t hval[kHashN];
+  unsigned long long ekey[kEdgeN];
+  uint32_t eval[kEdgeN];
+  uint32_t hslot[3 * kFMaxN];
+  uint32_t hold[3 * kFMaxN];
+};
 template <int kHashN, int kFMaxN>
-struct AWSTail<true, kHashN, kFMaxN> {
+struct AWSTail<kHashN, kFMaxN, 0> {
   // the visited set is needed only while the cavity is searched, the edge table only while the
   // ball is built: they share their bytes
   union {
@@ -67,30 +75,18 @@ struct AWSTail<true, kHashN, kFMaxN> {
     uint16_t tab[32 * 32];
   };
 };
-template <int kHashN, int kFMaxN>
-struct AWSTail<false, kHashN, kFMaxN> {
-  static constexpr uint32_t kEdgeN = 4096;
-  uint32_t hkey[kHashN];
-  uint8_t hval[kHashN];
-  unsigned long long ekey[kEdgeN];
-  uint32_t eval[kEdgeN];
-  uint32_t hslot[3 * kFMaxN];
-  uint32_t hold[3 * kFMaxN];
-};
-
 // Working storage of one warp: the cavity's tetrahedra with their records as read, the outside
 // tetrahedra with their vertices as read, the boundary facets, the ball's slots, a private pool
 // of free slots, deferred points, and the warp's state (uniform across its lanes, written by
-// lane 0). Held: the type of a lane's lock mask (one bit per lock-list entry of the lane).
-template <int kHashN, int kCMaxN, int kAMaxN, int kFMaxN, bool kTableB, class HeldT, bool kCacheB>
-struct AWS : AWSTail<kTableB, kHashN, kFMaxN> {
+// lane 0). kEdgeSlots: slots of the edge hash, 0 for the edge table.
+template <int kHashN, int kCMaxN, int kAMaxN, int kFMaxN, int kEdgeSlots, bool kCacheB>
+struct AWS : AWSTail<kHashN, kFMaxN, kEdgeSlots> {
   static constexpr int kHash = kHashN, kCMax = kCMaxN, kAMax = kAMaxN, kFMax = kFMaxN;
   static constexpr bool kCache = kCacheB;  // conflict tests through the sub-determinant cache
   static constexpr int kPool = kFMaxN + 36;  // a refill of 32 slots always fits below kFMax
-  static constexpr bool kTable = kTableB;
-  using Held = HeldT;
+  static constexpr bool kTable = kEdgeSlots == 0;
   using CI = typename std::conditional<(kCMaxN > 255), uint16_t, uint8_t>::type;
-  static_assert(kCMaxN + kAMaxN + kFMaxN <= 32 * 8 * (int)sizeof(HeldT), "lock mask holds every entry");
+  static_assert(!kTable || kCMaxN + kAMaxN + kFMaxN <= 32 * 32, "a lane's lock mask holds its entries");
   uint32_t cl[kCMaxN];       // cavity slots
   Tet cr[kCMaxN];            // their records as read
   uint32_t al[kAMaxN];       // outside slots
@@ -111,12 +107,15 @@ struct AWS : AWSTail<kTableB, kHashN, kFMaxN> {
 };
 
 // Shared-memory workspace of the main kernel (cavities of up to 64 tetrahedra and 60 boundary
-// facets) and the global-memory one of the large-cavity kernel.
+// facets), the global-memory one a warp borrows for a larger cavity (145 KB), and that of the
+// large-cavity kernel (1.6 MB: the sphere's empty interior, a surface's first inner points).
 template <bool kCache>
-using SmallWST = AWS<256, 64, 64, 60, true, unsigned, kCache>;
+using SmallWST = AWS<256, 64, 64, 60, 0, kCache>;
 template <bool kCache>
-using LargeWST = AWS<4096, 640, 704, 704, false, unsigned long long, kCache>;
+using LargeWST = AWS<4096, 640, 704, 704, 4096, kCache>;
 using LargeWS = LargeWST<false>;  // the same layout with and without the cache
+template <bool kCache>
+using HugeWST = AWS<32768, 6144, 6144, 6144, 32768, kCache>;
 
 __device__ __forceinline__ Tet ld_tet(const Tet* T, uint32_t t) { return load_tet_cg(T, t); }
 
@@ -532,13 +531,29 @@ __device__ __forceinline__ uint32_t lock_entry(const W& w, int i, int nc, int na
   return i < nx ? w.ex[i] : kNone;
 }
 
-// Releases the locks of the entries this lane took (bit k of `held` = entry lane + 32 k).
+// The locks a lane holds. With the edge table (few entries a lane) bit k stands for entry
+// lane + 32 k, and every entry is tried, so that the compare-and-swaps overlap; larger workspaces
+// count: the entries are taken in order up to the first that is held by another warp.
 template <class W>
-__device__ __forceinline__ void release_held(const W& w, uint32_t* lock, typename W::Held held, int nc, int na,
-                                             int nx) {
+__device__ __forceinline__ bool take_locks(const W& w, uint32_t* lock, uint32_t me, int nc, int na, int nx,
+                                           uint32_t* held) {
+  const int lane = threadIdx.x & 31, nl = nc + na + nx;
+  bool ok = true;
+  uint32_t h = 0;
+  for (int k = 0; lane + 32 * k < nl && (W::kTable || ok); ++k) {
+    if (atomicCAS(&lock[lock_entry(w, lane + 32 * k, nc, na, nx)], 0u, me) != 0u) ok = false;
+    else h = W::kTable ? h | (1u << k) : h + 1;
+  }
+  *held = h;
+  return __all_sync(kFull, ok);
+}
+
+// Releases the locks of the entries this lane took.
+template <class W>
+__device__ __forceinline__ void release_held(const W& w, uint32_t* lock, uint32_t held, int nc, int na, int nx) {
   const int lane = threadIdx.x & 31;
-  for (int k = 0; held; ++k, held >>= 1)
-    if (held & 1u) __stcg(&lock[lock_entry(w, lane + 32 * k, nc, na, nx)], 0u);
+  for (int k = 0; W::kTable ? (held >> k) != 0 : k < (int)held; ++k)
+    if (!W::kTable || ((held >> k) & 1u)) __stcg(&lock[lock_entry(w, lane + 32 * k, nc, na, nx)], 0u);
 }
 
 // Takes n slots from the warp's pool into w.ex, refilling it from the allocator (free list,
@@ -589,17 +604,17 @@ __device__ __forceinline__ void pool_give(const Ctx& c, W& w, const uint32_t* s,
   __syncwarp();
 }
 
-// One attempt at inserting p (steps 1-5). w.hint is the warp's last ball, updated on success.
+// One attempt at inserting p (steps 1-5). start: where a walk begins (kNone: where p was last
+// located, else the grid's hints). w.hint is the warp's last ball, updated on success.
 template <bool kExact, class W>
 __device__ __forceinline__ int try_insert(const Ctx& c, W& w, uint32_t* lock, uint32_t me, uint32_t p,
-                                          const InsertLog& lg, bool ball_start) {
+                                          const InsertLog& lg, bool ball_start, uint32_t start) {
   const int lane = threadIdx.x & 31;
   const PtF FP = load_ptf(c.ptf, p);
   // 1. a start in conflict with p. Consecutive points of a segment are close, so p is often
   //    inside the circumsphere of a tetrahedron of the previous ball (it will be joined to the
   //    previous point): the search's first pass tests them all, without a walk. Otherwise walk.
   int ball = ball_start ? w.bn : 0;
-  uint32_t start = w.hint;
   __syncwarp();
   if (lane == 0) w.bn = 0;  // used once
   for (int attempt = 0; attempt <= kARetry;) {
@@ -632,6 +647,7 @@ __device__ __forceinline__ int try_insert(const Ctx& c, W& w, uint32_t* lock, ui
     const int r = cavity_async<kExact>(c, w, ball, t0, tn, p, FP);
     ball = 0;
     if (r == kANoSeed) continue;  // walk from the warp's last ball
+    if (r == kABig && lane == 0) c.point_hint[p] = w.cl[0];
     if (r == kABig || r == kAExact) return r;
     start = kNone;  // a further attempt starts from the grid
     ++attempt;
@@ -643,16 +659,9 @@ __device__ __forceinline__ int try_insert(const Ctx& c, W& w, uint32_t* lock, ui
     const int reuse = min(nc, nb), nx = nb - reuse;
     if (nx > 0 && !pool_take(c, w, nx)) return kALost;
     // 3. lock C, A and the extra slots
-    const int nl = nc + na + nx;
-    typename W::Held held = 0;
-    bool ok = true;
-    for (int k = 0; lane + 32 * k < nl; ++k) {
-      const uint32_t s = lock_entry(w, lane + 32 * k, nc, na, nx);
-      if (s == kNone) continue;
-      if (atomicCAS(&lock[s], 0u, me) == 0u) held |= (typename W::Held)1 << k;
-      else ok = false;
-    }
-    if (!__all_sync(kFull, ok)) {
+    uint32_t held;
+    if (!take_locks(w, lock, me, nc, na, nx, &held)) {
+      if (lane == 0) c.point_hint[p] = w.cl[0];  // a retry starts in the cavity
       release_held(w, lock, held, nc, na, nx);
       if (nx > 0) pool_give(c, w, w.ex, nx);
       return kALost;
@@ -795,7 +804,7 @@ __device__ __forceinline__ int try_insert(const Ctx& c, W& w, uint32_t* lock, ui
         __stcg(c.subdet + 2 * (size_t)s, q0);
         __stcg(c.subdet + 2 * (size_t)s + 1, q1);
       }
-      if constexpr (kExact) {  // this kernel keeps no cache: the entry it replaces is void
+      if constexpr (!W::kCache && (kExact || !W::kTable)) {  // no cache kept here: the entry it replaces is void
         if (c.subdet) __stcg(c.subdet + 2 * (size_t)s + 1, make_float4(0.f, 0.f, 0.f, 0.f));
       }
       __stcg(reinterpret_cast<uint32_t*>(&c.tets[out].n) + back, s);
@@ -852,7 +861,7 @@ __device__ __forceinline__ void to_queue(const AsyncIO& io, const Ctx& c, int q,
 
 // A cavity too large for the warp's shared-memory workspace: the same insertion again in a
 // global-memory workspace borrowed from the launch's pool (tried at a few places, never waited
-// for). Returns kABig when none is free or the cavity exceeds it too. The borrowed workspace's
+// for). Returns kABig when the cavity exceeds it too, kALost when none is free. The borrowed workspace's
 // counters, spare slots and ball hint come back to the warp's own. Out of line: it runs for
 // about one point in 1500, and inlined it would double the kernel's instruction footprint.
 template <bool kExact, class W>
@@ -867,7 +876,7 @@ __device__ __noinline__ int try_insert_large(const Ctx& c, const AsyncIO& io, W&
       if (atomicCAS(&io.big_busy[cand], 0u, 1u) == 0u) k = (int)cand;
     }
   k = __shfl_sync(kFull, k, 0);
-  if (k < 0) return kABig;
+  if (k < 0) return kALost;
   LargeWST<W::kCache>& L = static_cast<LargeWST<W::kCache>*>(io.big_ws)[k];
   if (lane == 0) {
     L.fa = w.fa;
@@ -878,7 +887,7 @@ __device__ __noinline__ int try_insert_large(const Ctx& c, const AsyncIO& io, W&
     for (int q = 0; q < 8; ++q) L.cnt[q] = 0;
   }
   __syncwarp();
-  const int r = try_insert<kExact>(c, L, lock, me, p, lg, false);
+  const int r = try_insert<kExact>(c, L, lock, me, p, lg, false, kNone);
   pool_give(c, w, L.pool, L.np);
   if (lane == 0) {
     w.cnt[0] += L.cnt[0];
@@ -895,11 +904,14 @@ __device__ __noinline__ int try_insert_large(const Ctx& c, const AsyncIO& io, W&
   return r;
 }
 
-// One warp's work: segment [b0, e0) of io's list in order, deferred points retried after later
-// insertions, then what is left handed on, unused slots returned and counters flushed.
+// One warp's work: its share [k0, k1) of the points carried over from earlier launches, each
+// started where it was last located, then segment [b0, e0) of io's list in order; deferred points
+// are retried after later insertions. At the end what is left is handed on, unused slots return
+// and counters are flushed.
 template <bool kExact, class W>
 __device__ __forceinline__ void run_segment(const Ctx& c, const AsyncIO& io, W& w, uint32_t* lock, uint32_t me,
-                                            uint64_t b0, uint64_t e0, const uint8_t* vflag, const InsertLog& lg) {
+                                            uint64_t b0, uint64_t e0, uint64_t k0, uint64_t k1, const uint8_t* vflag,
+                                            const InsertLog& lg) {
   const int lane = threadIdx.x & 31;
   if (lane == 0) {
     w.fa = __ldcg(&c.st->free_avail);
@@ -907,7 +919,7 @@ __device__ __forceinline__ void run_segment(const Ctx& c, const AsyncIO& io, W& 
     w.np = 0;
     w.bn = 0;
     for (int k = 0; k < 8; ++k) w.cnt[k] = 0;
-    w.hint = b0 < e0 ? c.point_hint[io.q ? io.q[b0] : io.qbase + (uint32_t)b0] : kNone;
+    w.hint = kNone;
   }
   __syncwarp();
   int nd = 0, dhead = 0;
@@ -915,23 +927,28 @@ __device__ __forceinline__ void run_segment(const Ctx& c, const AsyncIO& io, W& 
   int since = 0;  // insertions since the last retry of a deferred point
   for (;;) {
     __syncwarp();  // lane 0's writes to the deferred list are seen by every lane below
-    uint32_t p;
-    bool retried = false;
-    if (nd > 0 && (i >= e0 || since >= 4)) {
+    uint32_t p, start = kNone;
+    bool retried = false, follows = false;  // follows: the point after the last inserted one
+    if (nd > 0 && ((i >= e0 && k0 >= k1) || since >= 4)) {
       p = w.defer[dhead];
       dhead = (dhead + 1) % kADefer;
       --nd;
       retried = true;
       since = 0;
+    } else if (k0 < k1) {
+      p = io.carry[k0];
+      ++k0;
     } else if (i < e0) {
       p = io.q ? io.q[i] : io.qbase + (uint32_t)i;
+      follows = i > b0;
+      if (follows) start = w.hint;
       ++i;
       if (vflag[p] != 0) continue;
     } else {
       break;
     }
     if (lane == 0) w.cnt[2] += 1;
-    int r = try_insert<kExact>(c, w, lock, me, p, lg, io.ball_start != 0);
+    int r = try_insert<kExact>(c, w, lock, me, p, lg, follows && io.ball_start != 0, start);
     if constexpr (W::kTable) {
       if (r == kABig) r = try_insert_large<kExact>(c, io, w, lock, me, p, lg);
     }
@@ -992,14 +1009,15 @@ __global__ void __launch_bounds__(kAW * 32, kMinBlocks) k_async(Ctx c, AsyncIO i
   const uint32_t seg = blockIdx.x * kAW + wid;
   if (seg >= io.W) return;
   uint64_t b0, e0;
-  if (io.bounds) {  // segments of equal predicted work (the learned schedule)
+  if (io.bounds && io.m) {  // segments of equal predicted work (the learned schedule)
     b0 = io.bounds[seg];
     e0 = io.bounds[seg + 1];
   } else {
     b0 = (uint64_t)seg * io.L;
     e0 = b0 + io.L < io.m ? b0 + io.L : io.m;
   }
-  run_segment<kExact>(c, io, s_ws[wid], lock, seg + 1, b0, e0, vflag, lg);
+  run_segment<kExact>(c, io, s_ws[wid], lock, seg + 1, b0, e0, io.carry_n * seg / io.W, io.carry_n * (seg + 1) / io.W, vflag,
+                      lg);
 }
 
 // Large cavities (beyond the shared-memory workspaces): the same insertion with each warp's
@@ -1007,12 +1025,10 @@ __global__ void __launch_bounds__(kAW * 32, kMinBlocks) k_async(Ctx c, AsyncIO i
 // runs beside k_async, so warp numbers may repeat across the two.
 template <bool kCache, bool kExact>
 __global__ void __launch_bounds__(128) k_async_big(Ctx c, AsyncIO io, uint32_t* lock, const uint8_t* __restrict__ vflag,
-                                                  InsertLog lg, LargeWST<kCache>* ws) {
+                                                  InsertLog lg, HugeWST<kCache>* ws) {
   const uint32_t seg = blockIdx.x * 4 + (threadIdx.x >> 5);
   if (seg >= io.W) return;
-  const uint64_t b0 = (uint64_t)seg * io.L;
-  const uint64_t e0 = b0 + io.L < io.m ? b0 + io.L : io.m;
-  run_segment<kExact>(c, io, ws[seg], lock, seg + 1, b0, e0, vflag, lg);
+  run_segment<kExact>(c, io, ws[seg], lock, seg + 1, 0, 0, io.carry_n * seg / io.W, io.carry_n * (seg + 1) / io.W, vflag, lg);
 }
 
 // Folds the allocator of the launch into the free list, as a round close does
@@ -1029,8 +1045,9 @@ __global__ void k_async_close_copy(Ctx c) {
     c.freelist[nfa + i] = __ldcg(&c.pending[i]);
 }
 
-__global__ void k_async_close_state(Ctx c) {
+__global__ void k_async_close_state(Ctx c, int consumed_q) {
   DevState* st = c.st;
+  if (consumed_q >= 0) st->q[consumed_q] = 0;  // the launch took the whole list
   const unsigned long long used = st->alloc_cursor, fa = st->free_avail;
   const unsigned long long consumed = used < fa ? used : fa, nfa = fa - consumed;
   unsigned long long np = st->pending;
@@ -1046,57 +1063,54 @@ __global__ void k_async_close_state(Ctx c) {
   st->blocks_done = 0;
 }
 
-int g_async_blocks = 0;  // resident blocks per SM the kernel is built for (0: not chosen yet)
+// Resident blocks per SM the FP32 kernel is built for: 8 (32 warps per SM at 64 registers)
+// measured fastest, 255 ms per 1e7 uniform step when first built against 265 at 6 (80 registers),
+// 276 at 5 and 301 at 4; 6 is kept for sweeps. The kernel with the exact stages holds 128 registers
+// at 4 blocks: its calls save and restore fewer of them.
+constexpr int kExactBlocks = 4;
 
-int async_blocks_per_sm() {
-  if (!g_async_blocks) {
-    // 8 resident blocks (32 warps) per SM at 64 registers measured fastest: 255 ms per 1e7 uniform
-    // step against 265 (6 blocks, 80 registers), 276 (5, 96) and 301 (4, 128)
-    int v = 8;
-    if (const char* e = std::getenv("DT_ASYNC_BLOCKS")) v = std::atoi(e);
-    g_async_blocks = (v == 4 || v == 5 || v == 6 || v == 7 || v == 8) ? v : 8;
-  }
-  return g_async_blocks;
+bool async_six_blocks() {
+  static const bool six = [] {
+    const char* e = std::getenv("DT_ASYNC_BLOCKS");
+    const int v = e ? std::atoi(e) : 8;
+    return v >= 4 && v <= 6;
+  }();
+  return six;
 }
 
 }  // namespace
 
 int async_launch(const Ctx& c, const AsyncIO& io, uint32_t* lock, const uint8_t* vflag, const InsertLog& lg,
                  cudaStream_t s) {
-  if (io.W == 0 || io.m == 0) return DT_OK;
+  if (io.W == 0 || (io.m == 0 && io.carry_n == 0)) return DT_OK;
   Ctx cc = c;
   cc.coherent = 1;
   cc.max_walk = io.max_walk;
   const unsigned blocks = (io.W + kAW - 1) / kAW;
-  // the sub-determinant cache ablation is built for the default 8 blocks per SM only
-  switch (c.subdet ? 0 : async_blocks_per_sm()) {
-    case 0: k_async<8, true><<<blocks, kAW * 32, 0, s>>>(cc, io, lock, vflag, lg); break;
-    case 4: k_async<4><<<blocks, kAW * 32, 0, s>>>(cc, io, lock, vflag, lg); break;
-    case 5: k_async<5><<<blocks, kAW * 32, 0, s>>>(cc, io, lock, vflag, lg); break;
-    case 6: k_async<6><<<blocks, kAW * 32, 0, s>>>(cc, io, lock, vflag, lg); break;
-    case 7: k_async<7><<<blocks, kAW * 32, 0, s>>>(cc, io, lock, vflag, lg); break;
-    default: k_async<8><<<blocks, kAW * 32, 0, s>>>(cc, io, lock, vflag, lg); break;
-  }
+  if (io.exact) k_async<kExactBlocks, false, true><<<blocks, kAW * 32, 0, s>>>(cc, io, lock, vflag, lg);
+  else if (c.subdet) k_async<8, true><<<blocks, kAW * 32, 0, s>>>(cc, io, lock, vflag, lg);
+  else if (async_six_blocks()) k_async<6><<<blocks, kAW * 32, 0, s>>>(cc, io, lock, vflag, lg);
+  else k_async<8><<<blocks, kAW * 32, 0, s>>>(cc, io, lock, vflag, lg);
   k_async_close_copy<<<152, 256, 0, s>>>(cc);
-  k_async_close_state<<<1, 1, 0, s>>>(cc);
+  k_async_close_state<<<1, 1, 0, s>>>(cc, io.carry_n ? io.carry_q : -1);
   g_kernel_launches += 3;
   return cudaPeekAtLastError() == cudaSuccess ? DT_OK : DT_ECUDA;
 }
 
-size_t async_big_ws_bytes() { return sizeof(LargeWS); }
+size_t async_borrow_ws_bytes() { return sizeof(LargeWS); }
+size_t async_big_ws_bytes() { return sizeof(HugeWST<false>); }
 
 int async_launch_big(const Ctx& c, const AsyncIO& io, uint32_t* lock, const uint8_t* vflag, const InsertLog& lg,
                      void* ws, cudaStream_t s) {
-  if (io.W == 0 || io.m == 0) return DT_OK;
+  if (io.W == 0 || io.carry_n == 0) return DT_OK;
   Ctx cc = c;
   cc.coherent = 1;
   cc.max_walk = io.max_walk;
-  if (c.subdet)
-    k_async_big<true, false><<<(io.W + 3) / 4, 128, 0, s>>>(cc, io, lock, vflag, lg, static_cast<LargeWST<true>*>(ws));
-  else
-    k_async_big<false, false><<<(io.W + 3) / 4, 128, 0, s>>>(cc, io, lock, vflag, lg, static_cast<LargeWS*>(ws));
+  HugeWST<false>* w = static_cast<HugeWST<false>*>(ws);
+  if (io.exact) k_async_big<false, true><<<(io.W + 3) / 4, 128, 0, s>>>(cc, io, lock, vflag, lg, w);
+  else k_async_big<false, false><<<(io.W + 3) / 4, 128, 0, s>>>(cc, io, lock, vflag, lg, w);
   k_async_close_copy<<<152, 256, 0, s>>>(cc);
-  k_async_close_state<<<1, 1, 0, s>>>(cc);
+  k_async_close_state<<<1, 1, 0, s>>>(cc, io.carry_q);
   g_kernel_launches += 3;
   return cudaPeekAtLastError() == cudaSuccess ? DT_OK : DT_ECUDA;
 }
@@ -1107,14 +1121,25 @@ int async_max_warps() {
     int dev = 0, sms = 0, per = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const int mb = async_blocks_per_sm();
-    cudaError_t e = mb == 4 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_async<4>, kAW * 32, 0)
-                  : mb == 5 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_async<5>, kAW * 32, 0)
-                  : mb == 6 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_async<6>, kAW * 32, 0)
-                  : mb == 7 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_async<7>, kAW * 32, 0)
-                            : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_async<8>, kAW * 32, 0);
-    if (e != cudaSuccess) per = mb;
+    const cudaError_t e =
+        async_six_blocks() ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_async<6>, kAW * 32, 0)
+                           : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_async<8>, kAW * 32, 0);
+    if (e != cudaSuccess) per = async_six_blocks() ? 6 : 8;
     cached = std::max(1, sms * std::max(per, 1) * kAW);
+  }
+  return cached;
+}
+
+int async_max_warps_exact() {
+  static int cached = 0;
+  if (!cached) {
+    int dev = 0, sms = 0, per = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_async<kExactBlocks, false, true>, kAW * 32, 0) !=
+        cudaSuccess)
+      per = kExactBlocks;
+    cached = std::min(std::max(1, sms * std::max(per, 1) * kAW), async_max_warps());
   }
   return cached;
 }

@@ -53,30 +53,34 @@ enum DevError : unsigned int {
   kErrWalk = 7,       // walk could not find a live start tetrahedron
 };
 
-// Counters and per-round allocator state, one instance in device memory per handle.
+// Counters and per-round allocator state, one instance in device memory per handle. What every
+// warp updates while a launch runs (the allocator's cursor, the freed slots, the queues, the
+// exact predicates' counters) has a cache line each, so that they do not queue behind one another.
 struct DevState {
   unsigned long long stamp;          // round stamp: upper 32 bits of claim priorities
   unsigned long long bump;           // first never-used tetrahedron slot
   unsigned long long capacity;       // tetrahedron slots allocated
   unsigned long long free_avail;     // free-list entries usable this round
-  unsigned long long alloc_cursor;   // virtual allocation cursor of this round
-  unsigned long long pending;        // slots freed this round (appended after the round)
   unsigned long long free_capacity;  // size of the free-list array
-  unsigned long long q[6];           // queue lengths: 0 next pass, 1 large cavities,
-                                     // 2 large-cavity retries, 3 serial path,
-                                     // 4 cavities too large for the shared-memory large rounds,
-                                     // 5 points the asynchronous engine hands to the rounds
   unsigned int blocks_done;          // blocks of the insert kernel that finished this round
-  unsigned int pad1;
   unsigned int error;                // first DevError raised
   unsigned int error_info;
   unsigned int anchor;               // a tetrahedron known to be live
-  unsigned int pad0;
+  alignas(128) unsigned long long alloc_cursor;  // virtual allocation cursor of this round
+  alignas(128) unsigned long long pending;       // slots freed this round (appended after the round)
+  alignas(128) unsigned long long q[7];  // queue lengths: 0 next pass, 1 large cavities,
+                                         // 2 large-cavity retries, 3 serial path,
+                                         // 4 cavities too large for the shared-memory large rounds,
+                                         // 5 points for the asynchronous engine's exact kernels,
+                                         // 6 with 0, the lists of one asynchronous launch and the next
   // statistics
-  unsigned long long n_inserted, n_conflicts, n_attempts, n_walk_limit, n_big, n_dups;
-  unsigned long long sum_cavity, sum_ball, sum_walk, n_exact, n_sos, max_walk;
+  alignas(128) unsigned long long n_inserted;
+  unsigned long long n_conflicts, n_attempts, n_walk_limit, n_big, n_dups;
+  unsigned long long sum_cavity, sum_ball, sum_walk, max_walk;
   unsigned long long n_restart;  // asynchronous insertions restarted after a failed re-read
   unsigned long long n_inserted_async;  // insertions made by the asynchronous engine
+  alignas(128) unsigned long long n_exact;
+  alignas(128) unsigned long long n_sos;
 };
 
 __device__ __forceinline__ void raise_error(DevState* st, unsigned int code, unsigned int info) {

@@ -22,8 +22,8 @@ constexpr int kCavWarps = 4;  // candidates per block of the cavity kernel (4 me
 constexpr int kInsWarps = 8;  // candidates per block of the ball kernel
 constexpr uint32_t kDefaultWalk = 48;          // walk steps per pass (a longer walk resumes next pass)
 constexpr uint32_t kAsyncWalk = 4096;          // walk steps per attempt of the asynchronous engine
-constexpr uint32_t kAsyncBigWarps = 512;       // warps (global-memory workspaces) of its large-cavity kernel
-constexpr uint32_t kAsyncBorrow = 256;         // large-cavity workspaces the main kernel's warps may borrow
+constexpr uint32_t kAsyncBigWarps = 64;        // warps (global-memory workspaces) of its large-cavity kernel
+constexpr uint32_t kAsyncBorrow = 512;         // large-cavity workspaces the main kernel's warps may borrow
 constexpr uint64_t kLongWalkBelow = 8192;      // retry lists shorter than this walk up to
 constexpr uint32_t kLongWalkSteps = 1u << 14;  // this many steps per pass
 constexpr uint32_t kScratchStride = kCMax + kFMax;
@@ -34,8 +34,9 @@ constexpr int kQBig = 1;    // cavity too large for shared memory: large-cavity 
 constexpr int kQBig2 = 2;   // lost a conflict in a large-cavity round: next large-cavity round
 constexpr int kQHuge = 3;   // cavity too large even for the large-cavity workspace: serial path
 constexpr int kQBigG = 4;   // cavity too large for the shared-memory large rounds: global-memory rounds
-constexpr int kQExact = 5;  // the asynchronous engine could not decide a predicate: round-based rounds
-constexpr int kNumQueues = 6;
+constexpr int kQExact = 5;  // the asynchronous engine's FP32 stage could not decide a predicate
+constexpr int kQCarry = 6;  // asynchronous engine: with kQNext, the lists of one launch and the next
+constexpr int kNumQueues = 7;
 static_assert(sizeof(DevState::q) / sizeof(DevState::q[0]) == kNumQueues, "one length per queue");
 
 // Large-cavity rounds, first tier: one warp per candidate with its workspaces in dynamic shared
@@ -915,7 +916,6 @@ struct dt_handle {
   double alpha = 0.02;   // candidates per round = alpha * mesh vertices (measured best at 1e7 and 1e8)
   double alpha_refine = 0.01;  // the same during dt_refine
   double refine_rebuild = 0.25;  // dt_refine: rebuild the mesh when an iteration adds this share
-  bool refine_rebuild_async = true;  // ... and let the rebuild use the asynchronous engine
   double gamma = 0.3;    // wave size = gamma * mesh vertices (round-based and batch engines)
   double gamma_async = 2.0;  // the asynchronous engine's waves (measured: 164.9 ms per 1e7 uniform
                              // step at 2.0 against 166.8 at 1.0, 175.0 at 0.5 and 185.6 at 0.3;
@@ -931,12 +931,9 @@ struct dt_handle {
                                    // 147 with lists of 32 or more, 152 with 256, 155 with 2048); a
                                    // retry pass without progress moves the list to the rounds anyway
   uint64_t async_warps = 0;        // cap on the asynchronous engine's warps (0: all that fit)
-  bool async_off = false;          // this call's inputs defeat the asynchronous engine's FP32 stage
   uint32_t async_ball_start = 1;   // start from the previous ball's tetrahedra before walking
-  double async_handoff_frac = 0.2; // hand-offs per point of a pass that switch it off for the call
-                                   // (degenerate mix: 42.8 Mtets/s at 0.2, 34.7 at 0.5; never
-                                   // switching off sends points back and forth, 3.2)
-  uint64_t async_handoff_min = 4096; // passes shorter than this never switch it off
+  double async_handoff_frac = 0.1;  // hand-offs per point given so far that switch a call to the
+  uint64_t async_handoff_min = 16;  // exact kernels, and the fewest that do
   uint8_t* wcost = nullptr;        // learned schedule: predicted insertion work per vertex
   bool wcost_ready = false;
   uint32_t* seg_prefix = nullptr;  // prefix sums of a pass's predicted work
@@ -1300,6 +1297,7 @@ int run_big(dt_handle* h, const Ctx& c) {
     if (tier == 2) {
       int rc = set_queue_lengths(h, {kQBigG});
       if (rc != DT_OK) return rc;
+      h->st_host->q[kQBigG] = 0;  // the tier below reads it, also when no round of this one runs
     } else if (smem) {
       // the cavities the shared-memory tier could not hold become the global tier's list
       std::swap(h->queue[kQBig], h->queue[kQBigG]);
@@ -1342,23 +1340,35 @@ int run_big(dt_handle* h, const Ctx& c) {
   return DT_OK;
 }
 
-// Large cavities of an asynchronous pass: the asynchronous kernel with global-memory
+int zero_queue(dt_handle* h, int q) {
+  h->st_host->q[q] = 0;
+  return cudaMemsetAsync(&h->st->q[q], 0, 8, h->stream) == cudaSuccess ? DT_OK : DT_ECUDA;
+}
+
+// Large cavities of an asynchronous pass: the asynchronous kernel with large global-memory
 // workspaces, again on its losers while that makes progress; whatever is left (and cavities
 // beyond those workspaces) goes through the large-cavity rounds and the serial path.
-int run_big_async(dt_handle* h, const Ctx& c) {
+int run_big_async(dt_handle* h, const Ctx& c, bool exact) {
   uint64_t nbig = h->st_host->q[kQBig];
   if (nbig > 0 && !h->async_big_ws &&
       cudaMalloc(&h->async_big_ws, (size_t)kAsyncBigWarps * async_big_ws_bytes()) != cudaSuccess)
     return DT_ENOMEM;
   for (int iter = 0; nbig > 0 && iter < 8; ++iter) {
-    int rc = set_queue_lengths(h, {kQBig2});
+    int rc = zero_queue(h, kQBig2);
     if (rc != DT_OK) return rc;
-    uint64_t W = std::min<uint64_t>(nbig, kAsyncBigWarps);
-    const uint64_t L = (nbig + W - 1) / W;
-    W = (nbig + L - 1) / L;
-    AsyncIO io{h->queue[kQBig], 0, nbig, L, (uint32_t)W, h->cfg.max_walk_steps ? h->cfg.max_walk_steps : kAsyncWalk,
-               h->queue[kQBig2], kQBig2, h->queue[kQHuge], kQHuge, h->queue[kQExact], kQExact,
-               nullptr, nullptr, nullptr, 0, h->async_ball_start};
+    AsyncIO io{};
+    io.W = (uint32_t)std::min<uint64_t>(nbig, kAsyncBigWarps);
+    io.max_walk = h->cfg.max_walk_steps ? h->cfg.max_walk_steps : kAsyncWalk;
+    io.carry = h->queue[kQBig];
+    io.carry_n = nbig;
+    io.carry_q = kQBig;
+    io.lose_out = h->queue[kQBig2];
+    io.lose_q = kQBig2;
+    io.big_out = h->queue[kQHuge];
+    io.big_q = kQHuge;
+    io.exact_out = h->queue[kQExact];
+    io.exact_q = kQExact;
+    io.exact = exact;
     if ((rc = async_launch_big(c, io, h->lock, h->vflag, make_log(h), h->async_big_ws, h->stream)) != DT_OK)
       return rc;
     h->stats.n_async++;
@@ -1371,28 +1381,35 @@ int run_big_async(dt_handle* h, const Ctx& c) {
     if (left >= nbig) break;  // no progress: the rounds below settle the rest
     nbig = left;
   }
-  return run_big(h, c);
+  if (h->st_host->q[kQBig] || h->st_host->q[kQHuge]) {
+    const int rc = run_big(h, c);
+    if (rc != DT_OK) return rc;
+  }
+  int rc = zero_queue(h, kQBig);
+  return rc != DT_OK ? rc : zero_queue(h, kQHuge);
 }
 
 // One pass: rounds over q[0..m) (or the vertex range qbase + [0, m)) split into R segments of
 // length L (segment s offers q[s*L + j] in round j), then the large cavities of the pass.
 int run_pass(dt_handle* h, const Ctx& c, const uint32_t* q, uint32_t qbase, uint64_t m, bool reset_next,
-             float alpha_scale = 1.f, bool rounds_only = false);
+             float alpha_scale = 1.f);
 
-
-int run_pass_async(dt_handle* h, const Ctx& c, const uint32_t* q, uint32_t qbase, uint64_t m, bool reset_next) {
-  uint64_t mesh = h->st_host->n_inserted;
+// One launch of the asynchronous engine: the points carried over (carry_n of them; the queue
+// carry_q is emptied when it is not negative) and the list q[0, m). What it does not insert goes to the
+// queues out, kQBig (settled here) and kQExact.
+int run_pass_async(dt_handle* h, const Ctx& c, const uint32_t* q, uint64_t m, const uint32_t* carry, uint64_t carry_n,
+                   int carry_q, int out, bool exact) {
+  const uint64_t mesh = h->st_host->n_inserted;
   uint64_t W = (uint64_t)std::max(1.0, h->alpha_async * (double)mesh);
   W = std::min<uint64_t>(W, h->async_warps ? h->async_warps : (uint64_t)async_max_warps());
-  W = std::min<uint64_t>(W, m);
+  if (exact) W = std::min<uint64_t>(W, (uint64_t)async_max_warps_exact());
+  W = std::min<uint64_t>(W, std::max(m, carry_n));
   const uint64_t L = (m + W - 1) / W;
-  W = (m + L - 1) / L;
-  int rc = reset_next ? set_queue_lengths(h, {kQNext, kQBig, kQHuge}) : set_queue_lengths(h, {kQBig, kQHuge});
-  if (rc != DT_OK) return rc;
-  if ((rc = set_queue_lengths(h, {kQExact})) != DT_OK) return rc;
+  if (m >= carry_n) W = (m + L - 1) / L;
+  int rc = DT_OK;
   // learned schedule: segments of equal predicted work (a fixed part plus the predicted cavity)
   const uint32_t* seg_bounds = nullptr;
-  if (h->wcost_ready && h->cfg.schedule == DT_SCHED_LEARNED) {
+  if (m > 0 && h->wcost_ready && h->cfg.schedule == DT_SCHED_LEARNED) {
     if (m > h->cap_seg) {
       cudaFree(h->seg_prefix);
       h->seg_prefix = nullptr;
@@ -1401,22 +1418,22 @@ int run_pass_async(dt_handle* h, const Ctx& c, const uint32_t* q, uint32_t qbase
     }
     if (!h->seg_bounds && cudaMalloc(&h->seg_bounds, ((size_t)async_max_warps() + 1) * 4) != cudaSuccess)
       return DT_ENOMEM;
-    k_seg_cost<<<grid_for(m, 256), 256, 0, h->stream>>>(q, qbase, m, h->wcost, h->seg_prefix);
+    k_seg_cost<<<grid_for(m, 256), 256, 0, h->stream>>>(q, 0, m, h->wcost, h->seg_prefix);
     prefix_sum_exclusive(h->seg_prefix, m, h->ows.hist, h->stream);
-    k_seg_bounds<<<grid_for(W + 1, 256), 256, 0, h->stream>>>(h->seg_prefix, q, qbase, m, h->wcost, (uint32_t)W,
+    k_seg_bounds<<<grid_for(W + 1, 256), 256, 0, h->stream>>>(h->seg_prefix, q, 0, m, h->wcost, (uint32_t)W,
                                                                h->seg_bounds);
     g_kernel_launches += 2;
     seg_bounds = h->seg_bounds;
   }
   if (!h->async_borrow_ws) {
-    if (cudaMalloc(&h->async_borrow_ws, (size_t)kAsyncBorrow * async_big_ws_bytes()) != cudaSuccess ||
+    if (cudaMalloc(&h->async_borrow_ws, (size_t)kAsyncBorrow * async_borrow_ws_bytes()) != cudaSuccess ||
         cudaMalloc(&h->async_borrow_busy, kAsyncBorrow * sizeof(unsigned int)) != cudaSuccess)
       return DT_ENOMEM;
     cudaMemsetAsync(h->async_borrow_busy, 0, kAsyncBorrow * sizeof(unsigned int), h->stream);
   }
-  AsyncIO io{q, qbase, m, L, (uint32_t)W, h->cfg.max_walk_steps ? h->cfg.max_walk_steps : kAsyncWalk,
-             h->queue[kQNext], kQNext, h->queue[kQBig], kQBig, h->queue[kQExact], kQExact,
-             seg_bounds, h->async_borrow_ws, h->async_borrow_busy, kAsyncBorrow, h->async_ball_start};
+  AsyncIO io{q, 0, m, L, (uint32_t)W, h->cfg.max_walk_steps ? h->cfg.max_walk_steps : kAsyncWalk,
+             carry, carry_n, carry_q, h->queue[out], out, h->queue[kQBig], kQBig, h->queue[kQExact], kQExact,
+             exact ? 1 : 0, seg_bounds, h->async_borrow_ws, h->async_borrow_busy, kAsyncBorrow, h->async_ball_start};
   const bool prof = (h->cfg.flags & DT_FLAG_PROFILE) != 0;
   if (prof) cudaEventRecord(h->ev[3], h->stream);
   if ((rc = async_launch(c, io, h->lock, h->vflag, make_log(h), h->stream)) != DT_OK) return rc;
@@ -1429,26 +1446,11 @@ int run_pass_async(dt_handle* h, const Ctx& c, const uint32_t* q, uint32_t qbase
     cudaEventElapsedTime(&ms, h->ev[3], h->ev[4]);
     h->stats.ms_async += ms;
   }
-  // large cavities now (deferring them to the end of the BRIO round was measured slower: they
-  // then meet each other, 592 instead of 395 rounds per 1e7 uniform step)
-  if ((rc = run_big_async(h, c)) != DT_OK) return rc;
-  // points whose predicates the asynchronous engine's FP32 stage could not decide: one
-  // round-based pass with the full predicate cascade (its losers join the next pass's list)
-  const uint64_t ne = h->st_host->q[kQExact];
-  if (ne == 0) return DT_OK;
-  h->stats.n_exact_handoff += ne;
-  // when the FP32 stage cannot decide for a fifth of a pass's points (near-degenerate inputs:
-  // lattices, co-spherical surfaces, refinement centres), the work it did was mostly wasted:
-  // the rest of this call runs on the round-based engine. A short retry list says little about
-  // the input (its points are the hard ones by selection), so it never decides this
-  if (m >= h->async_handoff_min && (double)ne > h->async_handoff_frac * (double)m) h->async_off = true;
-  return run_pass(h, c, h->queue[kQExact], 0, ne, false, 1.f, true);
+  return h->st_host->q[kQBig] || h->st_host->q[kQHuge] ? run_big_async(h, c, exact) : DT_OK;
 }
 
 int run_pass(dt_handle* h, const Ctx& c, const uint32_t* q, uint32_t qbase, uint64_t m, bool reset_next,
-             float alpha_scale, bool rounds_only) {
-  if (h->use_async && !h->async_off && !rounds_only && (!reset_next || m >= h->async_min_retry))
-    return run_pass_async(h, c, q, qbase, m, reset_next);
+             float alpha_scale) {
   uint64_t& kind_rounds = reset_next ? h->stats.n_rounds_retry : h->stats.n_rounds_wave;
   uint64_t mesh = h->st_host->n_inserted;
   uint32_t R = choose_segments(h, mesh, m, alpha_scale);
@@ -1499,7 +1501,7 @@ int make_waves(dt_handle* h, uint32_t vbegin, uint32_t vend, int round, uint64_t
   double N = (double)std::max<uint64_t>(h->st_host->n_inserted, 4);
   uint64_t acc = 0;
   while (acc < m && cum.size() < 255) {
-    const double gamma = (h->use_async && !h->async_off) ? h->gamma_async : h->gamma;
+    const double gamma = h->use_async ? h->gamma_async : h->gamma;
     uint64_t w = (uint64_t)std::max(1.0, std::ceil(gamma * N));
     acc = std::min<uint64_t>(m, acc + w);
     cum.push_back((uint32_t)acc);
@@ -1601,9 +1603,7 @@ int run_brio_round(dt_handle* h, uint32_t vbegin, uint32_t vend, int round, uint
     // a short retry list is cheap per round: let its walks run long instead of over many passes
     Ctx cr = c;
     if (!h->cfg.max_walk_steps && nq < kLongWalkBelow) cr.max_walk = kLongWalkSteps;
-    // after a pass that made no progress the round-based engine takes over: its highest-priority
-    // located point always wins, where the asynchronous engine's retries might keep colliding
-    if ((rc = run_pass(h, cr, a2 ? h->ows.v1 : h->ows.v0, 0, nq, true, 1.f, stalled > 0)) != DT_OK) return rc;
+    if ((rc = run_pass(h, cr, a2 ? h->ows.v1 : h->ows.v0, 0, nq, true)) != DT_OK) return rc;
     nq = h->st_host->q[kQNext];
     // every pass shrinks the retry list (its highest-priority located point is inserted, or
     // moves to the large-cavity queue) or advances walks that hit their step limit; three
@@ -1620,11 +1620,108 @@ int run_brio_round(dt_handle* h, uint32_t vbegin, uint32_t vend, int round, uint
   return DT_OK;
 }
 
+// Whether the inputs defeat the asynchronous engine's FP32 stage: once it has handed on more than
+// a tenth of the points it was given (and more than a few), the kernels with the exact stages do
+// the rest of the call. They hold twice the registers, so half the warps are resident.
+bool handoffs_decide(dt_handle* h, uint64_t given) {
+  const uint64_t ne = h->st_host->q[kQExact];
+  return ne >= h->async_handoff_min && (double)ne > h->async_handoff_frac * (double)given;
+}
+
+// The whole call on the asynchronous engine: the BRIO rounds' waves in order, one launch each.
+// Points that lose are carried over to the next wave's launch, where the mesh is larger and the
+// conflicts are fewer, instead of being retried to the last one after every round; only after
+// the last wave is the list drained. Points the FP32 stage cannot decide wait for the end too
+// (few, on generic inputs), or switch the call to the kernels with the exact stages.
+int insert_async(dt_handle* h, uint64_t base, uint64_t n, bool exact) {
+  Ctx c = make_ctx(h);
+  cudaStream_t s = h->stream;
+  const uint32_t max_rounds = h->cfg.max_rounds ? h->cfg.max_rounds : (1u << 22);
+  int cur = kQNext, other = kQCarry, rc = DT_OK;
+  for (int q : {kQNext, kQCarry, kQExact, kQBig, kQHuge})
+    if ((rc = zero_queue(h, q)) != DT_OK) return rc;
+  uint64_t given = 0;
+  std::vector<uint32_t> cum;
+  std::vector<float> scale;
+  for (int r = 0;; ++r) {
+    const uint64_t b = r == 0 ? 0 : brio_round_end(r - 1);
+    if (b >= n) break;
+    const uint64_t e = std::min<uint64_t>(brio_round_end(r), n);
+    if (make_waves(h, (uint32_t)(base + b), (uint32_t)(base + e), r, base, cum, &scale) < 0) return DT_ECUDA;
+    uint64_t off = 0;
+    for (size_t w = 0; w < cum.size(); ++w) {
+      if ((rc = run_pass_async(h, c, h->wlist + off, cum[w] - off, h->queue[cur], h->st_host->q[cur], cur, other,
+                               exact)) != DT_OK)
+        return rc;
+      std::swap(cur, other);
+      given += cum[w] - off;
+      off = cum[w];
+      if (!exact && handoffs_decide(h, given)) {
+        exact = true;
+        h->stats.n_exact_handoff += h->st_host->q[kQExact];
+        if ((rc = run_pass_async(h, c, nullptr, 0, h->queue[kQExact], h->st_host->q[kQExact], kQExact, cur, true)) != DT_OK)
+          return rc;
+      }
+    }
+  }
+  uint32_t pass = 0;
+  int stalled = 0;
+  for (;;) {
+    if (h->stats.n_rounds > max_rounds) {
+      h->last_dev_error = 103;  // host-side: round budget exhausted
+      return DT_ELIMIT;
+    }
+    if (const uint64_t ne = h->st_host->q[kQExact]) {
+      exact = true;
+      h->stats.n_exact_handoff += ne;
+      if ((rc = run_pass_async(h, c, nullptr, 0, h->queue[kQExact], ne, kQExact, cur, true)) != DT_OK) return rc;
+      continue;
+    }
+    const uint64_t nq = h->st_host->q[cur], limited = h->st_host->n_walk_limit;
+    if (nq == 0) return DT_OK;
+    // a list of more points than warps is put into the order of a transformed curve (Section
+    // 3.3), so that the points of a neighbourhood meet in one warp and not in several; the top 24
+    // bits of the 63-bit key (8 levels of the curve) order them well enough
+    const bool rounds = stalled > 0 || nq < h->async_min_retry;
+    const uint32_t* list = h->queue[cur];
+    if (rounds || nq > (uint64_t)(h->alpha_async * (double)h->st_host->n_inserted)) {
+      transformed_keys(h->pts, list, nq, h->bbox_dev, h->cfg.seed + 0x51ED2701ull * (pass + 1) + base, h->ows.k0,
+                       h->ows.v0, s);
+      const bool a2 = radix_sort_pairs_bits(h->ows.k0, h->ows.v0, h->ows.k1, h->ows.v1, nq, 39, 63, h->ows.hist, s);
+      list = a2 ? h->ows.v1 : h->ows.v0;
+    }
+    if (rounds) {
+      // after a pass that made no progress the round-based engine takes over: its highest-priority
+      // located point always wins, where the asynchronous engine's retries might keep colliding
+      Ctx cr = c;
+      if (!h->cfg.max_walk_steps && nq < kLongWalkBelow) cr.max_walk = kLongWalkSteps;
+      if ((rc = zero_queue(h, cur)) != DT_OK || (rc = run_pass(h, cr, list, 0, nq, true)) != DT_OK ||
+          (rc = zero_queue(h, kQBig)) != DT_OK || (rc = zero_queue(h, kQHuge)) != DT_OK)
+        return rc;
+      cur = kQNext;
+      other = kQCarry;
+    } else {
+      if ((rc = run_pass_async(h, c, nullptr, 0, list, nq, cur, other, exact)) != DT_OK) return rc;
+      std::swap(cur, other);
+    }
+    // every pass shrinks the list or advances walks that hit their step limit; three passes that
+    // do neither are a bug, not a schedule
+    const bool walking = h->st_host->n_walk_limit > limited;
+    stalled = (h->st_host->q[cur] >= nq && !walking) ? stalled + 1 : 0;
+    if (stalled >= 3) {
+      h->last_dev_error = 102;  // host-side: retry passes stopped progressing
+      h->last_dev_info = (unsigned)((nq << 8) | (pass & 255));
+      return DT_ELIMIT;
+    }
+    ++pass;
+  }
+}
+
 int schedule_learned(dt_handle* h, uint64_t n);
 
-int insert_impl(dt_handle* h, const double* xyz, uint64_t n, bool allow_async = true) {
+// exact: start with the asynchronous engine's exact kernels (inputs known to be degenerate).
+int insert_impl(dt_handle* h, const double* xyz, uint64_t n, bool exact = false) {
   if (n == 0) return h->has_mesh ? DT_OK : DT_EDEGENERATE;
-  h->async_off = !allow_async;
   if (h->n_pts + n >= 0xFFFFFFF0ull) return DT_EINVAL;
   cudaStream_t s = h->stream;
   cudaEventRecord(h->ev[0], s);
@@ -1712,14 +1809,13 @@ int insert_impl(dt_handle* h, const double* xyz, uint64_t n, bool allow_async = 
     if ((rc = sync_state(h)) != DT_OK) return rc;
     h->has_mesh = true;
   }
-  for (int r = 0;; ++r) {
+  if (h->use_async && (rc = insert_async(h, base, n, exact)) != DT_OK) return rc;
+  for (int r = 0; !h->use_async; ++r) {
     uint64_t b = r == 0 ? 0 : brio_round_end(r - 1);
     if (b >= n) break;
     uint64_t e = std::min<uint64_t>(brio_round_end(r), n);
-    // the first BRIO round of a new triangulation: the asynchronous engine in waves (measured
-    // faster: 181.7 against 197.6 ms per 1e7 uniform step, 31 against 41 ms at 1e5), or the
-    // one-block engine when the round-based engine runs alone
-    if (r == 0 && h->st_host->n_inserted <= 4 && (!h->use_async || std::getenv("DT_CTA")) && !std::getenv("DT_NO_CTA"))
+    // the first BRIO round of a new triangulation runs on one thread block
+    if (r == 0 && h->st_host->n_inserted <= 4 && !std::getenv("DT_NO_CTA"))
       rc = run_cta_round(h, (uint32_t)(base + b), (uint32_t)(base + e), base);
     else
       rc = run_brio_round(h, (uint32_t)(base + b), (uint32_t)(base + e), r, base);
@@ -2244,7 +2340,6 @@ int dt_create(dt_handle** out, const dt_config* cfg) {
   if (const char* a = std::getenv("DT_ALPHA")) h->alpha = std::atof(a);
   if (const char* a = std::getenv("DT_ALPHA_REFINE")) h->alpha_refine = std::atof(a);
   if (const char* a = std::getenv("DT_REFINE_REBUILD")) h->refine_rebuild = std::atof(a);
-  if (const char* a = std::getenv("DT_REFINE_REBUILD_ASYNC")) h->refine_rebuild_async = std::atoi(a) != 0;
   if (const char* g = std::getenv("DT_GAMMA")) h->gamma = std::atof(g);
   if (const char* g = std::getenv("DT_GAMMA_ASYNC")) h->gamma_async = std::atof(g);
   if (const char* a = std::getenv("DT_ALPHA_CTA")) h->alpha_cta = std::atof(a);
@@ -2325,7 +2420,7 @@ int dt_insert(dt_handle* h, const double* xyz_dev, uint64_t n) {
 // the one inserting the ns points into the current mesh would give. An iteration of dt_refine
 // that adds many points into a mesh whose interior is empty meets cavities of thousands of
 // tetrahedra; in BRIO order over all points the cavities stay small.
-int rebuild_with(dt_handle* h, const double* extra, uint64_t ns, bool allow_async) {
+int rebuild_with(dt_handle* h, const double* extra, uint64_t ns) {
   const uint64_t n0 = h->n_pts, N = n0 + ns;
   double* all = nullptr;
   if (cudaMalloc(&all, N * 24) != cudaSuccess) return DT_ENOMEM;
@@ -2334,7 +2429,7 @@ int rebuild_with(dt_handle* h, const double* extra, uint64_t ns, bool allow_asyn
       cudaMemcpyAsync(all + 3 * n0, extra, ns * 24, cudaMemcpyDeviceToDevice, h->stream) != cudaSuccess)
     rc = DT_ECUDA;
   if (rc == DT_OK) rc = clear_mesh(h, true);
-  if (rc == DT_OK) rc = insert_impl(h, all, N, allow_async);
+  if (rc == DT_OK) rc = insert_impl(h, all, N);
   cudaStreamSynchronize(h->stream);
   cudaFree(all);
   return rc;
@@ -2389,11 +2484,11 @@ int dt_refine(dt_handle* h, double size, double ratio, double spacing, const dou
     // also as many new points as refinement had added so far: 1.90 s against 1.75 s)
     if (h->refine_rebuild > 0 && (double)ns >= h->refine_rebuild * (double)h->n_pts) {
       h->alpha = alpha_keep;  // a rebuild is a plain insertion of the whole set
-      rc = rebuild_with(h, h->rws.xyz, ns, h->refine_rebuild_async);
+      rc = rebuild_with(h, h->rws.xyz, ns);
       h->alpha = h->alpha_refine;
     }
     else
-      rc = insert_impl(h, h->rws.xyz, ns, false);
+      rc = insert_impl(h, h->rws.xyz, ns, true);
     if (rc != DT_OK) break;
     added += ns;
     ++iters;

@@ -131,20 +131,26 @@ void transformed_keys(const Pt* pts, const uint32_t* ids, uint64_t m, const doub
 struct Ctx;
 struct InsertLog;
 // Points q[0, m) (or the vertex range qbase + [0, m) when q is null) in W contiguous segments
-// of L points, segment w inserted by warp w in order. Points that lose or walk past max_walk
-// steps go to lose_out (queue lose_q), cavities too large for a warp's workspace to big_out.
+// of L points, segment w inserted by warp w in order, after the warp's share of the carry_n
+// points carried over from earlier launches (carry; queue carry_q, emptied by the launch, when it
+// is not negative). Points that lose or walk past max_walk steps go to lose_out (queue lose_q),
+// cavities too large for a warp's workspaces to big_out.
 struct AsyncIO {
   const uint32_t* q;
   uint32_t qbase;
   uint64_t m, L;
   uint32_t W;
   uint32_t max_walk;
+  const uint32_t* carry;
+  uint64_t carry_n;
+  int carry_q;
   uint32_t* lose_out;
   int lose_q;
   uint32_t* big_out;
   int big_q;
-  uint32_t* exact_out;  // predicates the FP32 stage cannot decide: the round-based engine's
+  uint32_t* exact_out;  // predicates the FP32 stage cannot decide: for a launch with exact set
   int exact_q;
+  int exact;            // 1: the kernel with the FP64 and exact predicate stages
   const uint32_t* bounds;  // W + 1 segment starts (learned schedule), or null: equal segments of L
   void* big_ws;         // global-memory workspaces a warp may borrow for a large cavity (or null)
   unsigned int* big_busy;  // one word per workspace: 0 free, 1 borrowed
@@ -155,11 +161,14 @@ struct AsyncIO {
 // word per tetrahedron slot, all zero before and after.
 int async_launch(const Ctx& c, const AsyncIO& io, uint32_t* lock, const uint8_t* vflag, const InsertLog& lg,
                  cudaStream_t s);
-// Warps of the asynchronous kernel that can be resident on the current device at once.
+// Warps of the asynchronous kernels (FP32 alone; with the exact stages) that can be resident on
+// the current device at once.
 int async_max_warps();
-// The same insertion for cavities beyond the main kernel's shared-memory workspaces: io.W warps
-// with one global-memory workspace of async_big_ws_bytes() each at ws (device). Points whose
-// cavities exceed even these go to io.big_out.
+int async_max_warps_exact();
+size_t async_borrow_ws_bytes();  // one workspace of AsyncIO::big_ws
+// The same insertion of the carried points for cavities beyond those workspaces: io.W warps with
+// one global-memory workspace of async_big_ws_bytes() each at ws (device). Points whose cavities
+// exceed even these go to io.big_out.
 size_t async_big_ws_bytes();
 int async_launch_big(const Ctx& c, const AsyncIO& io, uint32_t* lock, const uint8_t* vflag, const InsertLog& lg,
                      void* ws, cudaStream_t s);
