@@ -45,6 +45,7 @@ namespace {
 constexpr int kAW = 4;            // warps per block of the shared-memory kernel
 constexpr int kADefer = 16;       // aborted points waiting for a retry
 constexpr int kARetry = 3;        // immediate restarts after a failed re-read
+constexpr int kATail = 48;        // further tries at its deferred points by a warp that has no others left
 constexpr uint32_t kAChunk = 32;  // slots taken from the allocator at a time
 
 enum AStatus : int {
@@ -104,6 +105,11 @@ struct AWS : AWSTail<kHashN, kFMaxN, kEdgeSlots> {
   int bn;                       // tetrahedra of the warp's last ball (0: none); slots in slot[]
   int np;                       // slots in the pool
   int nc, na, nb;               // cavity, outside and boundary-facet counts of the last search
+  uint32_t emask;               // the edge hash's slots in use for this ball, less one
+  // the segment's place: here and not in registers, which an insertion needs for itself
+  uint32_t i, e0, k0, k1;       // next and end of the list's points, of the carried ones
+  int nd, dhead, since;         // deferred points, the first of them, insertions since a retry
+  int tail;                     // tries at them after the last of the segment's points
 };
 
 // Shared-memory workspace of the main kernel (cavities of up to 64 tetrahedra and 60 boundary
@@ -240,7 +246,7 @@ __device__ __forceinline__ int inside_maybe_cached(const Ctx& c, uint32_t u, con
 // often cannot decide: lattices, co-spherical and coplanar sets). Out of line: their code and
 // registers stay out of the common path.
 
-// orient3d of the finite tetrahedron v with vertex i replaced by p: the FP64 filter, then exact.
+// orient3d of the finite tetrahedron v with vertex i replaced by p.
 static __device__ __noinline__ int orient_exact_at(const Pt* pts, DevState* st, uint4 v, int i, uint32_t p) {
   const Pt a = load_pt(pts, i == 0 ? p : v.x), b = load_pt(pts, i == 1 ? p : v.y), d = load_pt(pts, i == 2 ? p : v.z),
            e = load_pt(pts, i == 3 ? p : v.w);
@@ -291,6 +297,7 @@ __device__ __forceinline__ int walk_async(const Ctx& c, uint32_t p, const PtF& F
   *steps_out = 0;
   *t_out = kNone;
   int hops = 0;
+#pragma unroll 1
   for (;;) {
     if (t == kNone || t >= c.ntets) t = __ldcg(&c.st->anchor);
     if (t >= c.ntets) return kARestart;
@@ -307,12 +314,15 @@ __device__ __forceinline__ int walk_async(const Ctx& c, uint32_t p, const PtF& F
     if (tet_dead(T.v) || !rec_ok(T, c.ntets, c.npts)) return kARestart;
   }
   uint32_t prev = kNone, steps = 0;
+#pragma unroll 1
   for (;;) {
     if (ghost_pos(T.v) >= 0) break;
     // lane i < 4: orientation of p against the facet opposite vertex i (0: undecided)
     int o = 1;
-    const bool mine = lane < 4 && get4(T.n, lane) != prev;  // p is on this side of the facet just crossed
+    const uint32_t nb = lane < 4 ? get4(T.n, lane) : prev;
+    const bool mine = nb != prev;  // p is on this side of the facet just crossed
     if (mine) {
+
       const PtF F0 = load_ptf(c.ptf, T.v.x), F1 = load_ptf(c.ptf, T.v.y), F2 = load_ptf(c.ptf, T.v.z),
                 F3 = load_ptf(c.ptf, T.v.w);
       o = orient_with_p(c, lane, FP, F0, F1, F2, F3);
@@ -420,6 +430,7 @@ __device__ __forceinline__ int cavity_async(const Ctx& c, W& w, int ball, uint32
                                             const PtF& FP) {
   const int lane = threadIdx.x & 31;
   static_assert(W::kHash % 128 == 0, "cleared by 16 bytes a lane");
+#pragma unroll 1
   for (int i = lane; i < W::kHash / 4; i += 32)
     reinterpret_cast<uint4*>(w.hkey)[i] = make_uint4(kNone, kNone, kNone, kNone);
   __syncwarp();
@@ -454,6 +465,7 @@ __device__ __forceinline__ int cavity_async(const Ctx& c, W& w, int ball, uint32
     __syncwarp();
   }
   int flag = 0, head = 0;
+#pragma unroll 1
   while (head < nc) {
     const int k = lane >> 2, f = lane & 3, ci = head + k;
     const bool active = ci < nc;
@@ -531,18 +543,34 @@ __device__ __forceinline__ uint32_t lock_entry(const W& w, int i, int nc, int na
   return i < nx ? w.ex[i] : kNone;
 }
 
-// The locks a lane holds. With the edge table (few entries a lane) bit k stands for entry
-// lane + 32 k, and every entry is tried, so that the compare-and-swaps overlap; larger workspaces
-// count: the entries are taken in order up to the first that is held by another warp.
+// Ownership words. A slot whose record is replaced (the cavity's, the ball's extra slots) is taken
+// exclusively; an outside tetrahedron, which only gets a back-pointer in a facet slot of its own,
+// is shared: two insertions whose cavities do not touch may hold the same one, each rewriting
+// another facet (the one that faces its cavity). The word is the number of sharers, plus
+// kExclusive while a warp holds it alone; a release subtracts what was added, so that an attempt
+// to share in between is not lost.
+constexpr uint32_t kExclusive = 0x80000000u;
+
+// Takes the locks of the lists' entries. With the edge table (few entries a lane) bit k of *held
+// stands for entry lane + 32 k, and every entry is tried, so that the atomics overlap; larger
+// workspaces count: the entries are taken in order up to the first that is held against them.
 template <class W>
-__device__ __forceinline__ bool take_locks(const W& w, uint32_t* lock, uint32_t me, int nc, int na, int nx,
-                                           uint32_t* held) {
+__device__ __forceinline__ bool take_locks(const W& w, uint32_t* lock, int nc, int na, int nx, uint32_t* held) {
   const int lane = threadIdx.x & 31, nl = nc + na + nx;
   bool ok = true;
   uint32_t h = 0;
+#pragma unroll 1
   for (int k = 0; lane + 32 * k < nl && (W::kTable || ok); ++k) {
-    if (atomicCAS(&lock[lock_entry(w, lane + 32 * k, nc, na, nx)], 0u, me) != 0u) ok = false;
-    else h = W::kTable ? h | (1u << k) : h + 1;
+    const int i = lane + 32 * k;
+    uint32_t* word = &lock[lock_entry(w, i, nc, na, nx)];
+    const bool shared = i >= nc && i < nc + na;
+    const uint32_t old = shared ? atomicAdd(word, 1u) : atomicCAS(word, 0u, kExclusive);
+    if (shared ? old >= kExclusive : old != 0u) {
+      ok = false;
+      if (shared) atomicSub(word, 1u);
+    } else {
+      h = W::kTable ? h | (1u << k) : h + 1;
+    }
   }
   *held = h;
   return __all_sync(kFull, ok);
@@ -552,8 +580,23 @@ __device__ __forceinline__ bool take_locks(const W& w, uint32_t* lock, uint32_t 
 template <class W>
 __device__ __forceinline__ void release_held(const W& w, uint32_t* lock, uint32_t held, int nc, int na, int nx) {
   const int lane = threadIdx.x & 31;
-  for (int k = 0; W::kTable ? (held >> k) != 0 : k < (int)held; ++k)
-    if (!W::kTable || ((held >> k) & 1u)) __stcg(&lock[lock_entry(w, lane + 32 * k, nc, na, nx)], 0u);
+#pragma unroll 1
+  for (int k = 0; W::kTable ? (held >> k) != 0 : k < (int)held; ++k) {
+    const int i = lane + 32 * k;
+    if (!W::kTable || ((held >> k) & 1u))
+      atomicSub(&lock[lock_entry(w, i, nc, na, nx)], i >= nc && i < nc + na ? 1u : kExclusive);
+  }
+}
+
+// The same, and the first `heldx` of this lane's extra slots of a large workspace.
+template <class W>
+__device__ __forceinline__ void release_all(const W& w, uint32_t* lock, uint32_t held, uint32_t heldx, int nc, int na,
+                                            int nx) {
+  release_held(w, lock, held, nc, na, nx);
+  if constexpr (!W::kTable) {
+#pragma unroll 1
+    for (uint32_t k = 0; k < heldx; ++k) atomicSub(&lock[w.ex[(threadIdx.x & 31) + 32 * k]], kExclusive);
+  }
 }
 
 // Takes n slots from the warp's pool into w.ex, refilling it from the allocator (free list,
@@ -562,6 +605,7 @@ template <class W>
 __device__ __forceinline__ bool pool_take(const Ctx& c, W& w, int n) {
   const int lane = threadIdx.x & 31;
   int np = w.np;
+#pragma unroll 1
   while (np < n) {
     unsigned long long base = 0;
     if (lane == 0) base = atomicAdd(&c.st->alloc_cursor, (unsigned long long)kAChunk);
@@ -576,6 +620,7 @@ __device__ __forceinline__ bool pool_take(const Ctx& c, W& w, int n) {
     np += 32;
     __syncwarp();
   }
+#pragma unroll 1
   for (int i = lane; i < n; i += 32) w.ex[i] = w.pool[np - 1 - i];
   __syncwarp();
   if (lane == 0) w.np = np - n;
@@ -589,11 +634,13 @@ __device__ __forceinline__ void pool_give(const Ctx& c, W& w, const uint32_t* s,
   const int lane = threadIdx.x & 31;
   const int np = w.np;
   const int keep = min(n, W::kPool - np);
+#pragma unroll 1
   for (int i = lane; i < keep; i += 32) w.pool[np + i] = s[i];
   if (n > keep) {
     unsigned long long pb = 0;
     if (lane == 0) pb = atomicAdd(&c.st->pending, (unsigned long long)(n - keep));
     pb = __shfl_sync(kFull, pb, 0);
+#pragma unroll 1
     for (int i = keep + lane; i < n; i += 32) {
       if (pb + (i - keep) < c.st->free_capacity) c.pending[pb + (i - keep)] = s[i];
       else raise_error(c.st, kErrFreeList, 0xA7u);
@@ -607,7 +654,7 @@ __device__ __forceinline__ void pool_give(const Ctx& c, W& w, const uint32_t* s,
 // One attempt at inserting p (steps 1-5). start: where a walk begins (kNone: where p was last
 // located, else the grid's hints). w.hint is the warp's last ball, updated on success.
 template <bool kExact, class W>
-__device__ __forceinline__ int try_insert(const Ctx& c, W& w, uint32_t* lock, uint32_t me, uint32_t p,
+__device__ __forceinline__ int try_insert(const Ctx& c, W& w, uint32_t* lock, uint32_t p,
                                           const InsertLog& lg, bool ball_start, uint32_t start) {
   const int lane = threadIdx.x & 31;
   const PtF FP = load_ptf(c.ptf, p);
@@ -617,6 +664,7 @@ __device__ __forceinline__ int try_insert(const Ctx& c, W& w, uint32_t* lock, ui
   int ball = ball_start ? w.bn : 0;
   __syncwarp();
   if (lane == 0) w.bn = 0;  // used once
+#pragma unroll 1
   for (int attempt = 0; attempt <= kARetry;) {
     uint32_t t0 = kNone;
     uint4 tn = make_uint4(kNone, kNone, kNone, kNone);
@@ -656,25 +704,50 @@ __device__ __forceinline__ int try_insert(const Ctx& c, W& w, uint32_t* lock, ui
       continue;
     }
     const int nc = w.nc, na = w.na, nb = w.nb;
-    const int reuse = min(nc, nb), nx = nb - reuse;
-    if (nx > 0 && !pool_take(c, w, nx)) return kALost;
+    const int reuse = min(nc, nb);
+    int nx = nb - reuse;
+    // a large ball's extra slots are taken once its cavity is held: slots that come back from a
+    // lost attempt would wait, beyond what the pool holds, for the launch's end
+    const int nx0 = W::kTable ? nx : 0;
+    if (nx0 > 0 && !pool_take(c, w, nx0)) return kALost;
     // 3. lock C, A and the extra slots
-    uint32_t held;
-    if (!take_locks(w, lock, me, nc, na, nx, &held)) {
+    uint32_t held, heldx = 0;
+    bool locked = take_locks(w, lock, nc, na, nx0, &held);
+    if constexpr (!W::kTable) {
+      if (locked && nx > 0) {
+        if (!pool_take(c, w, nx)) {
+          release_held(w, lock, held, nc, na, 0);
+          return kALost;
+        }
+        bool ok = true;
+#pragma unroll 1
+        for (int i = lane; i < nx && ok; i += 32) {
+          ok = atomicCAS(&lock[w.ex[i]], 0u, kExclusive) == 0u;
+          if (ok) ++heldx;
+        }
+        locked = __all_sync(kFull, ok);
+      } else if (!locked) {
+        nx = 0;
+      }
+    }
+    if (!locked) {
       if (lane == 0) c.point_hint[p] = w.cl[0];  // a retry starts in the cavity
-      release_held(w, lock, held, nc, na, nx);
+      release_all(w, lock, held, heldx, nc, na, nx0);
       if (nx > 0) pool_give(c, w, w.ex, nx);
       return kALost;
     }
     __threadfence();
     // 4. re-read under the locks
     bool same = true;
+#pragma unroll 1
     for (int i = lane; i < nc; i += 32) same = same && same_tet(ld_tet(c.tets, w.cl[i]), w.cr[i]);
+#pragma unroll 1
     for (int i = lane; i < na; i += 32) {
       const uint32_t a = w.al[i];
       same = same && same_v(__ldcg(reinterpret_cast<const uint4*>(c.tets + a)), w.av[i]);
     }
     // which facet of each outside tetrahedron faces the cavity (it is locked: this stays true)
+#pragma unroll 1
     for (int i = lane; i < nb; i += 32) {
       const int ci = w.bl_ci[i], f = w.bl_f[i] & 3;
       const uint32_t u = get4(w.cr[ci].n, f);
@@ -685,26 +758,33 @@ __device__ __forceinline__ int try_insert(const Ctx& c, W& w, uint32_t* lock, ui
     if constexpr (W::kCache) {
       // the cache's decisions were taken on entries read without locks: each is taken again on
       // the entry as it stands under the locks (an entry changes only with its record)
+#pragma unroll 1
       for (int i = lane; i < nc; i += 32) {
         const uint4 v = w.cr[i].v;
         if (ghost_pos(v) < 0) same = same && inside_maybe_cached(c, w.cl[i], v, FP) < 0;
       }
+#pragma unroll 1
       for (int i = lane; i < na; i += 32) {
         const uint4 v = w.av[i];
         if (ghost_pos(v) < 0) same = same && inside_maybe_cached(c, w.al[i], v, FP) > 0;
       }
     }
     if (!__all_sync(kFull, same)) {
-      release_held(w, lock, held, nc, na, nx);
+      release_all(w, lock, held, heldx, nc, na, nx0);
       if (nx > 0) pool_give(c, w, w.ex, nx);
       if (lane == 0) w.cnt[6] += 1;
       continue;
     }
     // 5. the ball: cavity slots first, then the extra slots
+#pragma unroll 1
     for (int i = lane; i < nb; i += 32) w.slot[i] = i < reuse ? w.cl[i] : w.ex[i - reuse];
     w.vkey[lane] = kNoVertex;
     if constexpr (!W::kTable) {
-      for (uint32_t i = lane; i < W::kEdgeN; i += 32) {
+      uint32_t en = 512;  // a power of two, at least 2.7 slots per edge (1.5 nb edges)
+      while (en < W::kEdgeN && en < 4u * (uint32_t)nb) en <<= 1;
+      if (lane == 0) w.emask = en - 1;
+#pragma unroll 1
+      for (uint32_t i = lane; i < en; i += 32) {
         w.ekey[i] = ~0ull;
         w.eval[i] = kNone;
       }
@@ -715,6 +795,7 @@ __device__ __forceinline__ int try_insert(const Ctx& c, W& w, uint32_t* lock, ui
     // the table path's vertex slots of this lane's facets (lane and lane + 32; nb <= 60), kept
     // for the partner lookups below
     uint32_t vs[2] = {0, 0};
+#pragma unroll 1
     for (int i = lane; i < nb; i += 32) {
       const int ci = w.bl_ci[i], f = w.bl_f[i] & 3;
       uint4 v = w.cr[ci].v;
@@ -736,15 +817,16 @@ __device__ __forceinline__ int try_insert(const Ctx& c, W& w, uint32_t* lock, ui
         for (int k = 0; k < 3; ++k) {
           const uint32_t x = get4(v, pos[(k + 1) % 3]), y = get4(v, pos[(k + 2) % 3]);
           const unsigned long long key = ((unsigned long long)min(x, y) << 32) | max(x, y);
-          uint32_t h = (uint32_t)((key * 0x9E3779B97F4A7C15ull) >> 40) & (W::kEdgeN - 1), sl = kNone;
+          const uint32_t em = w.emask;
+          uint32_t h = (uint32_t)((key * 0x9E3779B97F4A7C15ull) >> 40) & em, sl = kNone;
 #pragma unroll 1
-          for (uint32_t probe = 0; probe < W::kEdgeN; ++probe) {
+          for (uint32_t probe = 0; probe <= em; ++probe) {
             const unsigned long long old = atomicCAS(&w.ekey[h], ~0ull, key);
             if (old == ~0ull || old == key) {
               sl = h;
               break;
             }
-            h = (h + 1) & (W::kEdgeN - 1);
+            h = (h + 1) & em;
           }
           if (sl == kNone) {
             vfail = true;
@@ -759,6 +841,7 @@ __device__ __forceinline__ int try_insert(const Ctx& c, W& w, uint32_t* lock, ui
     // every internal facet was recorded by its two sides (the cavity was verified under the
     // locks, so its boundary is a closed surface); a lookup that finds no partner is a bug
     bool bad = __any_sync(kFull, vfail);
+#pragma unroll 1
     for (int i = lane; i < nb && !bad; i += 32) {
       const int ci = w.bl_ci[i], f = w.bl_f[i] & 3, back = w.bl_f[i] >> 2;
       uint4 v = w.cr[ci].v;
@@ -811,13 +894,14 @@ __device__ __forceinline__ int try_insert(const Ctx& c, W& w, uint32_t* lock, ui
     }
     if (__any_sync(kFull, bad)) {
       if (lane == 0) raise_error(c.st, kErrInternal, 0xA8u);
-      release_held(w, lock, held, nc, na, nx);
+      release_all(w, lock, held, heldx, nc, na, nx0);
       return kALost;
     }
     // cavity slots left over (|C| > |B|) die, keep a redirect into the ball, and join the pool
     const int freed = nc - nb;
     if (freed > 0) {
       const uint32_t redirect = w.slot[0];
+#pragma unroll 1
       for (int i = lane; i < freed; i += 32) {
         uint4* dst = reinterpret_cast<uint4*>(c.tets + w.cl[nb + i]);
         __stcg(dst, make_uint4(kDeadMark, kDeadMark, kDeadMark, kDeadMark));
@@ -825,7 +909,7 @@ __device__ __forceinline__ int try_insert(const Ctx& c, W& w, uint32_t* lock, ui
       }
     }
     __threadfence();
-    release_held(w, lock, held, nc, na, nx);
+    release_all(w, lock, held, heldx, nc, na, nx0);
     if (freed > 0) pool_give(c, w, w.cl + nb, freed);
     if (lane == 0) {
       const uint32_t s0 = w.slot[0];
@@ -840,10 +924,8 @@ __device__ __forceinline__ int try_insert(const Ctx& c, W& w, uint32_t* lock, ui
       log_outcome(lg, p, kCandInserted, nc);
       w.hint = s0;
       w.bn = W::kTable ? (nb < 32 ? nb : 32) : 0;
-      w.cnt[0] += 1;
-      w.cnt[3] += nc;
-      w.cnt[4] += nb;
     }
+    if (lane < 5) w.cnt[lane] += lane == 0 ? 1 : lane == 3 ? nc : lane == 4 ? nb : 0;
     __syncwarp();
     return kAInserted;
   }
@@ -860,45 +942,47 @@ __device__ __forceinline__ void to_queue(const AsyncIO& io, const Ctx& c, int q,
 }
 
 // A cavity too large for the warp's shared-memory workspace: the same insertion again in a
-// global-memory workspace borrowed from the launch's pool (tried at a few places, never waited
-// for). Returns kABig when the cavity exceeds it too, kALost when none is free. The borrowed workspace's
-// counters, spare slots and ball hint come back to the warp's own. Out of line: it runs for
-// about one point in 1500, and inlined it would double the kernel's instruction footprint.
-template <bool kExact, class W>
-__device__ __noinline__ int try_insert_large(const Ctx& c, const AsyncIO& io, W& w, uint32_t* lock, uint32_t me,
-                                             uint32_t p, const InsertLog& lg) {
-  if (!io.big_ws || io.big_n == 0) return kABig;
+// global-memory workspace (of type L) borrowed from the launch's pool (tried at a few places,
+// never waited for). Returns kABig when the cavity exceeds it too, kALost when none is free. The
+// borrowed workspace's counters, spare slots and ball hint come back to the warp's own. Out of
+// line: it runs for about one point in 1500, and inlined it would double the kernel's instruction
+// footprint.
+template <bool kExact, class L, class W>
+__device__ __noinline__ int try_insert_large(const Ctx& c, L* pool, unsigned int* busy, uint32_t n, W& w, uint32_t* lock,
+                                             uint32_t me, uint32_t p, const InsertLog& lg) {
+  if (!pool || n == 0) return kABig;
   const int lane = threadIdx.x & 31;
   int k = -1;
   if (lane == 0)
+#pragma unroll 1
     for (int t = 0; t < 8 && k < 0; ++t) {
-      const uint32_t cand = (me * 0x9E3779B1u + (uint32_t)t * 0x85EBCA6Bu) % io.big_n;
-      if (atomicCAS(&io.big_busy[cand], 0u, 1u) == 0u) k = (int)cand;
+      const uint32_t cand = (me * 0x9E3779B1u + (uint32_t)t * 0x85EBCA6Bu) % n;
+      if (atomicCAS(&busy[cand], 0u, 1u) == 0u) k = (int)cand;
     }
   k = __shfl_sync(kFull, k, 0);
   if (k < 0) return kALost;
-  LargeWST<W::kCache>& L = static_cast<LargeWST<W::kCache>*>(io.big_ws)[k];
+  L& b = pool[k];
   if (lane == 0) {
-    L.fa = w.fa;
-    L.bump = w.bump;
-    L.np = 0;
-    L.bn = 0;
-    L.hint = w.hint;
-    for (int q = 0; q < 8; ++q) L.cnt[q] = 0;
+    b.fa = w.fa;
+    b.bump = w.bump;
+    b.np = 0;
+    b.bn = 0;
+    b.hint = w.hint;
+    for (int q = 0; q < 8; ++q) b.cnt[q] = 0;
   }
   __syncwarp();
-  const int r = try_insert<kExact>(c, L, lock, me, p, lg, false, kNone);
-  pool_give(c, w, L.pool, L.np);
+  const int r = try_insert<kExact>(c, b, lock, p, lg, false, kNone);
+  pool_give(c, w, b.pool, b.np);
   if (lane == 0) {
-    w.cnt[0] += L.cnt[0];
-    w.cnt[3] += L.cnt[3];
-    w.cnt[4] += L.cnt[4];
-    w.cnt[5] += L.cnt[5];
-    w.cnt[6] += L.cnt[6];
-    if (r == kAInserted) w.hint = L.hint;
+    w.cnt[0] += b.cnt[0];
+    w.cnt[3] += b.cnt[3];
+    w.cnt[4] += b.cnt[4];
+    w.cnt[5] += b.cnt[5];
+    w.cnt[6] += b.cnt[6];
+    if (r == kAInserted) w.hint = b.hint;
     w.bn = 0;
     __threadfence();
-    atomicExch(&io.big_busy[k], 0u);
+    atomicExch(&busy[k], 0u);
   }
   __syncwarp();
   return r;
@@ -910,8 +994,7 @@ __device__ __noinline__ int try_insert_large(const Ctx& c, const AsyncIO& io, W&
 // and counters are flushed.
 template <bool kExact, class W>
 __device__ __forceinline__ void run_segment(const Ctx& c, const AsyncIO& io, W& w, uint32_t* lock, uint32_t me,
-                                            uint64_t b0, uint64_t e0, uint64_t k0, uint64_t k1, const uint8_t* vflag,
-                                            const InsertLog& lg) {
+                                            uint32_t b0, uint32_t e0, uint32_t k0, uint32_t k1, const InsertLog& lg) {
   const int lane = threadIdx.x & 31;
   if (lane == 0) {
     w.fa = __ldcg(&c.st->free_avail);
@@ -920,47 +1003,59 @@ __device__ __forceinline__ void run_segment(const Ctx& c, const AsyncIO& io, W& 
     w.bn = 0;
     for (int k = 0; k < 8; ++k) w.cnt[k] = 0;
     w.hint = kNone;
+    w.i = b0;
+    w.e0 = e0;
+    w.k0 = k0;
+    w.k1 = k1;
+    w.nd = w.dhead = w.since = w.tail = 0;
   }
-  __syncwarp();
-  int nd = 0, dhead = 0;
-  uint64_t i = b0;
-  int since = 0;  // insertions since the last retry of a deferred point
+#pragma unroll 1
   for (;;) {
-    __syncwarp();  // lane 0's writes to the deferred list are seen by every lane below
+    __syncwarp();  // lane 0's writes are seen by every lane below
+    const uint32_t i = w.i;
     uint32_t p, start = kNone;
     bool retried = false, follows = false;  // follows: the point after the last inserted one
-    if (nd > 0 && ((i >= e0 && k0 >= k1) || since >= 4)) {
-      p = w.defer[dhead];
-      dhead = (dhead + 1) % kADefer;
-      --nd;
+    if (w.nd > 0 && ((i >= w.e0 && w.k0 >= w.k1) || w.since >= 4)) {
+      p = w.defer[w.dhead];
       retried = true;
-      since = 0;
-    } else if (k0 < k1) {
-      p = io.carry[k0];
-      ++k0;
-    } else if (i < e0) {
-      p = io.q ? io.q[i] : io.qbase + (uint32_t)i;
+    } else if (w.k0 < w.k1) {
+      p = io.carry[w.k0];
+    } else if (i < w.e0) {
+      p = io.q[i];
       follows = i > b0;
       if (follows) start = w.hint;
-      ++i;
-      if (vflag[p] != 0) continue;
     } else {
       break;
     }
+    __syncwarp();
+    if (lane == 0) {
+      if (retried) {
+        w.dhead = (w.dhead + 1) % kADefer;
+        w.nd -= 1;
+        w.since = 0;
+      } else if (w.k0 < w.k1) {
+        w.k0 += 1;
+      } else {
+        w.i = i + 1;
+      }
+    }
+    if (p == kNone) continue;  // a duplicate or one of the first four
     if (lane == 0) w.cnt[2] += 1;
-    int r = try_insert<kExact>(c, w, lock, me, p, lg, follows && io.ball_start != 0, start);
+    int r = try_insert<kExact>(c, w, lock, p, lg, follows && io.ball_start != 0, start);
     if constexpr (W::kTable) {
-      if (r == kABig) r = try_insert_large<kExact>(c, io, w, lock, me, p, lg);
+      if (r == kABig)
+        r = try_insert_large<kExact>(c, static_cast<LargeWST<W::kCache>*>(io.big_ws), io.big_busy, io.big_n, w, lock, me, p,
+                                     lg);
     }
     // a raised error stops the launch; read every 16 points for the same reason as the anchor
     unsigned err = 0;
     if (lane == 0 && (w.cnt[2] & 15u) == 0) err = __ldcg(&c.st->error);
     if (__shfl_sync(kFull, err, 0) != 0u) break;
     if (r == kAInserted) {
-      ++since;
+      if (lane == 0) w.since += 1;
       continue;
     }
-    // every lane holds the same r, nd, dhead and `retried`: the decisions below are uniform
+    // every lane holds the same r and `retried` and reads the same nd: uniform decisions
     if (r == kALost && lane == 0) {
       w.cnt[1] += 1;
       log_outcome(lg, p, kCandLost, 0);
@@ -971,9 +1066,16 @@ __device__ __forceinline__ void run_segment(const Ctx& c, const AsyncIO& io, W& 
       if (lane == 0) to_queue(io, c, 1, p);
     } else if (r == kAExact) {
       if (lane == 0) to_queue(io, c, 2, p);
-    } else if (r == kALost && !retried && nd < kADefer) {
-      if (lane == 0) w.defer[(dhead + nd) % kADefer] = p;
-      ++nd;
+    } else if (r == kALost && w.nd < kADefer && (!retried || (i >= w.e0 && w.k0 >= w.k1 && w.tail < kATail))) {
+      // lost once: again after a few other insertions; at the segment's end, where the warps that
+      // it loses to are about done too, again and again (a bounded number of times)
+      __syncwarp();
+      if (lane == 0) {
+        w.defer[(w.dhead + w.nd) % kADefer] = p;
+        w.nd += 1;
+        w.tail += retried ? 1 : 0;
+      }
+      if (retried) __nanosleep(2000);
     } else {  // a walk over its step bound, or a point that lost again: the next pass
       if (lane == 0) to_queue(io, c, 0, p);
     }
@@ -981,12 +1083,14 @@ __device__ __forceinline__ void run_segment(const Ctx& c, const AsyncIO& io, W& 
   __syncwarp();
   // what is left: deferred points to the next pass, unused slots back to the allocator
   if (lane == 0)
-    for (int k = 0; k < nd; ++k) to_queue(io, c, 0, w.defer[(dhead + k) % kADefer]);
+#pragma unroll 1
+    for (int k = 0; k < w.nd; ++k) to_queue(io, c, 0, w.defer[(w.dhead + k) % kADefer]);
   const int np = w.np;
   if (np > 0) {
     unsigned long long pb = 0;
     if (lane == 0) pb = atomicAdd(&c.st->pending, (unsigned long long)np);
     pb = __shfl_sync(kFull, pb, 0);
+#pragma unroll 1
     for (int k = lane; k < np; k += 32) {
       if (pb + k < c.st->free_capacity) c.pending[pb + k] = w.pool[k];
       else raise_error(c.st, kErrFreeList, 0xA9u);
@@ -996,14 +1100,14 @@ __device__ __forceinline__ void run_segment(const Ctx& c, const AsyncIO& io, W& 
     unsigned long long* dst[8] = {&c.st->n_inserted, &c.st->n_conflicts, &c.st->n_attempts, &c.st->sum_cavity,
                                   &c.st->sum_ball, &c.st->sum_walk, &c.st->n_restart, &c.st->n_inserted_async};
     w.cnt[7] = w.cnt[0];
+#pragma unroll 1
     for (int k = 0; k < 8; ++k)
       if (w.cnt[k]) atomicAdd(dst[k], (unsigned long long)w.cnt[k]);
   }
 }
 
 template <int kMinBlocks, bool kCache = false, bool kExact = false>
-__global__ void __launch_bounds__(kAW * 32, kMinBlocks) k_async(Ctx c, AsyncIO io, uint32_t* lock,
-                                                               const uint8_t* __restrict__ vflag, InsertLog lg) {
+__global__ void __launch_bounds__(kAW * 32, kMinBlocks) k_async(Ctx c, AsyncIO io, uint32_t* lock, InsertLog lg) {
   __shared__ SmallWST<kCache> s_ws[kAW];
   const int wid = threadIdx.x >> 5;
   const uint32_t seg = blockIdx.x * kAW + wid;
@@ -1015,20 +1119,21 @@ __global__ void __launch_bounds__(kAW * 32, kMinBlocks) k_async(Ctx c, AsyncIO i
   } else {
     b0 = (uint64_t)seg * io.L;
     e0 = b0 + io.L < io.m ? b0 + io.L : io.m;
+    if (b0 > e0) b0 = e0;
   }
-  run_segment<kExact>(c, io, s_ws[wid], lock, seg + 1, b0, e0, io.carry_n * seg / io.W, io.carry_n * (seg + 1) / io.W, vflag,
-                      lg);
+  run_segment<kExact>(c, io, s_ws[wid], lock, seg + 1, (uint32_t)b0, (uint32_t)e0, (uint32_t)(io.carry_n * seg / io.W),
+                      (uint32_t)(io.carry_n * (seg + 1) / io.W), lg);
 }
 
 // Large cavities (beyond the shared-memory workspaces): the same insertion with each warp's
-// workspace in global memory. Owner words are per warp of the launch, and this kernel never
-// runs beside k_async, so warp numbers may repeat across the two.
+// workspace in global memory.
 template <bool kCache, bool kExact>
-__global__ void __launch_bounds__(128) k_async_big(Ctx c, AsyncIO io, uint32_t* lock, const uint8_t* __restrict__ vflag,
-                                                  InsertLog lg, HugeWST<kCache>* ws) {
+__global__ void __launch_bounds__(128) k_async_big(Ctx c, AsyncIO io, uint32_t* lock, InsertLog lg,
+                                                  HugeWST<kCache>* ws) {
   const uint32_t seg = blockIdx.x * 4 + (threadIdx.x >> 5);
   if (seg >= io.W) return;
-  run_segment<kExact>(c, io, ws[seg], lock, seg + 1, 0, 0, io.carry_n * seg / io.W, io.carry_n * (seg + 1) / io.W, vflag, lg);
+  run_segment<kExact>(c, io, ws[seg], lock, seg + 1, 0, 0, (uint32_t)(io.carry_n * seg / io.W),
+                      (uint32_t)(io.carry_n * (seg + 1) / io.W), lg);
 }
 
 // Folds the allocator of the launch into the free list, as a round close does
@@ -1080,17 +1185,16 @@ bool async_six_blocks() {
 
 }  // namespace
 
-int async_launch(const Ctx& c, const AsyncIO& io, uint32_t* lock, const uint8_t* vflag, const InsertLog& lg,
-                 cudaStream_t s) {
+int async_launch(const Ctx& c, const AsyncIO& io, uint32_t* lock, const InsertLog& lg, cudaStream_t s) {
   if (io.W == 0 || (io.m == 0 && io.carry_n == 0)) return DT_OK;
   Ctx cc = c;
   cc.coherent = 1;
   cc.max_walk = io.max_walk;
   const unsigned blocks = (io.W + kAW - 1) / kAW;
-  if (io.exact) k_async<kExactBlocks, false, true><<<blocks, kAW * 32, 0, s>>>(cc, io, lock, vflag, lg);
-  else if (c.subdet) k_async<8, true><<<blocks, kAW * 32, 0, s>>>(cc, io, lock, vflag, lg);
-  else if (async_six_blocks()) k_async<6><<<blocks, kAW * 32, 0, s>>>(cc, io, lock, vflag, lg);
-  else k_async<8><<<blocks, kAW * 32, 0, s>>>(cc, io, lock, vflag, lg);
+  if (io.exact) k_async<kExactBlocks, false, true><<<blocks, kAW * 32, 0, s>>>(cc, io, lock, lg);
+  else if (c.subdet) k_async<8, true><<<blocks, kAW * 32, 0, s>>>(cc, io, lock, lg);
+  else if (async_six_blocks()) k_async<6><<<blocks, kAW * 32, 0, s>>>(cc, io, lock, lg);
+  else k_async<8><<<blocks, kAW * 32, 0, s>>>(cc, io, lock, lg);
   k_async_close_copy<<<152, 256, 0, s>>>(cc);
   k_async_close_state<<<1, 1, 0, s>>>(cc, io.carry_n ? io.carry_q : -1);
   g_kernel_launches += 3;
@@ -1100,15 +1204,14 @@ int async_launch(const Ctx& c, const AsyncIO& io, uint32_t* lock, const uint8_t*
 size_t async_borrow_ws_bytes() { return sizeof(LargeWS); }
 size_t async_big_ws_bytes() { return sizeof(HugeWST<false>); }
 
-int async_launch_big(const Ctx& c, const AsyncIO& io, uint32_t* lock, const uint8_t* vflag, const InsertLog& lg,
-                     void* ws, cudaStream_t s) {
+int async_launch_big(const Ctx& c, const AsyncIO& io, uint32_t* lock, const InsertLog& lg, void* ws, cudaStream_t s) {
   if (io.W == 0 || io.carry_n == 0) return DT_OK;
   Ctx cc = c;
   cc.coherent = 1;
   cc.max_walk = io.max_walk;
   HugeWST<false>* w = static_cast<HugeWST<false>*>(ws);
-  if (io.exact) k_async_big<false, true><<<(io.W + 3) / 4, 128, 0, s>>>(cc, io, lock, vflag, lg, w);
-  else k_async_big<false, false><<<(io.W + 3) / 4, 128, 0, s>>>(cc, io, lock, vflag, lg, w);
+  if (io.exact) k_async_big<false, true><<<(io.W + 3) / 4, 128, 0, s>>>(cc, io, lock, lg, w);
+  else k_async_big<false, false><<<(io.W + 3) / 4, 128, 0, s>>>(cc, io, lock, lg, w);
   k_async_close_copy<<<152, 256, 0, s>>>(cc);
   k_async_close_state<<<1, 1, 0, s>>>(cc, io.carry_q);
   g_kernel_launches += 3;

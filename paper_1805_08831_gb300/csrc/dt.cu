@@ -22,7 +22,9 @@ constexpr int kCavWarps = 4;  // candidates per block of the cavity kernel (4 me
 constexpr int kInsWarps = 8;  // candidates per block of the ball kernel
 constexpr uint32_t kDefaultWalk = 48;          // walk steps per pass (a longer walk resumes next pass)
 constexpr uint32_t kAsyncWalk = 4096;          // walk steps per attempt of the asynchronous engine
-constexpr uint32_t kAsyncBigWarps = 64;        // warps (global-memory workspaces) of its large-cavity kernel
+constexpr uint32_t kAsyncBigWarps = 64;        // warps (workspaces) of a large-cavity launch
+constexpr double kSmallMeshWarps = 240;        // warps up to which a small mesh gets more than alpha allows
+constexpr uint64_t kDrainPoints = 8;           // points per warp of a list without a wave
 constexpr uint32_t kAsyncBorrow = 512;         // large-cavity workspaces the main kernel's warps may borrow
 constexpr uint64_t kLongWalkBelow = 8192;      // retry lists shorter than this walk up to
 constexpr uint32_t kLongWalkSteps = 1u << 14;  // this many steps per pass
@@ -529,7 +531,7 @@ __global__ void __launch_bounds__(kCtaWarps * 32) k_cta_insert(Ctx c, const uint
 __global__ void k_wave_keys(uint32_t vbegin, uint64_t m, uint64_t base, uint64_t rank0,
                             const uint32_t* __restrict__ perm, const uint32_t* __restrict__ rank,
                             const uint32_t* __restrict__ cum, int nwaves, const uint8_t* __restrict__ risky,
-                            uint64_t* keys, uint32_t* vals) {
+                            const uint8_t* __restrict__ skip, uint64_t* keys, uint32_t* vals) {
   for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < m;
        i += (uint64_t)gridDim.x * blockDim.x) {
     uint32_t v = vbegin + (uint32_t)i;
@@ -542,7 +544,7 @@ __global__ void k_wave_keys(uint32_t vbegin, uint64_t m, uint64_t base, uint64_t
     }
     // with the learned schedule, the points expected to lose go after the rest of their wave
     keys[i] = risky ? 2 * (uint64_t)lo + risky[v] : (uint64_t)lo;
-    vals[i] = v;
+    vals[i] = skip && skip[v] ? kNone : v;  // the asynchronous engine's lists leave flagged points out
   }
 }
 
@@ -816,18 +818,20 @@ __global__ void k_work(const float* __restrict__ pred, uint64_t n, uint32_t vb, 
   }
 }
 
-__global__ void k_seg_cost(const uint32_t* __restrict__ q, uint32_t qbase, uint64_t m, const uint8_t* __restrict__ wcost,
-                           uint32_t* out) {
+__device__ __forceinline__ uint32_t list_cost(const uint8_t* __restrict__ wcost, uint32_t v) {
+  return v == kNone ? 0u : wcost[v];
+}
+__global__ void k_seg_cost(const uint32_t* __restrict__ q, uint64_t m, const uint8_t* __restrict__ wcost, uint32_t* out) {
   for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < m; i += (uint64_t)gridDim.x * blockDim.x)
-    out[i] = wcost[q ? q[i] : qbase + (uint32_t)i];
+    out[i] = list_cost(wcost, q[i]);
 }
 
 // bounds[w] = the first list position whose exclusive prefix of work reaches w / W of the total.
-__global__ void k_seg_bounds(const uint32_t* __restrict__ prefix, const uint32_t* __restrict__ q, uint32_t qbase,
-                             uint64_t m, const uint8_t* __restrict__ wcost, uint32_t W, uint32_t* bounds) {
+__global__ void k_seg_bounds(const uint32_t* __restrict__ prefix, const uint32_t* __restrict__ q, uint64_t m,
+                             const uint8_t* __restrict__ wcost, uint32_t W, uint32_t* bounds) {
   const uint32_t w = blockIdx.x * blockDim.x + threadIdx.x;
   if (w > W) return;
-  const uint64_t total = (uint64_t)prefix[m - 1] + wcost[q ? q[m - 1] : qbase + (uint32_t)(m - 1)];
+  const uint64_t total = (uint64_t)prefix[m - 1] + list_cost(wcost, q[m - 1]);
   const uint64_t target = total * w / W;
   uint64_t lo = 0, hi = m;  // first i in [0, m] with prefix[i] >= target (prefix[m] = total)
   while (lo < hi) {
@@ -1083,7 +1087,7 @@ uint64_t device_bytes(const dt_handle* h) {
   }
   b += h->cap_q * 4 * kNumQueues + h->cap_w * 4;
   if (h->async_big_ws) b += (uint64_t)kAsyncBigWarps * async_big_ws_bytes();
-  if (h->async_borrow_ws) b += (uint64_t)kAsyncBorrow * (async_big_ws_bytes() + 4);
+  if (h->async_borrow_ws) b += (uint64_t)kAsyncBorrow * (async_borrow_ws_bytes() + 4);
   if (h->hugemem) b += carve(nullptr, 4 * h->huge_c, h->huge_c, h->huge_c, 4 * h->huge_c, nullptr);
   b += h->cap_log * 3 + h->cap_feat * (8 + 2) * 4 + h->cap_risky * 2 + h->cap_cells * 4;
   b += h->cap_bpts * 32 + h->cap_bws + h->cap_bstates * sizeof(DevState);
@@ -1113,9 +1117,19 @@ int reserve_points(dt_handle* h, uint64_t total) {
   return DT_OK;
 }
 
+// Warps of an asynchronous launch on a mesh: alpha per vertex, up to 2.4 times that while the mesh
+// is so small that a launch is a chain of insertions on a mostly empty chip (2047 points: 5.5 ms
+// at 0.05, 4.5 ms at 0.12; at 1e5 points and more 0.05 is the faster one).
+uint64_t async_warps_for(const dt_handle* h, uint64_t mesh) {
+  const double a = h->alpha_async * (double)mesh;
+  const uint64_t W = (uint64_t)std::max(1.0, std::max(a, std::min(2.4 * a, kSmallMeshWarps)));
+  return std::min<uint64_t>(W, h->async_warps ? h->async_warps : (uint64_t)async_max_warps());
+}
+
 int reserve_tets(dt_handle* h, uint64_t total_pts) {
   double f = h->cfg.tet_capacity_factor > 0 ? h->cfg.tet_capacity_factor : 8.0;
-  uint64_t need = (uint64_t)(f * (double)total_pts) + 4096;
+  // every warp of an asynchronous launch keeps a few dozen slots of its own while it runs
+  uint64_t need = (uint64_t)(f * (double)total_pts) + 4096 + 64 * async_warps_for(h, total_pts);
   if (need > kMaxSlots) need = kMaxSlots;
   // after a batch the store may be large enough while it has no owner words and a shorter free
   // list than this engine's
@@ -1369,7 +1383,7 @@ int run_big_async(dt_handle* h, const Ctx& c, bool exact) {
     io.exact_out = h->queue[kQExact];
     io.exact_q = kQExact;
     io.exact = exact;
-    if ((rc = async_launch_big(c, io, h->lock, h->vflag, make_log(h), h->async_big_ws, h->stream)) != DT_OK)
+    if ((rc = async_launch_big(c, io, h->lock, make_log(h), h->async_big_ws, h->stream)) != DT_OK)
       return rc;
     h->stats.n_async++;
     if ((rc = sync_state(h)) != DT_OK) return rc;
@@ -1400,8 +1414,8 @@ int run_pass(dt_handle* h, const Ctx& c, const uint32_t* q, uint32_t qbase, uint
 int run_pass_async(dt_handle* h, const Ctx& c, const uint32_t* q, uint64_t m, const uint32_t* carry, uint64_t carry_n,
                    int carry_q, int out, bool exact) {
   const uint64_t mesh = h->st_host->n_inserted;
-  uint64_t W = (uint64_t)std::max(1.0, h->alpha_async * (double)mesh);
-  W = std::min<uint64_t>(W, h->async_warps ? h->async_warps : (uint64_t)async_max_warps());
+  uint64_t W = async_warps_for(h, mesh);
+  if (m == 0) W = std::min<uint64_t>(W, (carry_n + kDrainPoints - 1) / kDrainPoints);
   if (exact) W = std::min<uint64_t>(W, (uint64_t)async_max_warps_exact());
   W = std::min<uint64_t>(W, std::max(m, carry_n));
   const uint64_t L = (m + W - 1) / W;
@@ -1418,9 +1432,9 @@ int run_pass_async(dt_handle* h, const Ctx& c, const uint32_t* q, uint64_t m, co
     }
     if (!h->seg_bounds && cudaMalloc(&h->seg_bounds, ((size_t)async_max_warps() + 1) * 4) != cudaSuccess)
       return DT_ENOMEM;
-    k_seg_cost<<<grid_for(m, 256), 256, 0, h->stream>>>(q, 0, m, h->wcost, h->seg_prefix);
+    k_seg_cost<<<grid_for(m, 256), 256, 0, h->stream>>>(q, m, h->wcost, h->seg_prefix);
     prefix_sum_exclusive(h->seg_prefix, m, h->ows.hist, h->stream);
-    k_seg_bounds<<<grid_for(W + 1, 256), 256, 0, h->stream>>>(h->seg_prefix, q, 0, m, h->wcost, (uint32_t)W,
+    k_seg_bounds<<<grid_for(W + 1, 256), 256, 0, h->stream>>>(h->seg_prefix, q, m, h->wcost, (uint32_t)W,
                                                                h->seg_bounds);
     g_kernel_launches += 2;
     seg_bounds = h->seg_bounds;
@@ -1431,12 +1445,12 @@ int run_pass_async(dt_handle* h, const Ctx& c, const uint32_t* q, uint64_t m, co
       return DT_ENOMEM;
     cudaMemsetAsync(h->async_borrow_busy, 0, kAsyncBorrow * sizeof(unsigned int), h->stream);
   }
-  AsyncIO io{q, 0, m, L, (uint32_t)W, h->cfg.max_walk_steps ? h->cfg.max_walk_steps : kAsyncWalk,
+  AsyncIO io{q, m, L, (uint32_t)W, h->cfg.max_walk_steps ? h->cfg.max_walk_steps : kAsyncWalk,
              carry, carry_n, carry_q, h->queue[out], out, h->queue[kQBig], kQBig, h->queue[kQExact], kQExact,
              exact ? 1 : 0, seg_bounds, h->async_borrow_ws, h->async_borrow_busy, kAsyncBorrow, h->async_ball_start};
   const bool prof = (h->cfg.flags & DT_FLAG_PROFILE) != 0;
   if (prof) cudaEventRecord(h->ev[3], h->stream);
-  if ((rc = async_launch(c, io, h->lock, h->vflag, make_log(h), h->stream)) != DT_OK) return rc;
+  if ((rc = async_launch(c, io, h->lock, make_log(h), h->stream)) != DT_OK) return rc;
   if (prof) cudaEventRecord(h->ev[4], h->stream);
   h->stats.n_async++;
   h->stats.n_passes++;
@@ -1515,7 +1529,8 @@ int make_waves(dt_handle* h, uint32_t vbegin, uint32_t vend, int round, uint64_t
   // lose (inserted with less concurrency)
   const bool split = scale && h->risky_ready;
   k_wave_keys<<<grid_for(m, 256), 256, 0, s>>>(vbegin, m, base, rank0, h->ows.perm, h->ows.rank, h->wave_cum,
-                                                (int)cum.size(), split ? h->risky : nullptr, h->ows.k0, h->ows.v0);
+                                                (int)cum.size(), split ? h->risky : nullptr, h->use_async ? h->vflag : nullptr, h->ows.k0,
+                                                h->ows.v0);
   ++g_kernel_launches;
   if (split) {
     const int nk = 2 * (int)cum.size();
@@ -1679,17 +1694,15 @@ int insert_async(dt_handle* h, uint64_t base, uint64_t n, bool exact) {
     }
     const uint64_t nq = h->st_host->q[cur], limited = h->st_host->n_walk_limit;
     if (nq == 0) return DT_OK;
-    // a list of more points than warps is put into the order of a transformed curve (Section
-    // 3.3), so that the points of a neighbourhood meet in one warp and not in several; the top 24
-    // bits of the 63-bit key (8 levels of the curve) order them well enough
+    // the points left come in clumps that lost to one another: in the order of a transformed curve
+    // (Section 3.3) those of a neighbourhood meet in one warp, which inserts them one after the
+    // other. (A warp each took 34 launches for the last 2900 points of 1e6: 291 of 1503 got in.) The
+    // top 24 bits of the 63-bit key (8 levels of the curve) order them well enough
     const bool rounds = stalled > 0 || nq < h->async_min_retry;
-    const uint32_t* list = h->queue[cur];
-    if (rounds || nq > (uint64_t)(h->alpha_async * (double)h->st_host->n_inserted)) {
-      transformed_keys(h->pts, list, nq, h->bbox_dev, h->cfg.seed + 0x51ED2701ull * (pass + 1) + base, h->ows.k0,
-                       h->ows.v0, s);
-      const bool a2 = radix_sort_pairs_bits(h->ows.k0, h->ows.v0, h->ows.k1, h->ows.v1, nq, 39, 63, h->ows.hist, s);
-      list = a2 ? h->ows.v1 : h->ows.v0;
-    }
+    transformed_keys(h->pts, h->queue[cur], nq, h->bbox_dev, h->cfg.seed + 0x51ED2701ull * (pass + 1) + base, h->ows.k0,
+                     h->ows.v0, s);
+    const bool a2 = radix_sort_pairs_bits(h->ows.k0, h->ows.v0, h->ows.k1, h->ows.v1, nq, 39, 63, h->ows.hist, s);
+    const uint32_t* list = a2 ? h->ows.v1 : h->ows.v0;
     if (rounds) {
       // after a pass that made no progress the round-based engine takes over: its highest-priority
       // located point always wins, where the asynchronous engine's retries might keep colliding

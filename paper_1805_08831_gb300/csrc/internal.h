@@ -130,14 +130,12 @@ void transformed_keys(const Pt* pts, const uint32_t* ids, uint64_t m, const doub
 // ---------------------------------------------------------------- async.cu (one launch per pass)
 struct Ctx;
 struct InsertLog;
-// Points q[0, m) (or the vertex range qbase + [0, m) when q is null) in W contiguous segments
-// of L points, segment w inserted by warp w in order, after the warp's share of the carry_n
+// Points q[0, m) (kNone: skipped) in W contiguous segments of L points, segment w inserted by warp w in order, after the warp's share of the carry_n
 // points carried over from earlier launches (carry; queue carry_q, emptied by the launch, when it
 // is not negative). Points that lose or walk past max_walk steps go to lose_out (queue lose_q),
 // cavities too large for a warp's workspaces to big_out.
 struct AsyncIO {
   const uint32_t* q;
-  uint32_t qbase;
   uint64_t m, L;
   uint32_t W;
   uint32_t max_walk;
@@ -159,8 +157,7 @@ struct AsyncIO {
 };
 // Enqueues the asynchronous insertion of one pass and the close of its allocator. lock: one
 // word per tetrahedron slot, all zero before and after.
-int async_launch(const Ctx& c, const AsyncIO& io, uint32_t* lock, const uint8_t* vflag, const InsertLog& lg,
-                 cudaStream_t s);
+int async_launch(const Ctx& c, const AsyncIO& io, uint32_t* lock, const InsertLog& lg, cudaStream_t s);
 // Warps of the asynchronous kernels (FP32 alone; with the exact stages) that can be resident on
 // the current device at once.
 int async_max_warps();
@@ -170,8 +167,7 @@ size_t async_borrow_ws_bytes();  // one workspace of AsyncIO::big_ws
 // one global-memory workspace of async_big_ws_bytes() each at ws (device). Points whose cavities
 // exceed even these go to io.big_out.
 size_t async_big_ws_bytes();
-int async_launch_big(const Ctx& c, const AsyncIO& io, uint32_t* lock, const uint8_t* vflag, const InsertLog& lg,
-                     void* ws, cudaStream_t s);
+int async_launch_big(const Ctx& c, const AsyncIO& io, uint32_t* lock, const InsertLog& lg, void* ws, cudaStream_t s);
 
 // ---------------------------------------------------------------- batch.cu (dt_batch)
 size_t batch_ws_stride();       // bytes of one warp's workspace
