@@ -75,7 +75,7 @@ typedef struct {
   uint64_t n_dups;        /* exact duplicates not inserted */
   uint64_t n_tets;        /* finite tetrahedra in the current triangulation */
   uint64_t n_slots;       /* tetrahedron slots in use (finite + ghost + free) */
-  uint64_t n_rounds;      /* concurrent insertion rounds launched */
+  uint64_t n_rounds;      /* concurrent insertion rounds launched (dt_batch: its launches) */
   uint64_t n_passes;      /* re-partition passes (Section 3.3) */
   uint64_t n_attempts;    /* insertion attempts (successes + retries) */
   uint64_t n_conflicts;   /* attempts lost to a higher-priority cavity */
@@ -101,9 +101,9 @@ typedef struct {
   uint64_t free_slots;     /* slots on the free list after the last round */
   uint64_t max_walk;       /* longest single walk (steps) */
   uint64_t n_clouds_degenerate; /* dt_batch: clouds with fewer than four non-coplanar points */
-  uint64_t batch_warps;    /* dt_batch: block shape used (warps per block, autotuned) */
-  double batch_alpha;      /* dt_batch: concurrent insertions per mesh vertex used (autotuned) */
-  double ms_batch_tune;    /* dt_batch: host time of the autotuning in the last call (0 = reused) */
+  uint64_t batch_warps;    /* dt_batch: block shape used (warps per block) */
+  double batch_alpha;      /* dt_batch: most concurrent insertions per mesh vertex */
+  double ms_batch_tune;    /* dt_batch: 0 (nothing is tuned by timing) */
   uint64_t batch_graph;    /* dt_batch: 1 if the last call replayed its captured CUDA graph */
   uint64_t batch_min_blocks; /* dt_batch: resident blocks per SM the chosen shape was built for */
   double ms_async;         /* summed device time of the asynchronous insertion launches
@@ -112,8 +112,8 @@ typedef struct {
   uint64_t n_restarts;     /* asynchronous insertions that found their cavity changed under the
                               locks and started over */
   uint64_t device_bytes;   /* device memory the handle holds */
-  uint64_t n_exact_handoff; /* points the asynchronous engine handed to the round-based engine
-                               because its FP32 predicate stage could not decide a test */
+  uint64_t n_exact_handoff; /* points the asynchronous engine's FP32 kernel handed to its exact
+                               kernel because its predicate stage could not decide a test */
   uint64_t n_inserted_async; /* insertions made by the asynchronous engine */
   uint64_t reserved[2];
 } dt_stats;
@@ -139,12 +139,11 @@ int dt_insert(dt_handle* h, const double* xyz_dev, uint64_t n);
 int dt_insert_host(dt_handle* h, const double* xyz_host, uint64_t n);
 
 /* Triangulates n_clouds independent clouds: one batched sort (each cloud gets its own box,
- * Moore keys, duplicates and BRIO rounds, exactly as dt_insert would give it alone), then ONE
- * persistent kernel launch in which every thread block takes whole clouds from a device work
- * counter (largest first) and runs Algorithm 1 for all of a cloud's points with its warps
- * inserting concurrently (the Section 3.2 conflict rules between them). The block shape (warps
- * per block) and the round size are chosen by an autotuner that times candidates on a sample of
- * the clouds the first time a batch of this kind (cloud count, size range) is seen.
+ * Moore keys, duplicates and BRIO rounds, exactly as dt_insert would give it alone), then one
+ * fixed sequence of launches of the asynchronous engine over all clouds at once, replayed from a
+ * CUDA graph when a batch of the same shape follows: launch k inserts the k-th wave of every cloud
+ * that has one, with as many warps per cloud as its mesh carries (fewer when many clouds fill the
+ * device); no parameter is tuned by timing.
  *  - xyz_dev: the clouds back to back, [sum n_i, 3] float64 (device);
  *  - offsets_host: n_clouds + 1 ascending entries (host), offsets_host[0] = 0; cloud c is rows
  *    offsets_host[c] .. offsets_host[c + 1].

@@ -23,6 +23,7 @@ constexpr int kInsWarps = 8;  // candidates per block of the ball kernel
 constexpr uint32_t kDefaultWalk = 48;          // walk steps per pass (a longer walk resumes next pass)
 constexpr uint32_t kAsyncWalk = 4096;          // walk steps per attempt of the asynchronous engine
 constexpr uint32_t kAsyncBigWarps = 64;        // warps (workspaces) of a large-cavity launch
+constexpr uint32_t kBatchBigWarps = 16;        // warps (workspaces) of a batch's largest cavities
 constexpr double kSmallMeshWarps = 240;        // warps up to which a small mesh gets more than alpha allows
 constexpr uint64_t kDrainPoints = 8;           // points per warp of a list without a wave
 constexpr uint32_t kAsyncBorrow = 512;         // large-cavity workspaces the main kernel's warps may borrow
@@ -965,8 +966,6 @@ struct dt_handle {
   std::vector<BatchCloud> bclouds_host;    // per-cloud ranges and results
   uint64_t* boff_dev = nullptr;
   BatchCloud* bclouds = nullptr;
-  uint32_t* border = nullptr;               // clouds by decreasing size
-  uint32_t* bsample = nullptr;              // the autotuner's sample of clouds
   uint64_t cap_bclouds = 0;
   uint32_t* bcid = nullptr;
   uint8_t* bdup = nullptr;                  // duplicate flags by vertex (sorted position)
@@ -974,22 +973,21 @@ struct dt_handle {
   uint64_t cap_bpts = 0;
   uint32_t *bhint_f = nullptr, *bhint_c = nullptr;
   double* bcbox = nullptr;
-  DevState* bstates = nullptr;
-  uint64_t cap_bstates = 0;
-  char* bws = nullptr;
-  size_t cap_bws = 0;
-  unsigned long long* bstats = nullptr;
-  unsigned int* bnext = nullptr;
-  int batch_W = 0;                          // autotuned block shape (warps per block), 0 = not tuned
-  float batch_alpha = 0.f;                  // autotuned concurrent insertions per mesh vertex
-  uint64_t batch_sig = 0;                   // workload signature the tuning belongs to
-  double batch_tune_ms = 0.0;
+  DevState* bstates = nullptr;              // one per cloud
+  char* bws = nullptr;                      // workspaces for cavities beyond the borrowed ones
+  unsigned long long* bstats = nullptr;     // kBatchTotals
+  uint4* bsegs = nullptr;                   // every launch's segments
+  uint64_t cap_bsegs = 0;
+  std::vector<uint64_t> bplan_key;          // cloud sizes and parameters the segments were made for
+  std::vector<std::pair<uint64_t, uint64_t>> bplan;  // each launch's segments: first and number
   float* beta = nullptr;                    // device: the batch's FP32 error term
   cudaStream_t bs = nullptr;                // the handle's own stream for batches (capturable)
   cudaEvent_t bev[4] = {nullptr, nullptr, nullptr, nullptr};
   cudaGraph_t bgraph = nullptr;             // the captured steady-state batch
   cudaGraphExec_t bexec = nullptr;
   std::vector<uint64_t> bgraph_key;         // what the captured graph was made for
+  std::vector<uint64_t> bseen_key;          // the last batch's
+  int bgraph_src = 0;                       // the list its last launch leaves points in
   uint64_t bgraph_kernels = 0;              // kernels in the captured graph
   bool bgraph_used = false;                 // the last batch replayed the graph
   // learned scheduler
@@ -1055,6 +1053,7 @@ Ctx make_ctx(dt_handle* h) {
   // stopped, so one long walk does not hold up a whole round
   c.max_walk = h->cfg.max_walk_steps ? h->cfg.max_walk_steps : kDefaultWalk;
   c.coherent = 0;
+  c.tbase = 0;
   c.ntets = (uint32_t)h->cap_tets;
   c.npts = (uint32_t)h->cap_pts;
   c.subdet = h->use_subdet ? h->subdet : nullptr;
@@ -1090,7 +1089,8 @@ uint64_t device_bytes(const dt_handle* h) {
   if (h->async_borrow_ws) b += (uint64_t)kAsyncBorrow * (async_borrow_ws_bytes() + 4);
   if (h->hugemem) b += carve(nullptr, 4 * h->huge_c, h->huge_c, h->huge_c, 4 * h->huge_c, nullptr);
   b += h->cap_log * 3 + h->cap_feat * (8 + 2) * 4 + h->cap_risky * 2 + h->cap_cells * 4;
-  b += h->cap_bpts * 32 + h->cap_bws + h->cap_bstates * sizeof(DevState);
+  b += h->cap_bpts * 32 + h->cap_bclouds * sizeof(DevState) + h->cap_bsegs * sizeof(uint4);
+  if (h->bws) b += (uint64_t)kBatchBigWarps * batch_big_ws_bytes();
   return b;
 }
 
@@ -1174,6 +1174,15 @@ int reserve_tets(dt_handle* h, uint64_t total_pts) {
   cudaMemcpyAsync(&h->st->free_capacity, &vals[1], 8, cudaMemcpyHostToDevice, h->stream);
   cudaStreamSynchronize(h->stream);
   return DT_OK;
+}
+
+// The large-cavity workspaces that the asynchronous kernels' warps borrow.
+int reserve_borrow(dt_handle* h) {
+  if (h->async_borrow_ws) return DT_OK;
+  if (cudaMalloc(&h->async_borrow_busy, kAsyncBorrow * sizeof(unsigned int)) != cudaSuccess) return DT_ENOMEM;
+  cudaMemsetAsync(h->async_borrow_busy, 0, kAsyncBorrow * sizeof(unsigned int), h->stream);
+  return cudaMalloc(&h->async_borrow_ws, (size_t)kAsyncBorrow * async_borrow_ws_bytes()) == cudaSuccess ? DT_OK
+                                                                                                        : DT_ENOMEM;
 }
 
 // The serial path's workspace: cavities of a quarter of the tetrahedron store, between kHugeC
@@ -1439,13 +1448,8 @@ int run_pass_async(dt_handle* h, const Ctx& c, const uint32_t* q, uint64_t m, co
     g_kernel_launches += 2;
     seg_bounds = h->seg_bounds;
   }
-  if (!h->async_borrow_ws) {
-    if (cudaMalloc(&h->async_borrow_ws, (size_t)kAsyncBorrow * async_borrow_ws_bytes()) != cudaSuccess ||
-        cudaMalloc(&h->async_borrow_busy, kAsyncBorrow * sizeof(unsigned int)) != cudaSuccess)
-      return DT_ENOMEM;
-    cudaMemsetAsync(h->async_borrow_busy, 0, kAsyncBorrow * sizeof(unsigned int), h->stream);
-  }
-  AsyncIO io{q, m, L, (uint32_t)W, h->cfg.max_walk_steps ? h->cfg.max_walk_steps : kAsyncWalk,
+  if ((rc = reserve_borrow(h)) != DT_OK) return rc;
+  AsyncIO io{q, nullptr, m, L, (uint32_t)W, h->cfg.max_walk_steps ? h->cfg.max_walk_steps : kAsyncWalk,
              carry, carry_n, carry_q, h->queue[out], out, h->queue[kQBig], kQBig, h->queue[kQExact], kQExact,
              exact ? 1 : 0, seg_bounds, h->async_borrow_ws, h->async_borrow_busy, kAsyncBorrow, h->async_ball_start};
   const bool prof = (h->cfg.flags & DT_FLAG_PROFILE) != 0;
@@ -1854,13 +1858,6 @@ bool realloc_dev(T*& p, uint64_t n) {
   return cudaMalloc(&p, std::max<uint64_t>(n, 1) * sizeof(T)) == cudaSuccess;
 }
 
-int sm_count() {
-  int dev = 0, n = 0;
-  cudaGetDevice(&dev);
-  if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) n = 152;
-  return n;
-}
-
 // Device memory of a batch of nc clouds, N points and T tetrahedron slots (in total).
 int batch_reserve(dt_handle* h, uint64_t N, uint32_t nc, uint64_t T) {
   if (reserve_points(h, N) != DT_OK) return DT_ENOMEM;
@@ -1872,50 +1869,45 @@ int batch_reserve(dt_handle* h, uint64_t N, uint32_t nc, uint64_t T) {
     h->cap_bpts = N;
   }
   if (nc > h->cap_bclouds) {
-    if (!realloc_dev(h->boff_dev, (uint64_t)nc + 1) || !realloc_dev(h->bclouds, nc) || !realloc_dev(h->border, nc) ||
-        !realloc_dev(h->bsample, nc) || !realloc_dev(h->bhint_f, (uint64_t)nc * batch_hint_fine()) ||
+    h->cap_bclouds = 0;
+    if (!realloc_dev(h->boff_dev, (uint64_t)nc + 1) || !realloc_dev(h->bclouds, nc) || !realloc_dev(h->bstates, nc) ||
+        !realloc_dev(h->bhint_f, (uint64_t)nc * batch_hint_fine()) ||
         !realloc_dev(h->bhint_c, (uint64_t)nc * batch_hint_coarse()) || !realloc_dev(h->bcbox, 6ull * nc))
       return DT_ENOMEM;
     h->cap_bclouds = nc;
   }
   if (T > h->cap_tets) {
+    h->cap_tets = 0;
     if (!realloc_dev(h->tets, T) || !realloc_dev(h->claim, 2 * T)) return DT_ENOMEM;
     h->cap_tets = T;
   }
+  if (T > h->cap_lock) {
+    h->cap_lock = 0;
+    if (!realloc_dev(h->lock, T)) return DT_ENOMEM;
+    cudaMemsetAsync(h->lock, 0, T * sizeof(uint32_t), h->stream);
+    h->cap_lock = T;
+  }
   if (T > h->cap_free) {
+    h->cap_free = 0;
     if (!realloc_dev(h->freelist, T) || !realloc_dev(h->pending, T)) return DT_ENOMEM;
     h->cap_free = T;
   }
-  if (!h->bstats && (!realloc_dev(h->bstats, kBatchStatSlots) || !realloc_dev(h->bnext, 1))) return DT_ENOMEM;
-  // workspaces and states for the largest grid of any block shape
-  int shapes[8];
-  int ns = batch_shapes(shapes, 8);
-  uint64_t states = 0;
-  size_t ws = 0;
-  const int sms = sm_count();
-  for (int i = 0; i < ns; ++i) {
-    uint64_t blocks = (uint64_t)std::max(1, batch_blocks_per_sm(shapes[i])) * sms;
-    states = std::max(states, blocks);
-    ws = std::max(ws, (size_t)blocks * (shapes[i] & 255) * batch_ws_stride());
-  }
-  if (states > h->cap_bstates) {
-    if (!realloc_dev(h->bstates, states)) return DT_ENOMEM;
-    cudaMemsetAsync(h->bstates, 0, states * sizeof(DevState), h->stream);
-    h->cap_bstates = states;
-  }
-  if (ws > h->cap_bws) {
-    if (!realloc_dev(h->bws, ws)) return DT_ENOMEM;
-    h->cap_bws = ws;
-  }
-  return DT_OK;
+  if (!h->bstats && !realloc_dev(h->bstats, kBatchTotals)) return DT_ENOMEM;
+  return reserve_borrow(h);
 }
 
 Ctx batch_ctx(dt_handle* h) {
   Ctx c = make_ctx(h);
   c.coherent = 1;  // a block reads back the tetrahedra it writes
-  c.max_walk = h->cfg.max_walk_steps ? h->cfg.max_walk_steps : kDefaultWalk;
+  c.max_walk = h->cfg.max_walk_steps ? h->cfg.max_walk_steps : kAsyncWalk;
   c.subdet = nullptr;  // the batch store has no cache
   return c;
+}
+
+BatchMem batch_mem(dt_handle* h) {
+  return BatchMem{h->bclouds, h->n_clouds, h->bstates, h->vflag, h->bdup, {h->blist_a, h->blist_b}, h->blist_big,
+                  h->bhint_f, h->bhint_c, h->lock, h->async_borrow_ws, h->async_borrow_busy, kAsyncBorrow, h->beta,
+                  h->ows.bad, h->bstats};
 }
 
 // Batched S1..S4, the vertex records and the per-cloud hint grids: enqueued on the batch stream,
@@ -1923,7 +1915,7 @@ Ctx batch_ctx(dt_handle* h) {
 void batch_enqueue_prepare(dt_handle* h, const double* xyz, cudaStream_t s) {
   const uint64_t N = h->boff[h->n_clouds];
   cudaMemsetAsync(h->ows.bad, 0, 4, s);
-  order_batch(xyz, N, h->boff_dev, h->n_clouds, h->cfg.seed, h->gamma, h->ows, h->bcid, h->bcbox, s);
+  order_batch(xyz, N, h->boff_dev, h->n_clouds, h->cfg.seed, h->gamma_async, h->ows, h->bcid, h->bcbox, s);
   k_build_pts<<<grid_for(N, 256), 256, 0, s>>>(xyz, h->ows.perm, h->ows.dup, N, 0, h->pts, h->ptf, h->vflag,
                                                 h->point_hint);
   ++g_kernel_launches;
@@ -1931,84 +1923,157 @@ void batch_enqueue_prepare(dt_handle* h, const double* xyz, cudaStream_t s) {
   batch_prepare(h->bclouds, h->bcbox, h->n_clouds, h->beta, s);
 }
 
-// Reset of the clouds and the persistent launch over order[0 .. n) with block shape W.
-int batch_enqueue_insert(dt_handle* h, int W, float alpha, const uint32_t* order, uint32_t n, bool reset_all,
-                         cudaStream_t s) {
-  batch_reset(h->bclouds, reset_all ? nullptr : order, reset_all ? h->n_clouds : n, h->claim, h->bhint_f, h->bhint_c,
-              h->bdup, h->vflag, h->point_hint, s);
-  cudaMemsetAsync(h->bnext, 0, 4, s);
-  cudaMemsetAsync(h->bstats, 0, kBatchStatSlots * 8, s);
-  const unsigned blocks = (unsigned)std::max(1, batch_blocks_per_sm(W)) * (unsigned)sm_count();
-  return batch_launch(W, std::min<unsigned>(blocks, n), batch_ctx(h), h->bclouds, order, n, h->bnext, h->vflag,
-                      h->blist_a, h->blist_b, h->blist_big, h->bhint_f, h->bhint_c, h->bstates, h->bws,
-                      batch_ws_stride(), alpha, h->gamma, h->beta, h->bstats, s);
-}
-
-// One timed launch over order[0 .. n) (the autotuner's trials); device ms, or < 0 on failure.
-float batch_run(dt_handle* h, int W, float alpha, const uint32_t* order, uint32_t n, bool reset_all) {
-  cudaStream_t s = h->bs;
-  cudaEventRecord(h->bev[2], s);
-  int rc = batch_enqueue_insert(h, W, alpha, order, n, reset_all, s);
-  cudaEventRecord(h->bev[3], s);
-  if (rc != DT_OK || cudaStreamSynchronize(s) != cudaSuccess) return -1.f;
-  float ms = 0.f;
-  cudaEventElapsedTime(&ms, h->bev[2], h->bev[3]);
-  return ms;
-}
-
-// Autotuner: block shape (warps per block) and round size (concurrent insertions per mesh
-// vertex) timed on a sample of the clouds spread over the size order; the fastest is kept for
-// batches with the same signature (cloud count and size range).
-int batch_tune(dt_handle* h, const std::vector<uint32_t>& by_size, uint64_t sig) {
-  const uint32_t nc = h->n_clouds;
-  // DT_BATCH_WARPS / DT_BATCH_ALPHA restrict the candidates (warps per block; round size)
-  const char* fw = std::getenv("DT_BATCH_WARPS");
-  const char* fa = std::getenv("DT_BATCH_ALPHA");
-  h->batch_tune_ms = 0.0;
-  // the sample: every k-th cloud of the size order, a quarter of the batch (at least enough to
-  // fill the GPU several times), so that the trials see the batch's tail as well as its bulk
-  const uint32_t want = std::min<uint32_t>(nc, std::max<uint32_t>(8u * (uint32_t)sm_count(), nc / 4));
-  const uint32_t step = std::max<uint32_t>(1, nc / std::max<uint32_t>(want, 1));
-  std::vector<uint32_t> sample;
-  for (uint32_t k = 0; k < nc && sample.size() < want; k += step) sample.push_back(by_size[k]);
-  if (cudaMemcpyAsync(h->bsample, sample.data(), sample.size() * 4, cudaMemcpyHostToDevice, h->bs) != cudaSuccess)
-    return DT_ECUDA;
-  int shapes[8];
-  int ns = batch_shapes(shapes, 8);
-  if (const char* fs = std::getenv("DT_BATCH_SHAPE")) {  // one exact shape: warps | (min blocks << 8)
-    shapes[0] = std::atoi(fs);
-    ns = 1;
-  }
-  std::vector<float> alphas = {0.1f, 0.3f};
-  if (fa) alphas = {(float)std::atof(fa)};
-  float best = -1.f;
-  auto t0 = std::chrono::steady_clock::now();
-  for (int i = 0; i < ns; ++i) {
-    if (fw && std::atoi(fw) != (shapes[i] & 255)) continue;
-    for (float a : alphas) {
-      float ms = batch_run(h, shapes[i], a, h->bsample, (uint32_t)sample.size(), false);
-      if (ms < 0.f) return DT_ECUDA;
-      if (best < 0.f || ms < best) {
-        best = ms;
-        h->batch_W = shapes[i];
-        h->batch_alpha = a;
+// The segments of every launch of a batch, from the cloud sizes alone. Launch k takes the k-th
+// wave of every cloud that has one, in as many segments as a launch on that cloud alone would
+// have warps, and a few warps for the points that the other clouds carry over (a launch empties
+// every cloud's list); three launches without waves follow for the points that lost, the last of
+// them with one warp per cloud, which nothing can hold up.
+int batch_plan(dt_handle* h, const uint64_t* off, uint32_t nc, cudaStream_t s) {
+  std::vector<uint64_t> key = {nc, h->async_warps};
+  uint64_t bits[2];
+  std::memcpy(&bits[0], &h->alpha_async, 8);
+  std::memcpy(&bits[1], &h->gamma_async, 8);
+  key.insert(key.end(), bits, bits + 2);
+  key.insert(key.end(), off, off + nc + 1);
+  if (key == h->bplan_key) return DT_OK;
+  std::vector<std::vector<uint4>> launch;
+  constexpr uint64_t kMostSegs = 4096;  // of one cloud: the segment's number has 16 bits
+  // the vertices that all clouds together hold before each launch: many clouds fill the chip with
+  // fewer warps each, which lose less to one another (512 clouds: 98.7 ms at alpha 0.05, 78.5 at 0.02,
+  // 71.4 at 0.01, 73.2 at 0.004)
+  std::vector<uint64_t> before;
+  for (uint32_t c = 0; c < nc; ++c) {
+    const uint64_t n = off[c + 1] - off[c];
+    size_t k = 0;
+    for (int r = 0; brio_round_begin(r) < n; ++r) {
+      const uint64_t b = brio_round_begin(r), m = std::min(brio_round_begin(r + 1), n) - b;
+      for (int w = 0; w < kMaxWaves; ++w, ++k) {
+        const uint64_t lo = w == 0 ? 0 : wave_end(m, b, h->gamma_async, w - 1);
+        if (lo >= m) break;
+        if (before.size() <= k) before.resize(k + 1, 0);
+        before[k] += b + lo;
       }
     }
   }
-  h->batch_tune_ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
-  h->batch_sig = sig;
-  return h->batch_W ? DT_OK : DT_ELIMIT;
+  for (uint32_t c = 0; c < nc; ++c) {
+    const uint64_t n = off[c + 1] - off[c];
+    size_t k = 0;
+    for (int r = 0; brio_round_begin(r) < n; ++r) {
+      const uint64_t b = brio_round_begin(r), m = std::min(brio_round_begin(r + 1), n) - b;
+      uint64_t lo = 0;
+      for (int w = 0; w < kMaxWaves && lo < m; ++w, ++k) {
+        const uint64_t hi = wave_end(m, b, h->gamma_async, w), len = hi - lo, first = off[c] + b + lo;
+        const uint64_t mesh = std::max<uint64_t>(b + lo, 4);
+        const double most = std::max(0.01, 2.0 * async_max_warps_exact() / (double)std::max<uint64_t>(before[k], 1));
+        uint64_t W = std::min({async_warps_for(h, mesh), (uint64_t)std::max(1.0, most * (double)mesh), len, kMostSegs});
+        const uint64_t L = (len + W - 1) / W;
+        W = (len + L - 1) / L;
+        if (launch.size() <= k) launch.resize(k + 1);
+        for (uint64_t i = 0; i < W; ++i)
+          launch[k].push_back(make_uint4(c, (uint32_t)(first + i * L), (uint32_t)(first + std::min(len, (i + 1) * L)),
+                                         (uint32_t)(i | (W << 16))));
+        lo = hi;
+      }
+    }
+  }
+  const auto carry_only = [&](std::vector<uint4>& l, uint32_t c, uint64_t W) {
+    for (uint64_t i = 0; off[c + 1] - off[c] > 4 && i < W; ++i) l.push_back(make_uint4(c, 0, 0, (uint32_t)(i | (W << 16))));
+  };
+  const auto few = [&](uint32_t c) { return std::min<uint64_t>((off[c + 1] - off[c]) / 512 + 1, 256); };
+  std::vector<uint32_t> met(nc, 0);  // the last launch + 1 that holds a segment of the cloud
+  for (size_t k = 0; k < launch.size(); ++k) {
+    for (const uint4& g : launch[k]) met[g.x] = (uint32_t)k + 1;
+    for (uint32_t c = 0; c < nc; ++c)
+      if (met[c] != k + 1) carry_only(launch[k], c, few(c));
+  }
+  for (int pass = 0; pass < 3; ++pass) {
+    launch.emplace_back();
+    for (uint32_t c = 0; c < nc; ++c) carry_only(launch.back(), c, pass == 2 ? 1 : few(c));
+  }
+  std::vector<uint4> all;
+  h->bplan.clear();
+  h->bplan_key.clear();
+  for (const auto& l : launch) {
+    h->bplan.emplace_back(all.size(), l.size());
+    all.insert(all.end(), l.begin(), l.end());
+  }
+  if (all.size() > h->cap_bsegs) {
+    h->cap_bsegs = 0;
+    if (!realloc_dev(h->bsegs, all.size())) return DT_ENOMEM;
+    h->cap_bsegs = all.size();
+  }
+  if (!all.empty() &&
+      cudaMemcpyAsync(h->bsegs, all.data(), all.size() * sizeof(uint4), cudaMemcpyHostToDevice, s) != cudaSuccess)
+    return DT_ECUDA;
+  if (cudaStreamSynchronize(s) != cudaSuccess) return DT_ECUDA;
+  h->bplan_key = key;
+  return DT_OK;
+}
+
+// A new mesh in every cloud, then the planned launches. *src: the list the points left are in.
+int batch_enqueue_insert(dt_handle* h, int warps, uint64_t slots, int* src, cudaStream_t s) {
+  const Ctx c = batch_ctx(h);
+  const BatchMem b = batch_mem(h);
+  // slots not handed out read as dead (see reserve_tets)
+  if (cudaMemsetAsync(h->tets, 0, slots * sizeof(Tet), s) != cudaSuccess) return DT_ECUDA;
+  batch_init(c, b, s);
+  *src = 0;
+  for (const auto& l : h->bplan) {
+    if (l.second == 0) continue;
+    const int rc = batch_launch(warps, c, b, h->bsegs + l.first, (uint32_t)l.second, *src, s);
+    if (rc != DT_OK) return rc;
+    *src = 1 - *src;
+  }
+  batch_finish(c, b, *src, s);
+  return DT_OK;
+}
+
+// Points that the planned launches left (large cavities, long walks): one warp per cloud until
+// none is left; as long as some are inserted, or a bounded number of times if not.
+int batch_leftovers(dt_handle* h, int src, unsigned long long* totals, cudaStream_t s) {
+  const Ctx c = batch_ctx(h);
+  const BatchMem b = batch_mem(h);
+  for (uint32_t idle = 0; totals[kBLeft] + totals[kBBig] > 0;) {
+    const unsigned long long before = totals[kBInserted];
+    int rc = DT_OK;
+    if (totals[kBBig] > 0) {
+      if (!h->bws && !realloc_dev(h->bws, kBatchBigWarps * batch_big_ws_bytes())) return DT_ENOMEM;
+      if ((rc = batch_launch_big(c, b, h->bws, kBatchBigWarps, src, s)) != DT_OK) return rc;
+    }
+    const auto& last = h->bplan.back();
+    if ((rc = batch_launch(4, c, b, h->bsegs + last.first, (uint32_t)last.second, src, s)) != DT_OK) return rc;
+    src = 1 - src;
+    batch_finish(c, b, src, s);
+    if (cudaMemcpyAsync(totals, h->bstats, kBatchTotals * 8, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+        cudaStreamSynchronize(s) != cudaSuccess)
+      return DT_ECUDA;
+    idle = totals[kBInserted] == before ? idle + 1 : 0;
+    if (idle > 64) {
+      h->last_dev_error = 102;  // host-side: retry passes stopped progressing
+      h->last_dev_info = (unsigned)totals[kBLeft];
+      return DT_ELIMIT;
+    }
+  }
+  return DT_OK;
 }
 
 int batch_impl(dt_handle* h, const double* xyz, const uint64_t* off, uint32_t nc) {
+  // DT_BATCH_ALPHA: warps per mesh vertex of this batch
+  struct AlphaGuard {
+    dt_handle* h;
+    double keep;
+    ~AlphaGuard() { h->alpha_async = keep; }
+  } guard{h, h->alpha_async};
+  if (const char* e = std::getenv("DT_BATCH_ALPHA")) h->alpha_async = std::max(1e-4, std::atof(e));
   const uint64_t N = off[nc];
   double f = h->cfg.tet_capacity_factor > 0 ? h->cfg.tet_capacity_factor : 8.0;
-  // slots per cloud: f per point plus room for the first tetrahedra and ghosts
+  // slots per cloud: f per point, room for the first tetrahedra and ghosts, and the few dozen slots
+  // that each of a launch's warps keeps of its own while it runs
   std::vector<BatchCloud> cl(nc);
   uint64_t T = 0, hash = 1469598103934665603ull;
   for (uint32_t c = 0; c < nc; ++c) {
     uint64_t n = off[c + 1] - off[c];
-    uint64_t cap = (uint64_t)(f * (double)n) + 64;
+    uint64_t cap = (uint64_t)(f * (double)n) + 64 + 64 * std::min<uint64_t>(async_warps_for(h, n), n);
     cl[c] = BatchCloud{};
     cl[c].vb = (uint32_t)off[c];
     cl[c].ve = (uint32_t)off[c + 1];
@@ -2032,45 +2097,36 @@ int batch_impl(dt_handle* h, const double* xyz, const uint64_t* off, uint32_t nc
   cudaStreamWaitEvent(s, h->bev[0], 0);
   h->n_clouds = nc;
   h->boff.assign(off, off + nc + 1);
-  std::vector<uint32_t> by_size(nc);
-  for (uint32_t c = 0; c < nc; ++c) by_size[c] = c;
-  std::stable_sort(by_size.begin(), by_size.end(), [&](uint32_t a, uint32_t b) {
-    return off[a + 1] - off[a] > off[b + 1] - off[b];
-  });
   if (cudaMemcpyAsync(h->boff_dev, off, (nc + 1) * 8ull, cudaMemcpyHostToDevice, s) != cudaSuccess ||
-      cudaMemcpyAsync(h->bclouds, cl.data(), nc * sizeof(BatchCloud), cudaMemcpyHostToDevice, s) != cudaSuccess ||
-      cudaMemcpyAsync(h->border, by_size.data(), nc * 4ull, cudaMemcpyHostToDevice, s) != cudaSuccess)
+      cudaMemcpyAsync(h->bclouds, cl.data(), nc * sizeof(BatchCloud), cudaMemcpyHostToDevice, s) != cudaSuccess)
     return DT_ECUDA;
   if (cudaStreamSynchronize(s) != cudaSuccess) return DT_ECUDA;  // host vectors go out of scope
   h->n_pts = N;
   h->batch_mode = true;
   unsigned int bad = 0;
-  // the autotuner needs the ordered points: prepare once eagerly, then time the candidates
-  uint64_t big = off[by_size[0] + 1] - off[by_size[0]];
-  uint64_t sig = ((uint64_t)nc << 40) ^ ((uint64_t)(64 - __builtin_clzll(N | 1)) << 32) ^
-                 (uint64_t)(64 - __builtin_clzll(big | 1));
-  const bool fixed = std::getenv("DT_BATCH_WARPS") || std::getenv("DT_BATCH_ALPHA") || std::getenv("DT_BATCH_SHAPE");
-  if (fixed || !h->batch_W || h->batch_sig != sig) {
-    batch_enqueue_prepare(h, xyz, s);
-    cudaMemcpyAsync(&bad, h->ows.bad, 4, cudaMemcpyDeviceToHost, s);
-    if (cudaStreamSynchronize(s) != cudaSuccess) return DT_ECUDA;
-    if (bad) return DT_EINVAL;
-    if ((rc = batch_tune(h, by_size, sig)) != DT_OK) return rc;
-  } else {
-    h->batch_tune_ms = 0.0;
-  }
-  // the steady state: sort, records, reset and the persistent launch, replayed from a CUDA graph
-  // while the batch keeps its shape (same input buffer, cloud sizes, block shape and round size)
+  if ((rc = batch_plan(h, off, nc, s)) != DT_OK) return rc;
+  int warps = 4;  // per block; larger blocks are slower and kept for comparison
+  if (const char* e = std::getenv("DT_BATCH_WARPS")) warps = std::atoi(e);
+  if (const char* e = std::getenv("DT_BATCH_SHAPE")) warps = std::atoi(e) & 255;
+  warps = warps >= 1 && warps <= 32 ? warps : 4;
+  if (!batch_ready()) return DT_ECUDA;
+  int src = 0;
+  // sort, records, first tetrahedra and all launches, replayed from a CUDA graph while the batch
+  // keeps its shape (same input buffer, cloud sizes and block shape)
   // (every buffer the graph names is part of the key: an insert in between may have moved some)
   const void* const named[] = {xyz, h->pts, h->ptf, h->vflag, h->point_hint, h->tets, h->claim, h->freelist, h->pending,
                                h->ows.keys, h->ows.k0, h->ows.k1, h->ows.v0, h->ows.v1, h->ows.rounds, h->ows.dup,
                                h->ows.perm, h->ows.rank, h->ows.hist, h->ows.bad, h->bcid, h->bdup, h->blist_a,
-                               h->blist_b, h->blist_big, h->boff_dev, h->bclouds, h->border, h->bhint_f, h->bhint_c,
-                               h->bcbox, h->bstates, h->bws, h->bstats, h->bnext, h->beta};
-  std::vector<uint64_t> key = {N, nc, hash, h->cap_tets, h->cap_pts, h->cap_free, (uint64_t)h->batch_W, (uint64_t)(h->batch_alpha * 1e6f), h->cfg.seed,
-                               (uint64_t)(h->gamma * 1e9)};
+                               h->blist_b, h->blist_big, h->boff_dev, h->bclouds, h->bhint_f, h->bhint_c, h->bcbox,
+                               h->bstates, h->bstats, h->bsegs, h->lock, h->async_borrow_ws, h->async_borrow_busy,
+                               h->beta};
+  std::vector<uint64_t> key = {N, nc, hash, T, h->cap_tets, h->cap_pts, h->cap_free, (uint64_t)warps, h->cfg.seed,
+                               h->cfg.max_walk_steps};
   for (const void* p : named) key.push_back((uint64_t)(uintptr_t)p);
-  const bool use_graph = !std::getenv("DT_BATCH_NO_GRAPH");
+  key.insert(key.end(), h->bplan_key.begin(), h->bplan_key.end());
+  // (the first batch of a shape runs eagerly: a graph pays for its making only when it is replayed)
+  const bool use_graph = !std::getenv("DT_BATCH_NO_GRAPH") && key == h->bseen_key;
+  h->bseen_key = key;
   h->bgraph_used = false;
   if (use_graph && !(h->bexec && key == h->bgraph_key)) {
     if (h->bexec) cudaGraphExecDestroy(h->bexec);
@@ -2084,13 +2140,14 @@ int batch_impl(dt_handle* h, const double* xyz, const uint64_t* off, uint32_t nc
       cudaEventRecordWithFlags(h->bev[1], s, cudaEventRecordExternal);
       batch_enqueue_prepare(h, xyz, s);
       cudaEventRecordWithFlags(h->bev[2], s, cudaEventRecordExternal);
-      int rl = batch_enqueue_insert(h, h->batch_W, h->batch_alpha, h->border, nc, true, s);
+      int rl = batch_enqueue_insert(h, warps, T, &src, s);
       cudaEventRecordWithFlags(h->bev[3], s, cudaEventRecordExternal);
       ok = cudaStreamEndCapture(s, &h->bgraph) == cudaSuccess && rl == DT_OK;
     }
     if (ok) ok = cudaGraphInstantiate(&h->bexec, h->bgraph, 0) == cudaSuccess;
     if (ok) {
       h->bgraph_key = key;
+      h->bgraph_src = src;
       h->bgraph_kernels = g_kernel_launches - k0;
     } else {
       cudaGetLastError();  // capture unsupported here: run the same sequence eagerly
@@ -2104,21 +2161,24 @@ int batch_impl(dt_handle* h, const double* xyz, const uint64_t* off, uint32_t nc
     if (cudaGraphLaunch(h->bexec, s) != cudaSuccess) return DT_ECUDA;
     g_kernel_launches += h->bgraph_kernels;
     h->bgraph_used = true;
+    src = h->bgraph_src;
   } else {
     cudaEventRecord(h->bev[1], s);
     batch_enqueue_prepare(h, xyz, s);
     cudaEventRecord(h->bev[2], s);
-    if ((rc = batch_enqueue_insert(h, h->batch_W, h->batch_alpha, h->border, nc, true, s)) != DT_OK) return rc;
+    if ((rc = batch_enqueue_insert(h, warps, T, &src, s)) != DT_OK) return rc;
     cudaEventRecord(h->bev[3], s);
   }
-  // results: per-cloud status and sizes, and the batch counters
-  h->bclouds_host.resize(nc);
-  unsigned long long st[kBatchStatSlots];
+  // results: the totals, what the planned launches left, then every cloud's status and size
+  unsigned long long st[kBatchTotals];
   cudaMemcpyAsync(&bad, h->ows.bad, 4, cudaMemcpyDeviceToHost, s);
-  cudaMemcpyAsync(h->bclouds_host.data(), h->bclouds, nc * sizeof(BatchCloud), cudaMemcpyDeviceToHost, s);
   cudaMemcpyAsync(st, h->bstats, sizeof(st), cudaMemcpyDeviceToHost, s);
   if (cudaStreamSynchronize(s) != cudaSuccess) return DT_ECUDA;
   if (bad) return DT_EINVAL;
+  if ((rc = batch_leftovers(h, src, st, s)) != DT_OK) return rc;
+  h->bclouds_host.resize(nc);
+  cudaMemcpyAsync(h->bclouds_host.data(), h->bclouds, nc * sizeof(BatchCloud), cudaMemcpyDeviceToHost, s);
+  if (cudaStreamSynchronize(s) != cudaSuccess) return DT_ECUDA;
   float ms_sort = 0.f, ms_ins = 0.f;
   if (cudaEventElapsedTime(&ms_sort, h->bev[1], h->bev[2]) != cudaSuccess) ms_sort = 0.f;
   if (cudaEventElapsedTime(&ms_ins, h->bev[2], h->bev[3]) != cudaSuccess) ms_ins = 0.f;
@@ -2134,26 +2194,24 @@ int batch_impl(dt_handle* h, const double* xyz, const uint64_t* off, uint32_t nc
       h->last_dev_info = b.info;
     }
   }
-  agg.n_inserted = st[0];
-  agg.n_conflicts = st[1];
-  agg.n_attempts = st[2];
-  agg.sum_cavity = st[3];
-  agg.sum_ball = st[4];
-  agg.sum_walk = st[5];
-  agg.n_big = st[7];
-  agg.n_exact = st[9];
-  agg.n_sos = st[10];
+  agg.n_inserted = st[kBInserted];
+  agg.n_conflicts = st[kBConflicts];
+  agg.n_attempts = st[kBAttempts];
+  agg.sum_cavity = st[kBCavity];
+  agg.sum_ball = st[kBBall];
+  agg.sum_walk = st[kBWalk];
+  agg.n_exact = st[kBExact];
+  agg.n_sos = st[kBSos];
   agg.bump = used;
   std::memcpy(h->st_host, &agg, sizeof(agg));
   h->stats.ms_sort = ms_sort;
   h->stats.ms_insert = ms_ins;
-  h->stats.n_rounds = st[8];
+  h->stats.n_rounds = h->bplan.size();
   h->stats.n_passes = 0;
   h->stats.n_clouds_degenerate = degenerate;
-  h->stats.batch_warps = (uint64_t)(h->batch_W & 255);
-  h->stats.batch_min_blocks = (uint64_t)(h->batch_W >> 8);
-  h->stats.batch_alpha = h->batch_alpha;
-  h->stats.ms_batch_tune = h->batch_tune_ms;
+  h->stats.batch_warps = (uint64_t)warps;
+  h->stats.batch_min_blocks = warps <= 4 ? 4 : 1;
+  h->stats.batch_alpha = h->alpha_async;
   h->stats.batch_graph = h->bgraph_used ? 1 : 0;
   // DT_EDEGENERATE only when no cloud could be triangulated
   if (h->last_dev_error) return map_dev_error(h->last_dev_error);
@@ -2801,8 +2859,7 @@ void dt_destroy(dt_handle* h) {
   cudaFree(h->bbox_dev);
   cudaFree(h->boff_dev);
   cudaFree(h->bclouds);
-  cudaFree(h->border);
-  cudaFree(h->bsample);
+  cudaFree(h->bsegs);
   cudaFree(h->bcid);
   cudaFree(h->bdup);
   cudaFree(h->blist_a);
@@ -2814,7 +2871,6 @@ void dt_destroy(dt_handle* h) {
   cudaFree(h->bstates);
   cudaFree(h->bws);
   cudaFree(h->bstats);
-  cudaFree(h->bnext);
   cudaFree(h->beta);
   cudaFree(h->log_nc);
   cudaFree(h->log_lost);

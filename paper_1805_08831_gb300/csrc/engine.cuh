@@ -56,7 +56,8 @@ struct Ctx {
   int cb;  // bits per axis of the hint grid
   uint32_t max_walk;
   int coherent;  // 1 when this kernel also writes the tetrahedra it reads (L2 loads)
-  uint32_t ntets;  // tetrahedron slots allocated (bounds of every id read from the mesh)
+  uint32_t tbase;  // first slot of the mesh (0, or a batch cloud's)
+  uint32_t ntets;  // end of its tetrahedron slots (bounds of every id read from the mesh)
   uint32_t npts;   // vertex slots allocated
   float4* subdet;  // sub-determinant cache of the asynchronous engine (two float4 per slot) or
                    // null; the engines that do not fill it mark the entries they replace invalid

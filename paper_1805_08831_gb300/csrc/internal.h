@@ -136,6 +136,7 @@ struct InsertLog;
 // cavities too large for a warp's workspaces to big_out.
 struct AsyncIO {
   const uint32_t* q;
+  const uint8_t* vflag;  // with q null: segments are vertex ranges, flagged vertices left out
   uint64_t m, L;
   uint32_t W;
   uint32_t max_walk;
@@ -170,25 +171,48 @@ size_t async_big_ws_bytes();
 int async_launch_big(const Ctx& c, const AsyncIO& io, uint32_t* lock, const InsertLog& lg, void* ws, cudaStream_t s);
 
 // ---------------------------------------------------------------- batch.cu (dt_batch)
-size_t batch_ws_stride();       // bytes of one warp's workspace
 uint32_t batch_hint_fine();     // fine hint cells per cloud
 uint32_t batch_hint_coarse();   // coarse hint cells per cloud
 int batch_cb();                 // bits per axis of a cloud's fine hint grid
-int batch_shapes(int* shapes, int max_n);  // block shapes: warps | (min blocks per SM << 8)
-int batch_blocks_per_sm(int shape);         // resident blocks per SM of a shape
-constexpr int kBatchStatSlots = 11;      // accumulators batch_launch adds into
-// One persistent launch over the clouds order[0 .. n_clouds) (see batch.cu); *next must be 0.
-int batch_launch(int shape, unsigned blocks, const Ctx& c, BatchCloud* clouds, const uint32_t* order, uint32_t n_clouds,
-                 unsigned int* next, uint8_t* vflag, uint32_t* list_a, uint32_t* list_b, uint32_t* list_big,
-                 uint32_t* hint_fine, uint32_t* hint_coarse, DevState* states, char* wsmem, size_t wsstride,
-                 float alpha, double gamma, const float* eta, unsigned long long* stats, cudaStream_t s);
+// Totals of a batch: inserted, conflicts, attempts, sum |C|, sum |B|, walk steps, large cavities
+// waiting, points waiting, duplicates met, exact and perturbed predicates.
+enum BatchTotal { kBInserted, kBConflicts, kBAttempts, kBCavity, kBBall, kBWalk, kBBig, kBLeft, kBDups, kBExact, kBSos,
+                  kBatchTotals };
+// The batch's arrays: clouds and, by cloud, the state (allocator, queues, counters) and hint
+// grids; by vertex, flags and the lists of points carried over and of large cavities (a cloud
+// uses its own range); owner words; borrowed large-cavity workspaces; the FP32 error term.
+struct BatchMem {
+  BatchCloud* clouds;
+  uint32_t n_clouds;
+  DevState* states;
+  uint8_t* vflag;
+  const uint8_t* dup;  // duplicates, by vertex
+  uint32_t *list[2], *list_big;
+  uint32_t *hint_fine, *hint_coarse;
+  uint32_t* lock;
+  void* big_ws;
+  unsigned int* big_busy;
+  uint32_t big_n;
+  const float* eta;
+  const unsigned int* bad;     // non-zero: bad coordinates, nothing is inserted
+  unsigned long long* totals;  // kBatchTotals
+};
+bool batch_ready();  // the kernels' shared memory is set up (call before any capture)
+// A new mesh in every cloud: state, hints and flags, the first tetrahedra.
+void batch_init(const Ctx& c, const BatchMem& b, cudaStream_t s);
+// One launch over the segments segs[0, n) (x: cloud, y..z: vertices, w: index among the cloud's
+// segments | their number << 16), each after its share of the points of list `src`, and the close
+// of every cloud's allocator; what is not inserted goes to list 1 - src.
+int batch_launch(int warps, const Ctx& c, const BatchMem& b, const uint4* segs, uint32_t n, int src, cudaStream_t s);
+// Large cavities waiting, one warp per cloud (async_big_ws_bytes-like workspaces of
+// batch_big_ws_bytes() each at ws, n of them).
+size_t batch_big_ws_bytes();
+int batch_launch_big(const Ctx& c, const BatchMem& b, void* ws, uint32_t n, int src, cudaStream_t s);
+// Every cloud's outcome (status, slots used, vertices inserted) and the totals.
+void batch_finish(const Ctx& c, const BatchMem& b, int src, cudaStream_t s);
 // Per-cloud hint grids from the clouds' boxes cbox [6 n_clouds], and the FP32 stage's error
 // term eta (from the largest |coordinate| of the batch) into *eta, on the device.
 void batch_prepare(BatchCloud* clouds, const double* cbox, uint32_t n_clouds, float* eta, cudaStream_t s);
-// Resets the clouds list[0 .. n_list) (all clouds when list is null) for a new launch.
-void batch_reset(const BatchCloud* clouds, const uint32_t* list, uint32_t n_list, unsigned long long* claim,
-                 uint32_t* hint_fine, uint32_t* hint_coarse, const uint8_t* dup_sorted, uint8_t* vflag,
-                 uint32_t* point_hint, cudaStream_t s);
 // Finite tetrahedra per cloud with cloud-local ids: pass 0 counts into counts[c], pass 1
 // writes cloud c's from out_off[c].
 void batch_collect(const BatchCloud* clouds, uint32_t n_clouds, const Tet* tets, const Pt* pts, const uint64_t* in_off,

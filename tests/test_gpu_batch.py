@@ -182,3 +182,48 @@ def test_insert_after_a_larger_batch_on_the_same_handle():
         t.clear()
         t.insert(torch.from_numpy(x).cuda())
         assert np.array_equal(t.tets_numpy(), ref)
+
+
+@pytest.mark.parametrize("sizes", [(0, 3, 4, 5, 6), (2047, 2048, 2049), (14336, 14337, 40), (1,), (900, 20001)])
+def test_batch_at_the_edges_of_waves_and_segments(sizes):
+    """Cloud sizes around the BRIO round ends, clouds with nothing to insert, and a cloud whose
+    launches go on long after the others' last wave."""
+    clouds = [synth.uniform_cube(n, 300 + n) if n else np.zeros((0, 3)) for n in sizes]
+    if sizes == (1,):
+        with pytest.raises(dt.DTError) as e:
+            run_batch(clouds)
+        assert e.value.code == dt.DT_EDEGENERATE
+        return
+    got, st = run_batch(clouds)
+    assert st["n_clouds_degenerate"] == sum(n < 4 for n in sizes)
+    for c, x in enumerate(clouds):
+        ref = oracle.delaunay(x)[0] if len(x) >= 4 else np.zeros((0, 4), np.uint32)
+        assert np.array_equal(got[c], ref), c
+
+
+def test_batch_cavities_beyond_the_borrowed_workspaces():
+    """Centres of shells: cavities of hundreds to thousands of tetrahedra, in the borrowed and in the
+    largest workspaces, beside an ordinary cloud."""
+    g = np.random.default_rng(5)
+    clouds = [synth.uniform_cube(500, 6)]
+    for n in (300, 3000):
+        s = g.normal(size=(n, 3))
+        s /= np.linalg.norm(s, axis=1, keepdims=True)
+        clouds.append(np.concatenate([s, 0.01 * g.normal(size=(5, 3))]))
+    got, _ = run_batch(clouds)
+    assert_clouds_match(clouds, got)
+
+
+def test_batch_refuses_bad_coordinates_and_goes_on():
+    xyz, off = synth.batched_clouds(6, 8, lo=50, hi=500)
+    bad = xyz.copy()
+    bad[77, 1] = np.nan
+    with dt.Triangulation(seed=0) as t:
+        for _ in range(2):
+            with pytest.raises(dt.DTError) as e:
+                t.batch(torch.from_numpy(bad).cuda(), off)
+            assert e.value.code == dt.DT_EINVAL
+        t.clear()
+        t.batch(torch.from_numpy(xyz).cuda(), off)
+        tets, coff = t.tets_batch()
+    assert_clouds_match(split(xyz, off), [tets[int(coff[c]):int(coff[c + 1])] for c in range(6)])
