@@ -71,19 +71,26 @@ __global__ void k_async_close_state(Ctx c, int consumed_q) {
   st->blocks_done = 0;
 }
 
-// Resident blocks per SM the FP32 kernel is built for: 8 (32 warps per SM at 64 registers)
-// measured fastest, 255 ms per 1e7 uniform step when first built against 265 at 6 (80 registers),
-// 276 at 5 and 301 at 4; 6 is kept for sweeps. The kernel with the exact stages holds 128 registers
-// at 4 blocks: its calls save and restore fewer of them.
-constexpr int kExactBlocks = 4;
+// Resident blocks per SM the kernels are built for. The FP32 kernel: 8 (32 warps per SM at 64
+// registers) for launches that fill the chip, where it measured fastest (255 ms per 1e7 uniform step
+// when first built against 265 at 6, 276 at 5 and 301 at 4), 4 (128 registers, no spills) for
+// launches that fit the chip with that, where the latency of one insertion is what counts. The
+// kernel with the exact stages: 4, its calls save and restore fewer registers.
+constexpr int kFullBlocks = 8, kFewBlocks = 4, kExactBlocks = 4;
 
-bool async_six_blocks() {
-  static const bool six = [] {
-    const char* e = std::getenv("DT_ASYNC_BLOCKS");
-    const int v = e ? std::atoi(e) : 8;
-    return v >= 4 && v <= 6;
-  }();
-  return six;
+template <int kMinBlocks, bool kCache = false, bool kExact = false>
+int resident_warps() {
+  int dev = 0, sms = 0, per = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_async<kMinBlocks, kCache, kExact>, kAW * 32, 0) != cudaSuccess)
+    per = kMinBlocks;
+  return std::max(1, sms * std::max(per, 1) * kAW);
+}
+
+int async_max_warps_few() {
+  static const int cached = resident_warps<kFewBlocks>();
+  return cached;
 }
 
 }  // namespace
@@ -95,9 +102,9 @@ int async_launch(const Ctx& c, const AsyncIO& io, uint32_t* lock, const InsertLo
   cc.max_walk = io.max_walk;
   const unsigned blocks = (io.W + kAW - 1) / kAW;
   if (io.exact) k_async<kExactBlocks, false, true><<<blocks, kAW * 32, 0, s>>>(cc, io, lock, lg);
-  else if (c.subdet) k_async<8, true><<<blocks, kAW * 32, 0, s>>>(cc, io, lock, lg);
-  else if (async_six_blocks()) k_async<6><<<blocks, kAW * 32, 0, s>>>(cc, io, lock, lg);
-  else k_async<8><<<blocks, kAW * 32, 0, s>>>(cc, io, lock, lg);
+  else if (c.subdet) k_async<kFullBlocks, true><<<blocks, kAW * 32, 0, s>>>(cc, io, lock, lg);
+  else if (io.W <= (uint32_t)async_max_warps_few()) k_async<kFewBlocks><<<blocks, kAW * 32, 0, s>>>(cc, io, lock, lg);
+  else k_async<kFullBlocks><<<blocks, kAW * 32, 0, s>>>(cc, io, lock, lg);
   k_async_close_copy<<<152, 256, 0, s>>>(cc);
   k_async_close_state<<<1, 1, 0, s>>>(cc, io.carry_n ? io.carry_q : -1);
   g_kernel_launches += 3;
@@ -122,31 +129,12 @@ int async_launch_big(const Ctx& c, const AsyncIO& io, uint32_t* lock, const Inse
 }
 
 int async_max_warps() {
-  static int cached = 0;
-  if (!cached) {
-    int dev = 0, sms = 0, per = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const cudaError_t e =
-        async_six_blocks() ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_async<6>, kAW * 32, 0)
-                           : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_async<8>, kAW * 32, 0);
-    if (e != cudaSuccess) per = async_six_blocks() ? 6 : 8;
-    cached = std::max(1, sms * std::max(per, 1) * kAW);
-  }
+  static const int cached = resident_warps<kFullBlocks>();
   return cached;
 }
 
 int async_max_warps_exact() {
-  static int cached = 0;
-  if (!cached) {
-    int dev = 0, sms = 0, per = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_async<kExactBlocks, false, true>, kAW * 32, 0) !=
-        cudaSuccess)
-      per = kExactBlocks;
-    cached = std::min(std::max(1, sms * std::max(per, 1) * kAW), async_max_warps());
-  }
+  static const int cached = std::min(resident_warps<kExactBlocks, false, true>(), async_max_warps());
   return cached;
 }
 

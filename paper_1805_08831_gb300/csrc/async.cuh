@@ -1071,16 +1071,17 @@ __device__ __forceinline__ void run_segment(const Ctx& c, const AsyncIO& io, W& 
       if (lane == 0) to_queue(io, c, 1, p);
     } else if (r == kAExact) {
       if (lane == 0) to_queue(io, c, 2, p);
-    } else if (r == kALost && w.nd < kADefer && (!retried || (i >= w.e0 && w.k0 >= w.k1 && w.tail < kATail))) {
-      // lost once: again after a few other insertions; at the segment's end, where the warps that
-      // it loses to are about done too, again and again (a bounded number of times)
+    } else if (r == kALost && w.nd < kADefer && (!retried || w.nd < kADefer / 2) && w.tail < kATail) {
+      // lost: again after a few other insertions; at the segment's end, where the warps that it
+      // loses to are about done too, again and again (a bounded number of times)
+      const bool end = i >= w.e0 && w.k0 >= w.k1;
       __syncwarp();
       if (lane == 0) {
         w.defer[(w.dhead + w.nd) % kADefer] = p;
         w.nd += 1;
-        w.tail += retried ? 1 : 0;
+        w.tail += end ? 1 : 0;
       }
-      if (retried) __nanosleep(2000);
+      if (end) __nanosleep(2000);
     } else {  // a walk over its step bound, or a point that lost again: the next pass
       if (lane == 0) to_queue(io, c, 0, p);
     }

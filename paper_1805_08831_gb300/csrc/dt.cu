@@ -24,7 +24,7 @@ constexpr uint32_t kDefaultWalk = 48;          // walk steps per pass (a longer 
 constexpr uint32_t kAsyncWalk = 4096;          // walk steps per attempt of the asynchronous engine
 constexpr uint32_t kAsyncBigWarps = 64;        // warps (workspaces) of a large-cavity launch
 constexpr uint32_t kBatchBigWarps = 16;        // warps (workspaces) of a batch's largest cavities
-constexpr double kSmallMeshWarps = 240;        // warps up to which a small mesh gets more than alpha allows
+constexpr double kSmallMeshWarps = 300;        // warps up to which a small mesh gets more than alpha allows
 constexpr uint64_t kDrainPoints = 8;           // points per warp of a list without a wave
 constexpr uint32_t kAsyncBorrow = 512;         // large-cavity workspaces the main kernel's warps may borrow
 constexpr uint64_t kLongWalkBelow = 8192;      // retry lists shorter than this walk up to
@@ -1117,12 +1117,12 @@ int reserve_points(dt_handle* h, uint64_t total) {
   return DT_OK;
 }
 
-// Warps of an asynchronous launch on a mesh: alpha per vertex, up to 2.4 times that while the mesh
-// is so small that a launch is a chain of insertions on a mostly empty chip (2047 points: 5.5 ms
-// at 0.05, 4.5 ms at 0.12; at 1e5 points and more 0.05 is the faster one).
+// Warps of an asynchronous launch on a mesh: alpha per vertex, up to 3 times that while the mesh is
+// so small that a launch is a chain of insertions on a mostly empty chip (2047 points: 3.9 ms at
+// 0.12 per vertex, 3.65 at 0.17; at 1e5 points and more 0.05 to 0.07 measure the same).
 uint64_t async_warps_for(const dt_handle* h, uint64_t mesh) {
   const double a = h->alpha_async * (double)mesh;
-  const uint64_t W = (uint64_t)std::max(1.0, std::max(a, std::min(2.4 * a, kSmallMeshWarps)));
+  const uint64_t W = (uint64_t)std::max(1.0, std::max(a, std::min(3.0 * a, kSmallMeshWarps)));
   return std::min<uint64_t>(W, h->async_warps ? h->async_warps : (uint64_t)async_max_warps());
 }
 
