@@ -28,6 +28,20 @@ __global__ void __launch_bounds__(kAW * 32, kMinBlocks) k_async(Ctx c, AsyncIO i
                       (uint32_t)(io.carry_n * (seg + 1) / io.W), lg);
 }
 
+// A launch of at most kLocalWarps warps on a mesh of at most a few hundred vertices: one block, the
+// mesh read and written through its SM's L1 (async.cuh, ld_mesh). An insertion that runs alone is a
+// chain of some thirty dependent reads, 13.5 us of them through L2.
+constexpr uint32_t kLocalWarps = 16;
+
+template <bool kExact>
+__global__ void __launch_bounds__(kLocalWarps * 32, 1) k_async_local(Ctx c, AsyncIO io, uint32_t* lock, InsertLog lg) {
+  extern __shared__ __align__(16) char s_mem[];
+  const uint32_t seg = threadIdx.x >> 5;
+  const uint64_t b0 = std::min<uint64_t>(seg * io.L, io.m), e0 = std::min<uint64_t>(b0 + io.L, io.m);
+  run_segment<kExact>(c, io, reinterpret_cast<SmallWST<false, true>*>(s_mem)[seg], lock, seg + 1, (uint32_t)b0,
+                      (uint32_t)e0, (uint32_t)(io.carry_n * seg / io.W), (uint32_t)(io.carry_n * (seg + 1) / io.W), lg);
+}
+
 // Large cavities (beyond the shared-memory workspaces): the same insertion with each warp's
 // workspace in global memory.
 template <bool kCache, bool kExact>
@@ -101,7 +115,10 @@ int async_launch(const Ctx& c, const AsyncIO& io, uint32_t* lock, const InsertLo
   cc.coherent = 1;
   cc.max_walk = io.max_walk;
   const unsigned blocks = (io.W + kAW - 1) / kAW;
-  if (io.exact) k_async<kExactBlocks, false, true><<<blocks, kAW * 32, 0, s>>>(cc, io, lock, lg);
+  const size_t local = io.W * sizeof(SmallWST<false, true>);
+  if (io.local && io.exact) k_async_local<true><<<1, io.W * 32, local, s>>>(cc, io, lock, lg);
+  else if (io.local) k_async_local<false><<<1, io.W * 32, local, s>>>(cc, io, lock, lg);
+  else if (io.exact) k_async<kExactBlocks, false, true><<<blocks, kAW * 32, 0, s>>>(cc, io, lock, lg);
   else if (c.subdet) k_async<kFullBlocks, true><<<blocks, kAW * 32, 0, s>>>(cc, io, lock, lg);
   else if (io.W <= (uint32_t)async_max_warps_few()) k_async<kFewBlocks><<<blocks, kAW * 32, 0, s>>>(cc, io, lock, lg);
   else k_async<kFullBlocks><<<blocks, kAW * 32, 0, s>>>(cc, io, lock, lg);
@@ -126,6 +143,16 @@ int async_launch_big(const Ctx& c, const AsyncIO& io, uint32_t* lock, const Inse
   k_async_close_state<<<1, 1, 0, s>>>(cc, io.carry_q);
   g_kernel_launches += 3;
   return cudaPeekAtLastError() == cudaSuccess ? DT_OK : DT_ECUDA;
+}
+
+// Most warps of a launch that runs as one block (AsyncIO::local), 0 if it cannot.
+uint32_t async_local_warps() {
+  static const bool ready =
+      cudaFuncSetAttribute(k_async_local<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)(kLocalWarps * sizeof(SmallWST<false, true>))) == cudaSuccess &&
+      cudaFuncSetAttribute(k_async_local<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)(kLocalWarps * sizeof(SmallWST<false, true>))) == cudaSuccess;
+  return ready ? kLocalWarps : 0;
 }
 
 int async_max_warps() {

@@ -79,12 +79,14 @@ struct AWSTail<kHashN, kFMaxN, 0> {
 // tetrahedra with their vertices as read, the boundary facets, the ball's slots, a private pool
 // of free slots, deferred points, and the warp's state (uniform across its lanes, written by
 // lane 0). kEdgeSlots: slots of the edge hash, 0 for the edge table.
-template <int kHashN, int kCMaxN, int kAMaxN, int kFMaxN, int kEdgeSlots, bool kCacheB>
+// kLocalB: the launch is one block, and the mesh is read and written through its SM's L1.
+template <int kHashN, int kCMaxN, int kAMaxN, int kFMaxN, int kEdgeSlots, bool kCacheB, bool kLocalB = false>
 struct AWS : AWSTail<kHashN, kFMaxN, kEdgeSlots> {
   static constexpr int kHash = kHashN, kCMax = kCMaxN, kAMax = kAMaxN, kFMax = kFMaxN;
   static constexpr bool kCache = kCacheB;  // conflict tests through the sub-determinant cache
   static constexpr int kPool = kFMaxN + 36;  // a refill of 32 slots always fits below kFMax
   static constexpr bool kTable = kEdgeSlots == 0;
+  static constexpr bool kLocal = kLocalB;
   using CI = typename std::conditional<(kCMaxN > 255), uint16_t, uint8_t>::type;
   static_assert(!kTable || kCMaxN + kAMaxN + kFMaxN <= 32 * 32, "a lane's lock mask holds its entries");
   uint32_t cl[kCMaxN];       // cavity slots
@@ -114,15 +116,57 @@ struct AWS : AWSTail<kHashN, kFMaxN, kEdgeSlots> {
 // Shared-memory workspace of the main kernel (cavities of up to 64 tetrahedra and 60 boundary
 // facets), the global-memory one a warp borrows for a larger cavity (145 KB), and that of the
 // large-cavity kernel (1.6 MB: the sphere's empty interior, a surface's first inner points).
-template <bool kCache>
-using SmallWST = AWS<256, 64, 64, 60, 0, kCache>;
-template <bool kCache>
-using LargeWST = AWS<4096, 640, 704, 704, 4096, kCache>;
+template <bool kCache, bool kLocal = false>
+using SmallWST = AWS<256, 64, 64, 60, 0, kCache, kLocal>;
+template <bool kCache, bool kLocal = false>
+using LargeWST = AWS<4096, 640, 704, 704, 4096, kCache, kLocal>;
 using LargeWS = LargeWST<false>;  // the same layout with and without the cache
 template <bool kCache>
 using HugeWST = AWS<32768, 6144, 6144, 6144, 32768, kCache>;
 
-__device__ __forceinline__ Tet ld_tet(const Tet* T, uint32_t t) { return load_tet_cg(T, t); }
+// Reads and writes of the mesh by warps that run beside its writers: through L2, or, when all of
+// them are in one block, through that block's L1, whose latency is a fraction (the first few
+// hundred insertions of a mesh are one chain of such reads).
+template <bool kLocal>
+__device__ __forceinline__ uint4 ld_mesh(const uint4* p) {
+  if constexpr (kLocal) {
+    uint4 r;
+    asm volatile("ld.relaxed.cta.global.v4.u32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w)
+                 : "l"(p)
+                 : "memory");
+    return r;
+  } else {
+    return __ldcg(p);
+  }
+}
+template <bool kLocal>
+__device__ __forceinline__ void st_mesh(uint4* p, const uint4& v) {
+  if constexpr (kLocal)
+    asm volatile("st.relaxed.cta.global.v4.u32 [%0], {%1, %2, %3, %4};" ::"l"(p), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w)
+                 : "memory");
+  else
+    __stcg(p, v);
+}
+template <bool kLocal>
+__device__ __forceinline__ void st_mesh(uint32_t* p, uint32_t v) {
+  if constexpr (kLocal) asm volatile("st.relaxed.cta.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+  else __stcg(p, v);
+}
+template <bool kLocal>
+__device__ __forceinline__ void fence_mesh() {
+  if constexpr (kLocal) __threadfence_block();
+  else __threadfence();
+}
+
+template <bool kLocal>
+__device__ __forceinline__ Tet ld_tet(const Tet* T, uint32_t t) {
+  Tet r;
+  const uint4* p = reinterpret_cast<const uint4*>(T + t);
+  r.v = ld_mesh<kLocal>(p);
+  r.n = ld_mesh<kLocal>(p + 1);
+  return r;
+}
 
 __device__ __forceinline__ bool same_tet(const Tet& a, const Tet& b) {
   return a.v.x == b.v.x && a.v.y == b.v.y && a.v.z == b.v.z && a.v.w == b.v.w && a.n.x == b.n.x &&
@@ -287,7 +331,7 @@ static __device__ __noinline__ int ghost_exact_at(const Pt* pts, DevState* st, c
 // the walk with kARestart (or it runs into its step bound); nothing is trusted before step 4
 // re-reads it under a lock. Called by the whole warp; the result is uniform. *n_out: the
 // neighbours of the tetrahedron reached.
-template <bool kExact>
+template <bool kExact, bool kLocal>
 __device__ __forceinline__ int walk_async(const Ctx& c, uint32_t p, const PtF& FP, uint32_t start, uint32_t salt,
                                           uint32_t max_steps, uint32_t* t_out, uint4* n_out, uint32_t* steps_out) {
   const int lane = threadIdx.x & 31;
@@ -300,7 +344,7 @@ __device__ __forceinline__ int walk_async(const Ctx& c, uint32_t p, const PtF& F
   for (;;) {
     if (t < c.tbase || t >= c.ntets) t = __ldcg(&c.st->anchor);
     if (t >= c.ntets) return kARestart;
-    T = ld_tet(c.tets, t);
+    T = ld_tet<kLocal>(c.tets, t);
     if (!tet_dead(T.v)) break;
     t = T.n.x;  // dead slot: follow its redirect
     if (++hops > 64) return kARestart;
@@ -309,7 +353,7 @@ __device__ __forceinline__ int walk_async(const Ctx& c, uint32_t p, const PtF& F
   int g = ghost_pos(T.v);
   if (g >= 0) {
     t = get4(T.n, g);
-    T = ld_tet(c.tets, t);
+    T = ld_tet<kLocal>(c.tets, t);
     if (tet_dead(T.v) || !rec_ok(T, c.ntets, c.npts)) return kARestart;
   }
   uint32_t prev = kNone, steps = 0;
@@ -359,7 +403,7 @@ __device__ __forceinline__ int walk_async(const Ctx& c, uint32_t p, const PtF& F
     const int exit = (__ffs(rot) - 1 + (int)((salt + steps) & 3)) & 3;
     prev = t;
     t = get4(T.n, exit);
-    T = ld_tet(c.tets, t);
+    T = ld_tet<kLocal>(c.tets, t);
     ++steps;
     if (tet_dead(T.v) || !rec_ok(T, c.ntets, c.npts)) {
       *t_out = t;
@@ -444,7 +488,7 @@ __device__ __forceinline__ int cavity_async(const Ctx& c, W& w, int ball, uint32
     int res = 0;
     Tet U;
     if (u < c.ntets) {
-      U = ld_tet(c.tets, u);
+      U = ld_tet<W::kLocal>(c.tets, u);
       res = conflict_async<W::kCache, kExact>(c, u, U, p, FP);
     }
     const unsigned m = __ballot_sync(kFull, res == 1);
@@ -478,7 +522,7 @@ __device__ __forceinline__ int cavity_async(const Ctx& c, W& w, int ball, uint32
     int res = 0;
     Tet U;
     if (first) {
-      U = ld_tet(c.tets, u);  // u < ntets: the record that names it was checked
+      U = ld_tet<W::kLocal>(c.tets, u);  // u < ntets: the record that names it was checked
       res = conflict_async<W::kCache, kExact>(c, u, U, p, FP);
       w.hval[h] = (uint8_t)res;
     }
@@ -677,7 +721,7 @@ __device__ __forceinline__ int try_insert(const Ctx& c, W& w, uint32_t* lock, ui
       }
       start = __shfl_sync(kFull, start, 0);
       uint32_t steps = 0;
-      const int ws = walk_async<kExact>(c, p, FP, start, p * 0x9E3779B1u >> 30, c.max_walk, &t0, &tn, &steps);
+      const int ws = walk_async<kExact, W::kLocal>(c, p, FP, start, p * 0x9E3779B1u >> 30, c.max_walk, &t0, &tn, &steps);
       if (lane == 0) {
         if (t0 != kNone && t0 < c.ntets) c.point_hint[p] = t0;
         w.cnt[5] += steps;
@@ -741,22 +785,22 @@ __device__ __forceinline__ int try_insert(const Ctx& c, W& w, uint32_t* lock, ui
       if (nx > 0) pool_give(c, w, w.ex, nx);
       return kALost;
     }
-    __threadfence();
+    fence_mesh<W::kLocal>();
     // 4. re-read under the locks
     bool same = true;
 #pragma unroll 1
-    for (int i = lane; i < nc; i += 32) same = same && same_tet(ld_tet(c.tets, w.cl[i]), w.cr[i]);
+    for (int i = lane; i < nc; i += 32) same = same && same_tet(ld_tet<W::kLocal>(c.tets, w.cl[i]), w.cr[i]);
 #pragma unroll 1
     for (int i = lane; i < na; i += 32) {
       const uint32_t a = w.al[i];
-      same = same && same_v(__ldcg(reinterpret_cast<const uint4*>(c.tets + a)), w.av[i]);
+      same = same && same_v(ld_mesh<W::kLocal>(reinterpret_cast<const uint4*>(c.tets + a)), w.av[i]);
     }
     // which facet of each outside tetrahedron faces the cavity (it is locked: this stays true)
 #pragma unroll 1
     for (int i = lane; i < nb; i += 32) {
       const int ci = w.bl_ci[i], f = w.bl_f[i] & 3;
       const uint32_t u = get4(w.cr[ci].n, f);
-      const int back = back_facet(__ldcg(reinterpret_cast<const uint4*>(&c.tets[u].n)), w.cl[ci]);
+      const int back = back_facet(ld_mesh<W::kLocal>(reinterpret_cast<const uint4*>(&c.tets[u].n)), w.cl[ci]);
       same = same && back >= 0;
       w.bl_f[i] = (uint8_t)(f | ((back & 3) << 2));
     }
@@ -883,8 +927,8 @@ __device__ __forceinline__ int try_insert(const Ctx& c, W& w, uint32_t* lock, ui
       set4(n4, cc, w.slot[ec >> 2]);
       const uint32_t s = w.slot[i];
       uint4* dst = reinterpret_cast<uint4*>(c.tets + s);
-      __stcg(dst, v);
-      __stcg(dst + 1, n4);
+      st_mesh<W::kLocal>(dst, v);
+      st_mesh<W::kLocal>(dst + 1, n4);
       if constexpr (W::kCache) {
         float4 q0 = make_float4(0.f, 0.f, 0.f, 0.f), q1 = q0;  // a ghost's entry stays invalid
         if (ghost_pos(v) < 0)
@@ -895,7 +939,7 @@ __device__ __forceinline__ int try_insert(const Ctx& c, W& w, uint32_t* lock, ui
       if constexpr (!W::kCache && (kExact || !W::kTable)) {  // no cache kept here: the entry it replaces is void
         if (c.subdet) __stcg(c.subdet + 2 * (size_t)s + 1, make_float4(0.f, 0.f, 0.f, 0.f));
       }
-      __stcg(reinterpret_cast<uint32_t*>(&c.tets[out].n) + back, s);
+      st_mesh<W::kLocal>(reinterpret_cast<uint32_t*>(&c.tets[out].n) + back, s);
     }
     if (__any_sync(kFull, bad)) {
       if (lane == 0) raise_error(c.st, kErrInternal, 0xA8u);
@@ -909,11 +953,11 @@ __device__ __forceinline__ int try_insert(const Ctx& c, W& w, uint32_t* lock, ui
 #pragma unroll 1
       for (int i = lane; i < freed; i += 32) {
         uint4* dst = reinterpret_cast<uint4*>(c.tets + w.cl[nb + i]);
-        __stcg(dst, make_uint4(kDeadMark, kDeadMark, kDeadMark, kDeadMark));
-        __stcg(dst + 1, make_uint4(redirect, kNone, kNone, kNone));
+        st_mesh<W::kLocal>(dst, make_uint4(kDeadMark, kDeadMark, kDeadMark, kDeadMark));
+        st_mesh<W::kLocal>(dst + 1, make_uint4(redirect, kNone, kNone, kNone));
       }
     }
-    __threadfence();
+    fence_mesh<W::kLocal>();
     release_all(w, lock, held, heldx, nc, na, nx0);
     if (freed > 0) pool_give(c, w, w.cl + nb, freed);
     if (lane == 0) {
@@ -1049,7 +1093,7 @@ __device__ __forceinline__ void run_segment(const Ctx& c, const AsyncIO& io, W& 
     int r = try_insert<kExact>(c, w, lock, p, lg, follows && io.ball_start != 0, start);
     if constexpr (W::kTable) {
       if (r == kABig)
-        r = try_insert_large<kExact>(c, static_cast<LargeWST<W::kCache>*>(io.big_ws), io.big_busy, io.big_n, w, lock, me, p,
+        r = try_insert_large<kExact>(c, static_cast<LargeWST<W::kCache, W::kLocal>*>(io.big_ws), io.big_busy, io.big_n, w, lock, me, p,
                                      lg);
     }
     // a raised error stops the launch; read every 16 points for the same reason as the anchor

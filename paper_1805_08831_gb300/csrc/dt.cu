@@ -25,6 +25,7 @@ constexpr uint32_t kAsyncWalk = 4096;          // walk steps per attempt of the 
 constexpr uint32_t kAsyncBigWarps = 64;        // warps (workspaces) of a large-cavity launch
 constexpr uint32_t kBatchBigWarps = 16;        // warps (workspaces) of a batch's largest cavities
 constexpr double kSmallMeshWarps = 300;        // warps up to which a small mesh gets more than alpha allows
+constexpr uint64_t kLocalMesh = 200;           // vertices up to which a launch is one block
 constexpr uint64_t kDrainPoints = 8;           // points per warp of a list without a wave
 constexpr uint32_t kAsyncBorrow = 512;         // large-cavity workspaces the main kernel's warps may borrow
 constexpr uint64_t kLongWalkBelow = 8192;      // retry lists shorter than this walk up to
@@ -1427,6 +1428,9 @@ int run_pass_async(dt_handle* h, const Ctx& c, const uint32_t* q, uint64_t m, co
   if (m == 0) W = std::min<uint64_t>(W, (carry_n + kDrainPoints - 1) / kDrainPoints);
   if (exact) W = std::min<uint64_t>(W, (uint64_t)async_max_warps_exact());
   W = std::min<uint64_t>(W, std::max(m, carry_n));
+  const uint64_t lw = async_local_warps();
+  const bool local = mesh <= kLocalMesh && lw > 0 && !h->use_subdet && !(h->wcost_ready && h->cfg.schedule == DT_SCHED_LEARNED);
+  if (local) W = std::min(W, lw);
   const uint64_t L = (m + W - 1) / W;
   if (m >= carry_n) W = (m + L - 1) / L;
   int rc = DT_OK;
@@ -1451,7 +1455,7 @@ int run_pass_async(dt_handle* h, const Ctx& c, const uint32_t* q, uint64_t m, co
   if ((rc = reserve_borrow(h)) != DT_OK) return rc;
   AsyncIO io{q, nullptr, m, L, (uint32_t)W, h->cfg.max_walk_steps ? h->cfg.max_walk_steps : kAsyncWalk,
              carry, carry_n, carry_q, h->queue[out], out, h->queue[kQBig], kQBig, h->queue[kQExact], kQExact,
-             exact ? 1 : 0, seg_bounds, h->async_borrow_ws, h->async_borrow_busy, kAsyncBorrow, h->async_ball_start};
+             exact ? 1 : 0, local ? 1 : 0, seg_bounds, h->async_borrow_ws, h->async_borrow_busy, kAsyncBorrow, h->async_ball_start};
   const bool prof = (h->cfg.flags & DT_FLAG_PROFILE) != 0;
   if (prof) cudaEventRecord(h->ev[3], h->stream);
   if ((rc = async_launch(c, io, h->lock, make_log(h), h->stream)) != DT_OK) return rc;

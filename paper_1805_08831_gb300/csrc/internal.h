@@ -150,6 +150,7 @@ struct AsyncIO {
   uint32_t* exact_out;  // predicates the FP32 stage cannot decide: for a launch with exact set
   int exact_q;
   int exact;            // 1: the kernel with the FP64 and exact predicate stages
+  int local;            // 1: one block (W <= async_local_warps()), the mesh through its L1
   const uint32_t* bounds;  // W + 1 segment starts (learned schedule), or null: equal segments of L
   void* big_ws;         // global-memory workspaces a warp may borrow for a large cavity (or null)
   unsigned int* big_busy;  // one word per workspace: 0 free, 1 borrowed
@@ -163,6 +164,7 @@ int async_launch(const Ctx& c, const AsyncIO& io, uint32_t* lock, const InsertLo
 // the current device at once.
 int async_max_warps();
 int async_max_warps_exact();
+uint32_t async_local_warps();  // most warps of a launch with AsyncIO::local set (0: none)
 size_t async_borrow_ws_bytes();  // one workspace of AsyncIO::big_ws
 // The same insertion of the carried points for cavities beyond those workspaces: io.W warps with
 // one global-memory workspace of async_big_ws_bytes() each at ws (device). Points whose cavities
