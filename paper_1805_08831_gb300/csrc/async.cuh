@@ -329,7 +329,10 @@ static __device__ __noinline__ int ghost_exact_at(const Pt* pts, DevState* st, c
 // vertex i), and the walk leaves through the first facet p sees, in an order that turns with
 // the steps. A record that is being rewritten may be read half old, half new: such reads end
 // the walk with kARestart (or it runs into its step bound); nothing is trusted before step 4
-// re-reads it under a lock. Called by the whole warp; the result is uniform. *n_out: the
+// re-reads it under a lock. Called by the whole warp; the result is uniform: every lane reads the
+// record, and while another warp rewrites it the lanes of one load may see it before and after, so
+// each decision is a vote or one lane's. (Branching on each lane's own copy let a warp fall apart,
+// once in some hundred calls on small clouds: a lost point, or an allocator in disorder.) *n_out: the
 // neighbours of the tetrahedron reached.
 template <bool kExact, bool kLocal>
 __device__ __forceinline__ int walk_async(const Ctx& c, uint32_t p, const PtF& FP, uint32_t start, uint32_t salt,
@@ -343,23 +346,24 @@ __device__ __forceinline__ int walk_async(const Ctx& c, uint32_t p, const PtF& F
 #pragma unroll 1
   for (;;) {
     if (t < c.tbase || t >= c.ntets) t = __ldcg(&c.st->anchor);
+    t = __shfl_sync(kFull, t, 0);
     if (t >= c.ntets) return kARestart;
     T = ld_tet<kLocal>(c.tets, t);
-    if (!tet_dead(T.v)) break;
-    t = T.n.x;  // dead slot: follow its redirect
+    if (__all_sync(kFull, !tet_dead(T.v))) break;
+    t = __shfl_sync(kFull, T.n.x, 0);  // dead slot: follow its redirect
     if (++hops > 64) return kARestart;
   }
-  if (!rec_ok(T, c.ntets, c.npts)) return kARestart;
-  int g = ghost_pos(T.v);
-  if (g >= 0) {
-    t = get4(T.n, g);
+  if (!__all_sync(kFull, rec_ok(T, c.ntets, c.npts))) return kARestart;
+  const int g = ghost_pos(T.v);
+  if (__any_sync(kFull, g >= 0)) {
+    t = __shfl_sync(kFull, get4(T.n, g), 0);
     T = ld_tet<kLocal>(c.tets, t);
-    if (tet_dead(T.v) || !rec_ok(T, c.ntets, c.npts)) return kARestart;
+    if (!__all_sync(kFull, !tet_dead(T.v) && rec_ok(T, c.ntets, c.npts))) return kARestart;
   }
   uint32_t prev = kNone, steps = 0;
 #pragma unroll 1
   for (;;) {
-    if (ghost_pos(T.v) >= 0) break;
+    if (__any_sync(kFull, ghost_pos(T.v) >= 0)) break;
     // lane i < 4: orientation of p against the facet opposite vertex i (0: undecided)
     int o = 1;
     const uint32_t nb = lane < 4 ? get4(T.n, lane) : prev;
@@ -402,10 +406,10 @@ __device__ __forceinline__ int walk_async(const Ctx& c, uint32_t p, const PtF& F
     const unsigned rot = ((sees | (sees << 4)) >> ((salt + steps) & 3)) & 0xFu;
     const int exit = (__ffs(rot) - 1 + (int)((salt + steps) & 3)) & 3;
     prev = t;
-    t = get4(T.n, exit);
+    t = __shfl_sync(kFull, get4(T.n, exit), exit);
     T = ld_tet<kLocal>(c.tets, t);
     ++steps;
-    if (tet_dead(T.v) || !rec_ok(T, c.ntets, c.npts)) {
+    if (!__all_sync(kFull, !tet_dead(T.v) && rec_ok(T, c.ntets, c.npts))) {
       *t_out = t;
       *steps_out = steps;
       return kARestart;
