@@ -86,7 +86,7 @@ struct OrderWS {
   uint64_t hist_cap = 0;
   double* bbox = nullptr;        // [6] lo xyz, hi xyz
   double* partial = nullptr;     // per-block bbox partials
-  unsigned int* bad = nullptr;   // non-finite or out-of-range coordinate seen
+  unsigned int* bad = nullptr;   // [2] non-finite or out-of-range coordinate seen; long run of ties
 };
 
 cudaError_t order_ws_reserve(OrderWS& ws, uint64_t n);
