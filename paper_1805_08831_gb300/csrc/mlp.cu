@@ -7,6 +7,7 @@
 // conflict at least once. Loss of one sample with targets (y0, y1):
 //   (out[0] - y0)^2 + softplus(out[1]) - y1 * out[1]      (squared error + binary cross-entropy)
 // averaged over the samples.
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -14,6 +15,8 @@
 #include <cstdint>
 
 #include "internal.h"
+
+namespace cg = cooperative_groups;
 
 namespace dtg {
 namespace {
@@ -76,15 +79,19 @@ __global__ void __launch_bounds__(kMlpThreads) k_mlp_forward(const float* __rest
 //
 // A block takes tiles of 32 samples and runs the layers as small matrix products in shared
 // memory, lane = hidden unit: forward, then backward, the products over the samples (the
-// weights' gradients) accumulated in registers over all of a block's tiles, so that each block
-// adds every gradient entry to global memory once. What bounds a training step is latency (one
-// launch, one gather of random rows, the layers' chain, one round of atomics): a minibatch of
-// 4096 takes 33 MFLOP. Adding every sample's 1410 products to one shared copy with atomics, as a
-// thread per sample, serialised the lanes on one address each and took 1.3 ms a step.
-constexpr int kS = 32;  // samples per tile
+// weights' gradients) accumulated in registers over all of a block's tiles. The eight blocks of a
+// cluster then add up their parts through shared memory, so that a minibatch of 4096 adds 16
+// terms to an entry in global memory, not 128: a longer chain rounds more (the loss of one step
+// was off by 2.9e-7 instead of 0.6e-7; with a shared copy per block 0.7e-7). What bounds a training
+// step is latency (one launch, one gather of random rows, the layers' chain, one round of
+// atomics; 0.02 ms): a minibatch of 4096 takes 33 MFLOP. Adding every sample's 1410 products to
+// one shared copy with atomics, as a thread per sample, serialised the lanes on one address each
+// and took 1.3 ms a step.
+constexpr int kS = 32;       // samples per tile
+constexpr int kCluster = 8;  // blocks that add up their parts before they go to global memory
 
 template <bool kDraw>
-__global__ void __launch_bounds__(kMlpThreads) k_mlp_step(float* params, const float* __restrict__ x,
+__global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kMlpThreads) k_mlp_step(float* params, const float* __restrict__ x,
                                                           const float* __restrict__ y, uint64_t n, uint64_t rows,
                                                           uint64_t draw_seed, float scale, float* grad, float* loss,
                                                           unsigned int* ticket, float* m, float* v, float lr, int t) {
@@ -93,6 +100,7 @@ __global__ void __launch_bounds__(kMlpThreads) k_mlp_step(float* params, const f
   __shared__ uint64_t row[kS];
   __shared__ unsigned int s_last;
   constexpr int kWarps = kMlpThreads / 32;
+  __shared__ float G[kParams + 1], s_sum[kWarps];
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   for (int i = tid; i < kIn * kH; i += kMlpThreads) W1[i / kH][i % kH] = __ldcg(&params[kOffW1 + i]);
   for (int i = tid; i < kH * kH; i += kMlpThreads) W2[i / kH][i % kH] = __ldcg(&params[kOffW2 + i]);
@@ -120,19 +128,30 @@ __global__ void __launch_bounds__(kMlpThreads) k_mlp_step(float* params, const f
       if (tid < kS * kOut) Y[tid / kOut][tid % kOut] = tid / kOut < ns ? y[row[tid / kOut] * kOut + tid % kOut] : 0.f;
     }
     __syncthreads();
-    for (int s = wid; s < kS; s += kWarps) {
+    // a warp's four samples go through a layer together: four independent sums per weight read
+    constexpr int kPer = kS / kWarps;
+    float h[kPer];
+#pragma unroll
+    for (int q = 0; q < kPer; ++q) {
       float a = B[lane];
-      for (int i = 0; i < kIn; ++i) a = fmaf(X[s][i], W1[i][lane], a);
-      H1[s][lane] = fmaxf(a, 0.f);
+      for (int i = 0; i < kIn; ++i) a = fmaf(X[wid + kWarps * q][i], W1[i][lane], a);
+      H1[wid + kWarps * q][lane] = fmaxf(a, 0.f);
     }
     __syncwarp();  // a sample stays with its warp until the products over the samples
-    for (int s = wid; s < kS; s += kWarps) {
-      float a = B[kH + lane];
+#pragma unroll
+    for (int q = 0; q < kPer; ++q) h[q] = B[kH + lane];
 #pragma unroll 8
-      for (int i = 0; i < kH; ++i) a = fmaf(H1[s][i], W2[i][lane], a);
-      const float h = fmaxf(a, 0.f);
-      H2[s][lane] = h;
-      float o0 = h * W3[lane][0], o1 = h * W3[lane][1];
+    for (int i = 0; i < kH; ++i) {
+      const float wt = W2[i][lane];
+#pragma unroll
+      for (int q = 0; q < kPer; ++q) h[q] = fmaf(H1[wid + kWarps * q][i], wt, h[q]);
+    }
+#pragma unroll
+    for (int q = 0; q < kPer; ++q) {
+      const int s = wid + kWarps * q;
+      h[q] = fmaxf(h[q], 0.f);
+      H2[s][lane] = h[q];
+      float o0 = h[q] * W3[lane][0], o1 = h[q] * W3[lane][1];
       for (int d = 16; d > 0; d >>= 1) {
         o0 += __shfl_xor_sync(0xFFFFFFFFu, o0, d);
         o1 += __shfl_xor_sync(0xFFFFFFFFu, o1, d);
@@ -143,15 +162,20 @@ __global__ void __launch_bounds__(kMlpThreads) k_mlp_step(float* params, const f
       if (lane == 0 && s < ns) sum += scale * (e * e + softplus(o1) - y1 * o1);
       const float d0 = s < ns ? 2.f * e * scale : 0.f, d1 = s < ns ? (sigmoid(o1) - y1) * scale : 0.f;
       if (lane < kOut) D3[s][lane] = lane == 0 ? d0 : d1;
-      D2[s][lane] = h > 0.f ? d0 * W3[lane][0] + d1 * W3[lane][1] : 0.f;
+      D2[s][lane] = h[q] > 0.f ? d0 * W3[lane][0] + d1 * W3[lane][1] : 0.f;
     }
     __syncwarp();
-    for (int s = wid; s < kS; s += kWarps) {
-      float a = 0.f;
+#pragma unroll
+    for (int q = 0; q < kPer; ++q) h[q] = 0.f;
 #pragma unroll 8
-      for (int j = 0; j < kH; ++j) a = fmaf(D2[s][j], W2[lane][j], a);
-      D1[s][lane] = H1[s][lane] > 0.f ? a : 0.f;
+    for (int j = 0; j < kH; ++j) {
+      const float wt = W2[lane][j];
+#pragma unroll
+      for (int q = 0; q < kPer; ++q) h[q] = fmaf(D2[wid + kWarps * q][j], wt, h[q]);
     }
+#pragma unroll
+    for (int q = 0; q < kPer; ++q)
+      D1[wid + kWarps * q][lane] = H1[wid + kWarps * q][lane] > 0.f ? h[q] : 0.f;
     __syncthreads();
 #pragma unroll 4
     for (int s = 0; s < kS; ++s) {  // a unit without a gradient takes no part, whatever its input
@@ -168,17 +192,32 @@ __global__ void __launch_bounds__(kMlpThreads) k_mlp_step(float* params, const f
     else if (tid < kH * kOut + 2 * kH + kOut)
       for (int s = 0; s < kS; ++s) gb3 += D3[s][lane];
   }
-  for (int k = 0; k < kH / kWarps; ++k) atomicAdd(&grad[kOffW2 + (wid + kWarps * k) * kH + lane], g2[k]);
-  atomicAdd(&grad[kOffW1 + wid * kH + lane], g1);
-  if (tid < kH * kOut) atomicAdd(&grad[kOffW3 + tid], g3);
-  else if (tid < kH * kOut + kH) atomicAdd(&grad[kOffB1 + lane], gb1);
-  else if (tid < kH * kOut + 2 * kH) atomicAdd(&grad[kOffB2 + lane], gb2);
-  else if (tid < kH * kOut + 2 * kH + kOut) atomicAdd(&grad[kOffB3 + lane], gb3);
-  if (lane == 0) atomicAdd(loss, sum);
+  // the cluster's blocks add up their parts, an eighth of the entries each
+  for (int k = 0; k < kH / kWarps; ++k) G[kOffW2 + (wid + kWarps * k) * kH + lane] = g2[k];
+  G[kOffW1 + wid * kH + lane] = g1;
+  if (tid < kH * kOut) G[kOffW3 + tid] = g3;
+  else if (tid < kH * kOut + kH) G[kOffB1 + lane] = gb1;
+  else if (tid < kH * kOut + 2 * kH) G[kOffB2 + lane] = gb2;
+  else if (tid < kH * kOut + 2 * kH + kOut) G[kOffB3 + lane] = gb3;
+  if (lane == 0) s_sum[wid] = sum;
+  __syncthreads();
+  if (tid == 0) {
+    float l = 0.f;
+    for (int k = 0; k < kWarps; ++k) l += s_sum[k];
+    G[kParams] = l;
+  }
+  cg::cluster_group cluster = cg::this_cluster();
+  cluster.sync();
+  for (int i = (int)cluster.block_rank() + kCluster * tid; i <= kParams; i += kCluster * kMlpThreads) {
+    float part[kCluster], a = 0.f;
+    for (int r = 0; r < kCluster; ++r) part[r] = cluster.map_shared_rank(G, r)[i];
+    for (int r = 0; r < kCluster; ++r) a += part[r];
+    atomicAdd(i < kParams ? &grad[i] : loss, a);
+  }
+  if constexpr (kDraw) __threadfence();
+  cluster.sync();  // every block's part has been read, and this block's sums are on their way
   if constexpr (kDraw) {
     // the last block to add its part holds the whole gradient
-    __threadfence();
-    __syncthreads();
     if (tid == 0) s_last = atomicAdd(ticket, 1u) == gridDim.x - 1 ? 1u : 0u;
     __syncthreads();
     if (!s_last) return;
@@ -197,9 +236,11 @@ __global__ void __launch_bounds__(kMlpThreads) k_mlp_step(float* params, const f
   }
 }
 
-// Blocks of a step: one tile each while that fills the chip, then tiles are taken in turn.
+// Blocks of a step: one tile each while that fills the chip, then tiles are taken in turn; whole
+// clusters.
 unsigned step_grid(uint64_t n) {
-  return (unsigned)std::max<uint64_t>(1, std::min<uint64_t>((n + kS - 1) / kS, 152ull * 4));
+  const uint64_t b = std::max<uint64_t>(1, std::min<uint64_t>((n + kS - 1) / kS, 152ull * 4));
+  return (unsigned)((b + kCluster - 1) / kCluster * kCluster);
 }
 
 unsigned mlp_grid(uint64_t n) {
