@@ -204,132 +204,122 @@ static __device__ __noinline__ int ex_det3(const Ex2* r0, const Ex2* r1, const E
 // When every coordinate of the points of a predicate is an integer multiple of one power of two
 // 2^E with at most 62 significant bits after scaling (lattice, grid and most clustered inputs),
 // the coordinates divided by 2^E are exact 64-bit integers, and both determinants are exact
-// polynomials in them: sums of products of at most five factors, a 3 x 3 minor (< 2^192) times
-// a squared length (< 2^128). They are evaluated in two's-complement arithmetic on 64-bit limbs
-// (4 limbs for orient3d, 6 for insphere) on the integer pipes, which GB300 runs far faster than
-// its FP64 pipe. Subnormal coordinates or exponents spread over more than about 9 bits keep the
-// expansion arithmetic below.
-struct IntCoord {
-  uint64_t mag;  // odd significand (0 for a zero coordinate)
-  int lo;        // exponent of its lowest bit
-  int bits;      // significant bits
-  bool neg;
+// polynomials in them: sums of products of at most five factors, a 3 x 3 minor (< 2^191) times
+// a squared length (< 2^128). They are evaluated in two's complement (192 bits for orient3d, 384
+// for insphere) on the integer pipes, which GB300 runs far faster than its FP64 pipe. Subnormal
+// coordinates or exponents spread over more than about 9 bits keep the expansion arithmetic below.
+// What bounds it is its length, in warps that have few lanes in it: so the code is straight-line
+// (the 3 x 3 minors share the 2 x 2 ones, no branch on signs or zeros, no arrays in local memory),
+// 72 products of 64 bits for an insphere. Terms formed one by one as sign and magnitude, with
+// loops over limbs, took 130 instead of 115 ms for the degenerate mix of 1e6 points, and 89 instead
+// of 79 ms for a box surface of 48 intervals and its refinement. Run before the FP64 filter it is
+// no faster (111 and 79 ms, but more calls on inputs that the filter decides).
+using u128 = unsigned __int128;
+using s128 = __int128;
+
+// The n coordinates as integers of one common power of two: false if one needs more than 62 bits,
+// or is subnormal, infinite or NaN.
+template <int n>
+__device__ __forceinline__ bool int_scale(const double* x, long long* X) {
+  int E = 1 << 20, top = -(1 << 20);  // exponents of the lowest bit and beyond the highest
+  bool ok = true;
+#pragma unroll
+  for (int i = 0; i < n; ++i) {
+    const uint64_t b = (uint64_t)__double_as_longlong(x[i]), m = b & 0xFFFFFFFFFFFFFull;
+    const int ex = (int)((b >> 52) & 0x7FF);
+    const bool zero = (b << 1) == 0;
+    ok = ok && (zero || (ex != 0 && ex != 0x7FF));
+    const int tz = m ? __ffsll((long long)m) - 1 : 52;
+    if (!zero) {
+      E = min(E, ex - 1075 + tz);
+      top = max(top, ex - 1022);
+    }
+  }
+  if (!ok || (top > E && top - E > 62)) return false;
+#pragma unroll
+  for (int i = 0; i < n; ++i) {
+    const uint64_t b = (uint64_t)__double_as_longlong(x[i]), m = (b & 0xFFFFFFFFFFFFFull) | (1ull << 52);
+    const int sh = (int)((b >> 52) & 0x7FF) - 1075 - E;  // -52 .. 9
+    const long long v = (b << 1) == 0 ? 0 : (long long)(sh >= 0 ? m << sh : m >> -sh);
+    X[i] = (b >> 63) ? -v : v;
+  }
+  return true;
+}
+
+struct S192 {  // lo + 2^64 hi, hi in two's complement
+  uint64_t lo;
+  u128 hi;
 };
 
-__device__ __forceinline__ bool int_coord(double x, IntCoord& c) {
-  const uint64_t b = (uint64_t)__double_as_longlong(x);
-  const int ex = (int)((b >> 52) & 0x7FF);
-  uint64_t m = b & 0xFFFFFFFFFFFFFull;
-  c.neg = (b >> 63) != 0;
-  if (ex == 0 && m == 0) {
-    c.mag = 0;
-    c.lo = 0x7FFFFFFF;
-    c.bits = 0;
-    return true;
-  }
-  if (ex == 0 || ex == 0x7FF) return false;  // subnormal, infinite or NaN
-  m |= 1ull << 52;
-  const int tz = __ffsll((long long)m) - 1;
-  c.mag = m >> tz;
-  c.lo = ex - 1075 + tz;
-  c.bits = 64 - __clzll((long long)c.mag);
-  return true;
+__device__ __forceinline__ S192 mul192(s128 m, long long z) {
+  const uint64_t ml = (uint64_t)m;
+  const u128 p = (u128)ml * (uint64_t)z;
+  S192 r;
+  r.lo = (uint64_t)p;
+  r.hi = (u128)((s128)(long long)(m >> 64) * z) + (uint64_t)(p >> 64) - (z < 0 ? ml : 0ull);
+  return r;
 }
 
-// The n coordinates as integers of one common power of two (false if one needs > 62 bits).
-__device__ __forceinline__ bool int_scale(const IntCoord* c, int n, long long* X) {
-  int E = 0x7FFFFFFF;
-  for (int i = 0; i < n; ++i) E = min(E, c[i].lo);
-  for (int i = 0; i < n; ++i) {
-    if (c[i].mag == 0) {
-      X[i] = 0;
-      continue;
-    }
-    const int sh = c[i].lo - E;
-    if (sh > 62 || c[i].bits + sh > 62) return false;
-    const long long v = (long long)(c[i].mag << sh);
-    X[i] = c[i].neg ? -v : v;
-  }
-  return true;
+__device__ __forceinline__ S192 add192(const S192& a, const S192& b) {
+  S192 r;
+  r.lo = a.lo + b.lo;
+  r.hi = a.hi + b.hi + (r.lo < a.lo ? 1u : 0u);
+  return r;
 }
 
-// acc (N limbs, two's complement) += m or -= m (m: an nm-limb magnitude).
-template <int N>
-__device__ __forceinline__ void wide_add(uint64_t* acc, const uint64_t* m, int nm, bool sub) {
-  uint64_t c = 0;
-  for (int i = 0; i < N; ++i) {
-    const uint64_t mi = i < nm ? m[i] : 0ull;
-    if (!sub) {
-      const uint64_t s = acc[i] + mi;
-      const uint64_t c1 = s < mi;
-      const uint64_t s2 = s + c;
-      c = c1 | (s2 < c);
-      acc[i] = s2;
-    } else {
-      const uint64_t dd = acc[i] - mi;
-      const uint64_t b1 = acc[i] < mi;
-      const uint64_t d2 = dd - c;
-      c = b1 | (dd < c);
-      acc[i] = d2;
-    }
-  }
+__device__ __forceinline__ S192 sub192(const S192& a, const S192& b) {
+  S192 r;
+  r.lo = a.lo - b.lo;
+  r.hi = a.hi - b.hi - (a.lo < b.lo ? 1u : 0u);
+  return r;
 }
 
-// out[0 .. nm] = m[0 .. nm) * v (magnitudes).
-__device__ __forceinline__ void mag_mul1(const uint64_t* m, int nm, uint64_t v, uint64_t* out) {
-  uint64_t carry = 0;
-  for (int i = 0; i < nm; ++i) {
-    uint64_t lo = m[i] * v;
-    uint64_t hi = __umul64hi(m[i], v);
-    lo += carry;
-    hi += (lo < carry);
-    out[i] = lo;
-    carry = hi;
-  }
-  out[nm] = carry;
+// The 2 x 2 minor of u and v in x and y; the 3 x 3 determinant from its rows' third coordinates
+// and their minors. Entries below 2^63 in magnitude: minors below 2^127, determinants (at most 4
+// times the entries' product) below 2^191, so both fit, and sums may wrap on the way.
+__device__ __forceinline__ s128 int_minor(const long long* u, const long long* v) {
+  return (s128)((u128)((s128)u[0] * v[1]) - (u128)((s128)u[1] * v[0]));
+}
+__device__ __forceinline__ S192 int_det3(long long za, long long zb, long long zc, s128 ab, s128 ac, s128 bc) {
+  return add192(sub192(mul192(bc, za), mul192(ac, zb)), mul192(ab, zc));
 }
 
-__device__ __forceinline__ uint64_t mag64(long long x) { return x < 0 ? (uint64_t)(-x) : (uint64_t)x; }
-
-// det[u; v; w] of integer rows into a 4-limb two's-complement accumulator.
-__device__ __forceinline__ void int_det3(const long long* u, const long long* v, const long long* w, uint64_t* acc) {
-  for (int i = 0; i < 4; ++i) acc[i] = 0;
-  const long long t[6][3] = {{u[0], v[1], w[2]}, {u[0], v[2], w[1]}, {u[1], v[0], w[2]},
-                             {u[1], v[2], w[0]}, {u[2], v[0], w[1]}, {u[2], v[1], w[0]}};
-  const bool minus[6] = {false, true, true, false, false, true};
-  for (int k = 0; k < 6; ++k) {
-    const long long a = t[k][0], b = t[k][1], c = t[k][2];
-    if (a == 0 || b == 0 || c == 0) continue;
-    const bool neg = minus[k] ^ (a < 0) ^ (b < 0) ^ (c < 0);
-    const uint64_t ab[2] = {mag64(a) * mag64(b), __umul64hi(mag64(a), mag64(b))};
-    uint64_t abc[3];
-    mag_mul1(ab, 2, mag64(c), abc);
-    wide_add<4>(acc, abc, 3, neg);
+// acc[K .. 6) += M * l.
+template <int K>
+__device__ __forceinline__ void mul_add(uint64_t* acc, const S192& M, uint64_t l) {
+  const uint64_t m1 = (uint64_t)M.hi, m2 = (uint64_t)(M.hi >> 64);
+  u128 c = (u128)M.lo * l;
+  uint64_t t[6];
+  t[0] = (uint64_t)c;
+  c = (u128)m1 * l + (uint64_t)(c >> 64);
+  t[1] = (uint64_t)c;
+  c = (u128)m2 * l + (uint64_t)(c >> 64);
+  t[2] = (uint64_t)c;
+  t[3] = (uint64_t)(c >> 64) - ((long long)m2 < 0 ? l : 0ull);
+  // l * M's sign: the value is below 2^255, so t[3] carries it
+  t[4] = t[5] = (uint64_t)((long long)t[3] >> 63);
+  c = 0;
+#pragma unroll
+  for (int i = K; i < 6; ++i) {
+    c += (u128)acc[i] + t[i - K];
+    acc[i] = (uint64_t)c;
+    c >>= 64;
   }
-}
-
-template <int N>
-__device__ __forceinline__ int wide_sign(const uint64_t* acc) {
-  if (acc[N - 1] >> 63) return -1;
-  for (int i = 0; i < N; ++i)
-    if (acc[i]) return 1;
-  return 0;
 }
 
 // Exact orient3d in integers: true (and *s) when the coordinates fit.
 __device__ __forceinline__ bool orient3d_int(const Pt& a, const Pt& b, const Pt& c, const Pt& d, int* s) {
   const double v[12] = {a.x, a.y, a.z, b.x, b.y, b.z, c.x, c.y, c.z, d.x, d.y, d.z};
-  IntCoord ic[12];
-  for (int i = 0; i < 12; ++i)
-    if (!int_coord(v[i], ic[i])) return false;
   long long X[12];
-  if (!int_scale(ic, 12, X)) return false;
+  if (!int_scale<12>(v, X)) return false;
   long long r[3][3];
+#pragma unroll
   for (int i = 0; i < 3; ++i)
+#pragma unroll
     for (int k = 0; k < 3; ++k) r[i][k] = X[3 * (i + 1) + k] - X[k];
-  uint64_t acc[4];
-  int_det3(r[0], r[1], r[2], acc);
-  *s = wide_sign<4>(acc);
+  const S192 M =
+      int_det3(r[0][2], r[1][2], r[2][2], int_minor(r[0], r[1]), int_minor(r[0], r[2]), int_minor(r[1], r[2]));
+  *s = (s128)M.hi < 0 ? -1 : (M.lo != 0 || M.hi != 0) ? 1 : 0;
   return true;
 }
 
@@ -338,47 +328,38 @@ __device__ __forceinline__ bool orient3d_int(const Pt& a, const Pt& b, const Pt&
 __device__ __forceinline__ bool insphere_int(const Pt& a, const Pt& b, const Pt& c, const Pt& d, const Pt& e,
                                              int* s) {
   const double v[15] = {a.x, a.y, a.z, b.x, b.y, b.z, c.x, c.y, c.z, d.x, d.y, d.z, e.x, e.y, e.z};
-  IntCoord ic[15];
-  for (int i = 0; i < 15; ++i)
-    if (!int_coord(v[i], ic[i])) return false;
   long long X[15];
-  if (!int_scale(ic, 15, X)) return false;
+  if (!int_scale<15>(v, X)) return false;
   long long D[4][3];
-  uint64_t L[4][2];
+  u128 L[4];  // squared lengths: < 3 * 2^126
+#pragma unroll
   for (int i = 0; i < 4; ++i) {
-    L[i][0] = L[i][1] = 0;
+    L[i] = 0;
+#pragma unroll
     for (int k = 0; k < 3; ++k) {
       D[i][k] = X[3 * (i + 1) + k] - X[k];
-      const uint64_t m = mag64(D[i][k]);
-      const uint64_t sq[2] = {m * m, __umul64hi(m, m)};
-      wide_add<2>(L[i], sq, 2, false);  // < 3 * 2^126: no carry out of two limbs
+      L[i] += (u128)((s128)D[i][k] * D[i][k]);
     }
   }
+  const s128 m01 = int_minor(D[0], D[1]), m02 = int_minor(D[0], D[2]), m03 = int_minor(D[0], D[3]),
+             m12 = int_minor(D[1], D[2]), m13 = int_minor(D[1], D[3]), m23 = int_minor(D[2], D[3]);
+  const S192 zero = {0, 0};
   uint64_t acc[6] = {0, 0, 0, 0, 0, 0};
-  for (int k = 0; k < 4; ++k) {
-    int r[3], j = 0;
-    for (int i = 0; i < 4; ++i)
-      if (i != k) r[j++] = i;
-    uint64_t M[4];
-    int_det3(D[r[0]], D[r[1]], D[r[2]], M);
-    const int sm = wide_sign<4>(M);
-    if (sm == 0 || (L[k][0] | L[k][1]) == 0) continue;
-    if (sm < 0) {  // magnitude of M
-      for (int i = 0; i < 4; ++i) M[i] = ~M[i];
-      const uint64_t one = 1;
-      wide_add<4>(M, &one, 1, false);
-    }
-    uint64_t p0[5], p1[5], prod[6];
-    mag_mul1(M, 4, L[k][0], p0);
-    mag_mul1(M, 4, L[k][1], p1);
-    for (int i = 0; i < 6; ++i) prod[i] = 0;
-    wide_add<6>(prod, p0, 5, false);
-    wide_add<5>(prod + 1, p1, 5, false);
-    // sign of the term: (-1)^(k+1) times the sign of the minor
-    const bool neg = ((k == 0 || k == 2) ? true : false) ^ (sm < 0);
-    wide_add<6>(acc, prod, 6, neg);
-  }
-  *s = wide_sign<6>(acc);
+  // term k: (-1)^(k+1) L_k times the determinant of the other rows
+  S192 M = sub192(zero, int_det3(D[1][2], D[2][2], D[3][2], m12, m13, m23));
+  mul_add<0>(acc, M, (uint64_t)L[0]);
+  mul_add<1>(acc, M, (uint64_t)(L[0] >> 64));
+  M = int_det3(D[0][2], D[2][2], D[3][2], m02, m03, m23);
+  mul_add<0>(acc, M, (uint64_t)L[1]);
+  mul_add<1>(acc, M, (uint64_t)(L[1] >> 64));
+  M = sub192(zero, int_det3(D[0][2], D[1][2], D[3][2], m01, m03, m13));
+  mul_add<0>(acc, M, (uint64_t)L[2]);
+  mul_add<1>(acc, M, (uint64_t)(L[2] >> 64));
+  M = int_det3(D[0][2], D[1][2], D[2][2], m01, m02, m12);
+  mul_add<0>(acc, M, (uint64_t)L[3]);
+  mul_add<1>(acc, M, (uint64_t)(L[3] >> 64));
+  const uint64_t low = acc[0] | acc[1] | acc[2] | acc[3] | acc[4];
+  *s = (acc[5] >> 63) ? -1 : (low | acc[5]) ? 1 : 0;
   return true;
 }
 
