@@ -938,7 +938,7 @@ struct dt_handle {
                                    // retry pass without progress moves the list to the rounds anyway
   uint64_t async_warps = 0;        // cap on the asynchronous engine's warps (0: all that fit)
   uint32_t async_ball_start = 1;   // start from the previous ball's tetrahedra before walking
-  double async_handoff_frac = 0.1;  // hand-offs per point given so far that switch a call to the
+  double async_handoff_frac = 0.03;  // hand-offs per point given so far that switch a call to the
   uint64_t async_handoff_min = 16;  // exact kernels, and the fewest that do
   uint8_t* wcost = nullptr;        // learned schedule: predicted insertion work per vertex
   bool wcost_ready = false;
@@ -1644,8 +1644,12 @@ int run_brio_round(dt_handle* h, uint32_t vbegin, uint32_t vend, int round, uint
 }
 
 // Whether the inputs defeat the asynchronous engine's FP32 stage: once it has handed on more than
-// a tenth of the points it was given (and more than a few), the kernels with the exact stages do
-// the rest of the call. They hold twice the registers, so half the warps are resident.
+// 3 % of the points it was given (and more than a few), the kernels with the exact stages do the
+// rest of the call. They hold twice the registers, so half the warps are resident; but a point
+// handed on is searched for twice, and the list of them, inserted at once, loses often (a
+// degenerate mix hands on 5 to 10 % of each wave). 1e6 points of it take 118 ms with the line at
+// a tenth, 95 at 5 %, 88 at 3 %, 89 at 1.5 % and 86 at 0.7 %; a slab of 1e6, which hands on 0.6 %,
+// takes 29.4 ms down to 1.5 % and 32.7 at 0.7 %; uniform clouds hand on 0.2 %.
 bool handoffs_decide(dt_handle* h, uint64_t given) {
   const uint64_t ne = h->st_host->q[kQExact];
   return ne >= h->async_handoff_min && (double)ne > h->async_handoff_frac * (double)given;
