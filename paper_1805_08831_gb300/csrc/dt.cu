@@ -2078,7 +2078,10 @@ int batch_impl(dt_handle* h, const double* xyz, const uint64_t* off, uint32_t nc
   // slots per cloud: f per point, room for the first tetrahedra and ghosts, and the few dozen slots
   // that each of a launch's warps keeps of its own while it runs
   std::vector<BatchCloud> cl(nc);
-  uint64_t T = 0, hash = 1469598103934665603ull;
+  // No cloud holds slot 0. A record read while it is first written may still have zero neighbours;
+  // with slot 0 in the first cloud, a walk of another cloud went on in that cloud's mesh and
+  // inserted its point there (one batch of 64 small clouds in some 1500). It reads as dead.
+  uint64_t T = 32, hash = 1469598103934665603ull;
   for (uint32_t c = 0; c < nc; ++c) {
     uint64_t n = off[c + 1] - off[c];
     uint64_t cap = (uint64_t)(f * (double)n) + 64 + 64 * std::min<uint64_t>(async_warps_for(h, n), n);
