@@ -208,22 +208,22 @@ static __device__ __noinline__ int ex_det3(const Ex2* r0, const Ex2* r1, const E
 // a squared length (< 2^128). They are evaluated in two's complement (192 bits for orient3d, 384
 // for insphere) on the integer pipes, which GB300 runs far faster than its FP64 pipe. Subnormal
 // coordinates or exponents spread over more than about 9 bits keep the expansion arithmetic below.
-// What bounds it is its length, in warps that have few lanes in it: so the code is straight-line
-// (the 3 x 3 minors share the 2 x 2 ones, no branch on signs or zeros, no arrays in local memory),
-// 72 products of 64 bits for an insphere. Terms formed one by one as sign and magnitude, with
-// loops over limbs, took 130 instead of 115 ms for the degenerate mix of 1e6 points, and 89 instead
-// of 79 ms for a box surface of 48 intervals and its refinement. Run before the FP64 filter it is
-// no faster (111 and 79 ms, but more calls on inputs that the filter decides).
+// What bounds it is the fetch of its instructions, run by few lanes of a warp and seldom enough to
+// be evicted in between: so the code is short (loops over the terms, the determinant of three rows
+// and the scaling out of line, one copy for both predicates), without branches on signs or zeros.
+// The degenerate mix of 1e6 points takes 73 ms, the box surface of 48 intervals with its
+// refinement 74; the same arithmetic unrolled, with shared 2 x 2 minors, 88 and 79 (an insphere
+// took 58,000 cycles); terms formed one by one as sign and magnitude about 100 and 89. Run before
+// the FP64 filter it takes 70 and 82.
 using u128 = unsigned __int128;
 using s128 = __int128;
 
 // The n coordinates as integers of one common power of two: false if one needs more than 62 bits,
 // or is subnormal, infinite or NaN.
-template <int n>
-__device__ __forceinline__ bool int_scale(const double* x, long long* X) {
+static __device__ __noinline__ bool int_scale(const double* x, int n, long long* X) {
   int E = 1 << 20, top = -(1 << 20);  // exponents of the lowest bit and beyond the highest
   bool ok = true;
-#pragma unroll
+#pragma unroll 1
   for (int i = 0; i < n; ++i) {
     const uint64_t b = (uint64_t)__double_as_longlong(x[i]), m = b & 0xFFFFFFFFFFFFFull;
     const int ex = (int)((b >> 52) & 0x7FF);
@@ -236,7 +236,7 @@ __device__ __forceinline__ bool int_scale(const double* x, long long* X) {
     }
   }
   if (!ok || (top > E && top - E > 62)) return false;
-#pragma unroll
+#pragma unroll 1
   for (int i = 0; i < n; ++i) {
     const uint64_t b = (uint64_t)__double_as_longlong(x[i]), m = (b & 0xFFFFFFFFFFFFFull) | (1ull << 52);
     const int sh = (int)((b >> 52) & 0x7FF) - 1075 - E;  // -52 .. 9
@@ -251,58 +251,48 @@ struct S192 {  // lo + 2^64 hi, hi in two's complement
   u128 hi;
 };
 
-__device__ __forceinline__ S192 mul192(s128 m, long long z) {
-  const uint64_t ml = (uint64_t)m;
-  const u128 p = (u128)ml * (uint64_t)z;
-  S192 r;
-  r.lo = (uint64_t)p;
-  r.hi = (u128)((s128)(long long)(m >> 64) * z) + (uint64_t)(p >> 64) - (z < 0 ? ml : 0ull);
+// The determinant of rows k + 1, k + 2, k + 3 (mod rows) of D, along its third column: entries
+// below 2^63 in magnitude, so 2 x 2 minors are below 2^127 and the determinant (at most 4 times
+// the entries' product) below 2^191, and sums may wrap on the way.
+static __device__ __noinline__ S192 int_det3(const long long* D, int k, int rows) {
+  S192 r = {0, 0};
+#pragma unroll 1
+  for (int j = 0; j < 3; ++j) {
+    const int j1 = j == 2 ? 0 : j + 1, j2 = j == 0 ? 2 : j - 1;
+    const long long* z = D + 3 * ((k + 1 + j) % rows) + 2;
+    const long long* u = D + 3 * ((k + 1 + j1) % rows);
+    const long long* v = D + 3 * ((k + 1 + j2) % rows);
+    const s128 m = (s128)((u128)((s128)u[0] * v[1]) - (u128)((s128)u[1] * v[0]));
+    const uint64_t ml = (uint64_t)m;
+    const u128 p = (u128)ml * (uint64_t)*z;
+    r.lo += (uint64_t)p;
+    r.hi += (u128)((s128)(long long)(m >> 64) * *z) + (uint64_t)(p >> 64) - (*z < 0 ? ml : 0ull) +
+            (r.lo < (uint64_t)p ? 1u : 0u);
+  }
   return r;
 }
 
-__device__ __forceinline__ S192 add192(const S192& a, const S192& b) {
-  S192 r;
-  r.lo = a.lo + b.lo;
-  r.hi = a.hi + b.hi + (r.lo < a.lo ? 1u : 0u);
-  return r;
-}
+struct S320 {
+  uint64_t w[5];
+};
 
-__device__ __forceinline__ S192 sub192(const S192& a, const S192& b) {
-  S192 r;
-  r.lo = a.lo - b.lo;
-  r.hi = a.hi - b.hi - (a.lo < b.lo ? 1u : 0u);
-  return r;
-}
-
-// The 2 x 2 minor of u and v in x and y; the 3 x 3 determinant from its rows' third coordinates
-// and their minors. Entries below 2^63 in magnitude: minors below 2^127, determinants (at most 4
-// times the entries' product) below 2^191, so both fit, and sums may wrap on the way.
-__device__ __forceinline__ s128 int_minor(const long long* u, const long long* v) {
-  return (s128)((u128)((s128)u[0] * v[1]) - (u128)((s128)u[1] * v[0]));
-}
-__device__ __forceinline__ S192 int_det3(long long za, long long zb, long long zc, s128 ab, s128 ac, s128 bc) {
-  return add192(sub192(mul192(bc, za), mul192(ac, zb)), mul192(ab, zc));
-}
-
-// acc[K .. 6) += M * l.
-template <int K>
-__device__ __forceinline__ void mul_add(uint64_t* acc, const S192& M, uint64_t l) {
+// acc += M * l.
+__device__ __forceinline__ void mul_add(S320& acc, const S192& M, uint64_t l) {
   const uint64_t m1 = (uint64_t)M.hi, m2 = (uint64_t)(M.hi >> 64);
   u128 c = (u128)M.lo * l;
-  uint64_t t[6];
+  uint64_t t[5];
   t[0] = (uint64_t)c;
   c = (u128)m1 * l + (uint64_t)(c >> 64);
   t[1] = (uint64_t)c;
   c = (u128)m2 * l + (uint64_t)(c >> 64);
   t[2] = (uint64_t)c;
   t[3] = (uint64_t)(c >> 64) - ((long long)m2 < 0 ? l : 0ull);
-  // l * M's sign: the value is below 2^255, so t[3] carries it
-  t[4] = t[5] = (uint64_t)((long long)t[3] >> 63);
+  t[4] = (uint64_t)((long long)t[3] >> 63);  // the product is below 2^255: t[3] carries its sign
   c = 0;
 #pragma unroll
-  for (int i = K; i < 6; ++i) {
-    c += (u128)acc[i] + t[i - K];
-    acc[i] = (uint64_t)c;
+  for (int i = 0; i < 5; ++i) {
+    c += (u128)acc.w[i] + t[i];
+    acc.w[i] = (uint64_t)c;
     c >>= 64;
   }
 }
@@ -311,14 +301,10 @@ __device__ __forceinline__ void mul_add(uint64_t* acc, const S192& M, uint64_t l
 __device__ __forceinline__ bool orient3d_int(const Pt& a, const Pt& b, const Pt& c, const Pt& d, int* s) {
   const double v[12] = {a.x, a.y, a.z, b.x, b.y, b.z, c.x, c.y, c.z, d.x, d.y, d.z};
   long long X[12];
-  if (!int_scale<12>(v, X)) return false;
-  long long r[3][3];
-#pragma unroll
-  for (int i = 0; i < 3; ++i)
-#pragma unroll
-    for (int k = 0; k < 3; ++k) r[i][k] = X[3 * (i + 1) + k] - X[k];
-  const S192 M =
-      int_det3(r[0][2], r[1][2], r[2][2], int_minor(r[0], r[1]), int_minor(r[0], r[2]), int_minor(r[1], r[2]));
+  if (!int_scale(v, 12, X)) return false;
+#pragma unroll 1
+  for (int i = 11; i >= 3; --i) X[i] -= X[i % 3];
+  const S192 M = int_det3(X + 3, 2, 3);
   *s = (s128)M.hi < 0 ? -1 : (M.lo != 0 || M.hi != 0) ? 1 : 0;
   return true;
 }
@@ -329,37 +315,36 @@ __device__ __forceinline__ bool insphere_int(const Pt& a, const Pt& b, const Pt&
                                              int* s) {
   const double v[15] = {a.x, a.y, a.z, b.x, b.y, b.z, c.x, c.y, c.z, d.x, d.y, d.z, e.x, e.y, e.z};
   long long X[15];
-  if (!int_scale<15>(v, X)) return false;
-  long long D[4][3];
-  u128 L[4];  // squared lengths: < 3 * 2^126
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    L[i] = 0;
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      D[i][k] = X[3 * (i + 1) + k] - X[k];
-      L[i] += (u128)((s128)D[i][k] * D[i][k]);
+  if (!int_scale(v, 15, X)) return false;
+#pragma unroll 1
+  for (int i = 14; i >= 3; --i) X[i] -= X[i % 3];
+  // sum over k of (-1)^(k+1) L_k M_k: L_k the squared length of row k (< 3 * 2^126), M_k the
+  // determinant of the others (an even permutation of them, whatever k); its two halves in L_k
+  S320 lo = {}, hi = {};
+#pragma unroll 1
+  for (int k = 0; k < 4; ++k) {
+    u128 L = 0;
+#pragma unroll 1
+    for (int j = 3 * k + 3; j < 3 * k + 6; ++j) L += (u128)((s128)X[j] * X[j]);
+    S192 M = int_det3(X + 3, k, 4);
+    if (!(k & 1)) {
+      M.hi = ~M.hi + (M.lo == 0 ? 1u : 0u);
+      M.lo = ~M.lo + 1;
     }
+    mul_add(lo, M, (uint64_t)L);
+    mul_add(hi, M, (uint64_t)(L >> 64));
   }
-  const s128 m01 = int_minor(D[0], D[1]), m02 = int_minor(D[0], D[2]), m03 = int_minor(D[0], D[3]),
-             m12 = int_minor(D[1], D[2]), m13 = int_minor(D[1], D[3]), m23 = int_minor(D[2], D[3]);
-  const S192 zero = {0, 0};
-  uint64_t acc[6] = {0, 0, 0, 0, 0, 0};
-  // term k: (-1)^(k+1) L_k times the determinant of the other rows
-  S192 M = sub192(zero, int_det3(D[1][2], D[2][2], D[3][2], m12, m13, m23));
-  mul_add<0>(acc, M, (uint64_t)L[0]);
-  mul_add<1>(acc, M, (uint64_t)(L[0] >> 64));
-  M = int_det3(D[0][2], D[2][2], D[3][2], m02, m03, m23);
-  mul_add<0>(acc, M, (uint64_t)L[1]);
-  mul_add<1>(acc, M, (uint64_t)(L[1] >> 64));
-  M = sub192(zero, int_det3(D[0][2], D[1][2], D[3][2], m01, m03, m13));
-  mul_add<0>(acc, M, (uint64_t)L[2]);
-  mul_add<1>(acc, M, (uint64_t)(L[2] >> 64));
-  M = int_det3(D[0][2], D[1][2], D[2][2], m01, m02, m12);
-  mul_add<0>(acc, M, (uint64_t)L[3]);
-  mul_add<1>(acc, M, (uint64_t)(L[3] >> 64));
-  const uint64_t low = acc[0] | acc[1] | acc[2] | acc[3] | acc[4];
-  *s = (acc[5] >> 63) ? -1 : (low | acc[5]) ? 1 : 0;
+  // lo + 2^64 hi
+  uint64_t any = lo.w[0], top = 0;
+  u128 cy = 0;
+#pragma unroll
+  for (int i = 1; i < 6; ++i) {
+    cy += (u128)(i < 5 ? lo.w[i] : (uint64_t)((long long)lo.w[4] >> 63)) + hi.w[i - 1];
+    top = (uint64_t)cy;
+    any |= top;
+    cy >>= 64;
+  }
+  *s = (top >> 63) ? -1 : any ? 1 : 0;
   return true;
 }
 
