@@ -41,7 +41,7 @@ ASYNC_TRAFFIC_PER_POINT = 4554.0
 ASYNC_TRAFFIC_SOURCES = "458cf26dc1ed6999"
 REFINE_K = 128  # the refinement workload: the unit cube at size 1/128 from its surface lattice
 # the files k_async is compiled from (the host code in dt.cu does not change it)
-KERNEL_SOURCES = ["async.cu", "engine.cuh", "common.cuh", "predicates.cuh", "internal.h"]
+KERNEL_SOURCES = ["async.cu", "async.cuh", "engine.cuh", "common.cuh", "predicates.cuh", "internal.h"]
 GOLDEN = os.path.join(ROOT, "tests", "golden", "fullsize.json")
 PAPER_1E7_EPYC = 31.3  # Fig. 9, AMD EPYC 7551, 1e7 uniform points (context)
 SEED = 2
@@ -477,7 +477,7 @@ def main_batch(args, rank, world, local):
 
 
 def run_batch(args, rank, world, local, dist):
-    """Batched workload: all clouds in one dt_batch call (one persistent graph-replayed launch)
+    """Batched workload: all clouds in one dt_batch call (one graph of launches, replayed)
     against one plain dt_insert launch sequence per cloud on a sample of the clouds."""
     import torch
     import paper_1805_08831_gb300 as dt
@@ -486,7 +486,7 @@ def run_batch(args, rank, world, local, dist):
     xd = torch.from_numpy(xyz).cuda()
     stream = torch.cuda.current_stream()
     tri = dt.Triangulation(seed=SEED, stream=stream)
-    for _ in range(max(args.warmup, 1)):  # the first call tunes the block shape and captures the graph
+    for _ in range(max(args.warmup, 1)):  # the second call of a shape captures the graph
         tri.clear()
         tri.batch(xd, off)
     torch.cuda.synchronize()

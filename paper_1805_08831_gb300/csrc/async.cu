@@ -4,6 +4,10 @@
 #include <algorithm>
 #include <cstdlib>
 
+namespace dtg {
+constexpr int kADefer = 16;  // aborted points waiting for a retry
+}
+
 #include "async.cuh"
 
 namespace dtg {

@@ -5,12 +5,13 @@
 // the insertion and retries it later. Here every warp is such a thread: warp w takes the w-th
 // contiguous segment of the wave's Moore order and inserts its points in that order, each walk
 // starting from the warp's previous ball (Algorithm 1). Ownership is a 32-bit word per
-// tetrahedron slot (0 = free, else the owning warp). One insertion:
+// tetrahedron slot (0 = free, kExclusive = held by one warp, else the number of its sharers). One
+// insertion:
 //   1. walk (Section 2.1) from the previous ball, reading the mesh without locks;
 //   2. cavity search (Section 2.1, Eq. 1) on those unlocked reads: the cavity C, its outside
 //      neighbours A and the boundary facets, with every record kept in shared memory;
-//   3. lock C, A and the slots the ball needs beyond C (Section 2.5 reuses C's slots first),
-//      one compare-and-swap each; any slot held by another warp aborts the insertion (rule
+//   3. lock C, A (shared) and the slots the ball needs beyond C (Section 2.5 reuses C's slots
+//      first), one atomic each; a slot held against it by another warp aborts the insertion (rule
 //      (1) of Section 3.2: a thread touches only tetrahedra it owns);
 //   4. re-read C (whole records) and A (vertices) under the locks: a difference means another
 //      warp changed them between steps 2 and 3, and the insertion starts over from the walk;
@@ -19,15 +20,18 @@
 //   5. write the ball (Section 2.5: one tetrahedron per boundary facet, adjacency through the
 //      edge table), the back-pointers of A, then release every lock after a fence.
 // Aborted points wait in a small per-warp list and are retried after later insertions; what is
-// still left when the segment ends goes to the next pass. A cavity larger than the per-warp
+// still left when the segment ends goes to the next launch. A cavity larger than the per-warp
 // shared-memory workspace is inserted again in a global-memory workspace borrowed from a pool,
 // else by a separate large-cavity launch; a predicate the FP32 stage cannot decide hands the
-// point to the round-based engine. No warp ever waits on another, so every loop here is
-// bounded by the segment length and fixed retry counts.
+// point to a launch of the kernels with the exact stages (kExact). No warp ever waits on another,
+// so every loop here is bounded by the segment length and fixed retry counts.
 //
 // The triangulation does not depend on the order of insertions (exact predicates and one
 // symbolic perturbation, Section 2.4), so this engine gives the same tetrahedra as the
 // round-based one.
+//
+// The file that includes this one sets kADefer, the aborted points a warp keeps for a retry (the
+// borrowed workspaces of all of them have one layout: the same number in each).
 #pragma once
 #include <cuda_runtime.h>
 
@@ -42,7 +46,6 @@ namespace dtg {
 namespace {
 
 constexpr int kAW = 4;            // warps per block of the shared-memory kernel
-constexpr int kADefer = 16;       // aborted points waiting for a retry
 constexpr int kARetry = 3;        // immediate restarts after a failed re-read
 constexpr int kATail = 48;        // further tries at its deferred points by a warp that has no others left
 constexpr uint32_t kAChunk = 32;  // slots taken from the allocator at a time
@@ -187,9 +190,9 @@ __device__ __forceinline__ bool rec_ok(const Tet& T, uint32_t ntets, uint32_t np
 
 // The predicates' FP32 stage on the double-float point copy (predicates.cuh: rigorous error
 // bounds, Section 2.4's filters moved to FP32). When it cannot decide, the insertion is handed to
-// the round-based engine, which runs the whole cascade (FP64 filter, exact arithmetic, symbolic
-// perturbation): keeping the exact stages out of this kernel keeps its registers free of the
-// save and restore traffic their calls would cost. A return of 0 means "undecided".
+// the kernels built with kExact, which run the whole cascade (FP64 filter, exact arithmetic,
+// symbolic perturbation): keeping the exact stages out of the common kernel keeps its registers
+// free of the save and restore traffic their calls would cost. A return of 0 means "undecided".
 
 __device__ __forceinline__ PtF pick(bool c, const PtF& x, const PtF& y) {
   PtF r;
@@ -986,7 +989,7 @@ __device__ __forceinline__ int try_insert(const Ctx& c, W& w, uint32_t* lock, ui
 }
 
 // Hands point p to a queue of the host's next step (0: next pass, 1: large cavities, 2: the
-// round-based engine's exact predicates). Lane 0.
+// kernels with the exact predicates). Lane 0.
 __device__ __forceinline__ void to_queue(const AsyncIO& io, const Ctx& c, int q, uint32_t p) {
   uint32_t* out = q == 0 ? io.lose_out : (q == 1 ? io.big_out : io.exact_out);
   const int qi = q == 0 ? io.lose_q : (q == 1 ? io.big_q : io.exact_q);

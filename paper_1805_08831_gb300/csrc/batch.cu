@@ -13,6 +13,10 @@
 
 #include <algorithm>
 
+namespace dtg {
+constexpr int kADefer = 16;  // aborted points waiting for a retry
+}
+
 #include "async.cuh"
 
 namespace dtg {

@@ -922,7 +922,7 @@ struct dt_handle {
   double alpha = 0.02;   // candidates per round = alpha * mesh vertices (measured best at 1e7 and 1e8)
   double alpha_refine = 0.01;  // the same during dt_refine
   double refine_rebuild = 0.25;  // dt_refine: rebuild the mesh when an iteration adds this share
-  double gamma = 0.3;    // wave size = gamma * mesh vertices (round-based and batch engines)
+  double gamma = 0.3;    // wave size = gamma * mesh vertices (round-based engine)
   double gamma_async = 2.0;  // the asynchronous engine's waves (measured: 164.9 ms per 1e7 uniform
                              // step at 2.0 against 166.8 at 1.0, 175.0 at 0.5 and 185.6 at 0.3;
                              // 1e8: 1192 ms at 2.0 against 1264 at 1.0): fewer, longer launches
@@ -2556,10 +2556,9 @@ int dt_refine(dt_handle* h, double size, double ratio, double spacing, const dou
     uint64_t m = 0, ns = 0;
     if ((rc = refine_step(h->rws, h->tets, h->st_host->bump, h->pts, h->n_pts, p, &m, &ns, h->stream)) != DT_OK) break;
     if (ns == 0) break;
-    // refinement centres lie almost on the spheres of their neighbours and the first iterations
-    // fill an empty interior (cavities of thousands of tetrahedra): the round-based engine,
-    // with its full predicate cascade and large-cavity tiers, is faster here (5.9 s against
-    // 10.9 s for the 1/128 box)
+    // refinement centres lie almost on the spheres of their neighbours: the exact kernels from
+    // the first launch (the round-based engine took 360 ms where these take 58, for the box of 48
+    // intervals)
     // a rebuild pays for the whole mesh again (the boundary points' degenerate predicates
     // included) but keeps every cavity small; inserting a quarter of the mesh's points or more
     // into it measured slower than rebuilding at every iteration of the 1/128 box (requiring
