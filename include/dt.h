@@ -150,7 +150,8 @@ int dt_insert_host(dt_handle* h, const double* xyz_host, uint64_t n);
  * Replaces the handle's content (dt_insert returns DT_ESTATE until dt_clear). A cloud with fewer
  * than four non-coplanar points gets no tetrahedra and is counted in n_clouds_degenerate; the
  * call returns DT_EDEGENERATE only if every cloud is so. Vertex ids in dt_get_tets are local to
- * each cloud. Each cloud's tetrahedra are those of dt_insert on that cloud alone. */
+ * each cloud. Each cloud's tetrahedra are those of dt_insert on that cloud alone. After a call that
+ * failed as a whole (bad coordinates, out of memory) the handle's list is empty. */
 int dt_batch(dt_handle* h, const double* xyz_dev, const uint64_t* offsets_host, uint32_t n_clouds);
 
 /* Delaunay refinement of the current triangulation inside an axis-aligned box (Section 4,

@@ -250,9 +250,13 @@ class Triangulation:
         off = np.ascontiguousarray(offsets, dtype=np.uint64)
         if off.ndim != 1 or off.size < 2:
             raise ValueError("offsets must hold n_clouds + 1 entries")
-        self._check_dev(lib().dt_batch(self._h, ctypes.c_void_p(xyz.data_ptr()),
-                                       off.ctypes.data_as(ctypes.c_void_p), off.size - 1), "dt_batch")
-        self._n_clouds = off.size - 1
+        rc = lib().dt_batch(self._h, ctypes.c_void_p(xyz.data_ptr()), off.ctypes.data_as(ctypes.c_void_p),
+                            off.size - 1)
+        # refused arguments leave the handle's last batch; any other outcome, an error too, replaces
+        # it, and the list writes this batch's n_clouds + 1 cloud offsets
+        if xyz.data_ptr() and off[0] == 0 and np.all(off[1:] >= off[:-1]) and 0 < off[-1] < 0xFFFFFFF0:
+            self._n_clouds = off.size - 1
+        self._check_dev(rc, "dt_batch")
 
     def tets_batch(self, canonical: bool = True, out=None):
         """After batch(): (tets numpy uint32 [T, 4] with cloud-local ids, cloud_offsets numpy

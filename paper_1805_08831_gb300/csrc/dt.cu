@@ -964,7 +964,7 @@ struct dt_handle {
   bool batch_mode = false;
   uint32_t n_clouds = 0;
   std::vector<uint64_t> boff;              // input offsets of the clouds
-  std::vector<BatchCloud> bclouds_host;    // per-cloud ranges and results
+  std::vector<BatchCloud> bclouds_host;    // per-cloud ranges and results; empty: the batch did not complete
   uint64_t* boff_dev = nullptr;
   BatchCloud* bclouds = nullptr;
   uint64_t cap_bclouds = 0;
@@ -2066,6 +2066,7 @@ int batch_leftovers(dt_handle* h, int src, unsigned long long* totals, cudaStrea
 }
 
 int batch_impl(dt_handle* h, const double* xyz, const uint64_t* off, uint32_t nc) {
+  h->bclouds_host.clear();  // no rows until the batch is complete
   // DT_BATCH_ALPHA: warps per mesh vertex of this batch
   struct AlphaGuard {
     dt_handle* h;
@@ -2256,6 +2257,11 @@ int batch_get_tets(dt_handle* h, uint32_t* tets_dev, uint64_t cap, uint64_t* n_t
                    int canonical) {
   cudaStream_t s = h->stream;
   const uint32_t nc = h->n_clouds;
+  if (h->bclouds_host.size() != nc) {  // refused or not completed: no list
+    h->stats.n_tets = 0;
+    if (cloud_offsets) std::fill(cloud_offsets, cloud_offsets + nc + 1, 0);
+    return DT_OK;
+  }
   unsigned long long *counts = nullptr, *ooff = nullptr;
   if (cudaMalloc(&counts, nc * 8ull) != cudaSuccess) return DT_ENOMEM;
   if (cudaMalloc(&ooff, (nc + 1) * 8ull) != cudaSuccess) {

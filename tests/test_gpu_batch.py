@@ -227,3 +227,34 @@ def test_batch_refuses_bad_coordinates_and_goes_on():
         t.batch(torch.from_numpy(xyz).cuda(), off)
         tets, coff = t.tets_batch()
     assert_clouds_match(split(xyz, off), [tets[int(coff[c]):int(coff[c + 1])] for c in range(6)])
+
+
+@pytest.mark.parametrize("earlier", [0, 2, 40])
+def test_no_rows_after_a_refused_batch(earlier):
+    """The list between a refused batch and the clear: no rows, on a fresh handle and after smaller
+    and larger batches, through every form of the list."""
+    xyz, off = synth.batched_clouds(6, 8, lo=50, hi=500)
+    bad = xyz.copy()
+    bad[77, 1] = np.inf
+    with dt.Triangulation(seed=0) as t:
+        if earlier:
+            x0, off0 = synth.batched_clouds(earlier, 9, lo=50, hi=300)
+            t.batch(torch.from_numpy(x0).cuda(), off0)
+        with pytest.raises(dt.DTError) as e:
+            t.batch(torch.from_numpy(bad).cuda(), off)
+        assert e.value.code == dt.DT_EINVAL
+        out = torch.zeros((9000, 4), dtype=torch.int32).pin_memory().numpy().view(np.uint32)
+        for canonical in (True, False):
+            assert len(t.tets_host(canonical=canonical, out=out)) == 0
+            for buf in (out, None):
+                rows, coff = t.tets_batch(canonical=canonical, out=buf)
+                assert len(rows) == 0 and coff.shape == (7,) and not coff.any()
+        assert t.num_tets() == 0 and not out.any()
+        t.batch(torch.from_numpy(xyz).cuda(), off)
+        tets, coff = t.tets_batch()
+        assert np.array_equal(t.tets_host(), tets)
+        with pytest.raises(dt.DTError):  # refused arguments: the last batch stays
+            t.batch(torch.from_numpy(xyz).cuda(), off[::-1].copy())
+        again, coff2 = t.tets_batch()
+        assert np.array_equal(again, tets) and np.array_equal(coff2, coff)
+    assert_clouds_match(split(xyz, off), [tets[int(coff[c]):int(coff[c + 1])] for c in range(6)])
