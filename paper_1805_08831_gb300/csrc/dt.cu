@@ -893,7 +893,8 @@ struct dt_handle {
   uint64_t mesh_pts = 0;       // vertices the mesh may hold (points whose records were built)
   bool use_subdet = false;
   uint64_t cap_tets = 0;
-  uint64_t cap_lock = 0;     // owner words (a batch grows the store without them)
+  uint64_t cap_lock = 0;     // owner words
+  uint64_t cap_subdet = 0;   // slots the cache has entries for (a batch grows the store without it)
   uint32_t* freelist = nullptr;
   uint32_t* pending = nullptr;
   uint64_t cap_free = 0;
@@ -1071,8 +1072,8 @@ InsertLog make_log(dt_handle* h) {
 uint64_t device_bytes(const dt_handle* h) {
   uint64_t b = 0;
   b += h->cap_pts * (sizeof(Pt) + sizeof(PtF) + 1 + 4);             // points, FP32 copy, flag, hint
-  b += h->cap_tets * (sizeof(Tet) + 16 + 4);                         // records, claim pair, owner word
-  if (h->subdet) b += h->cap_tets * 2 * sizeof(float4);              // sub-determinant cache
+  b += h->cap_tets * (sizeof(Tet) + 16) + h->cap_lock * 4;           // records, claim pair; owner words
+  b += h->cap_subdet * 2 * sizeof(float4);                           // sub-determinant cache
   b += h->in_cap * 24 + h->out_cap * 16;                             // host entry points' buffers
   b += canon_ws_bytes(h->canon);                                     // the canonical list's workspace
   b += h->cap_free * 8;                                              // free list and pending
@@ -1132,48 +1133,54 @@ int reserve_tets(dt_handle* h, uint64_t total_pts) {
   // every warp of an asynchronous launch keeps a few dozen slots of its own while it runs
   uint64_t need = (uint64_t)(f * (double)total_pts) + 4096 + 64 * async_warps_for(h, total_pts);
   if (need > kMaxSlots) need = kMaxSlots;
-  // after a batch the store may be large enough while it has no owner words and a shorter free
-  // list than this engine's
-  if (need <= h->cap_tets && h->cap_lock >= h->cap_tets) return DT_OK;
-  unsigned long long bump = h->has_mesh ? h->st_host->bump : 0;
   need = std::max(need, h->cap_tets);
-  if (need > h->cap_tets) {
-    if (grow(h->tets, bump, need, h->stream) != cudaSuccess) return DT_ENOMEM;
+  // free list: the slots a round frees, plus every warp's private slots that the asynchronous
+  // engine hands back when its launch ends
+  const uint64_t nf = std::max<uint64_t>(need / 4 + 4096 + (uint64_t)async_max_warps() * 160, h->cap_free);
+  // each array by its own capacity: a batch grows the records, the owner words and the free list
+  // (to an entry per slot, as many as there can be) but not the cache, and an allocation that
+  // failed leaves some arrays shorter than the others
+  const bool records = need > h->cap_tets, words = need > h->cap_lock,
+             cache = h->use_subdet && need > h->cap_subdet, lists = h->cap_free < std::min(nf, need);
+  if (!records && !words && !cache && !lists) return DT_OK;
+  const unsigned long long bump = h->has_mesh ? h->st_host->bump : 0;
+  cudaStream_t s = h->stream;
+  if (records) {
+    if (grow(h->tets, bump, need, s) != cudaSuccess) return DT_ENOMEM;
     // slots not yet handed out read as dead (v.x == v.y == 0): the asynchronous engine may read
     // a slot through a freshly written pointer before its record arrives, and must never find an
     // old, self-consistent mesh there
-    cudaMemsetAsync(h->tets + bump, 0, (need - bump) * sizeof(Tet), h->stream);
-    if (grow(h->claim, 2 * bump, 2 * need, h->stream) != cudaSuccess) return DT_ENOMEM;
+    if (cudaMemsetAsync(h->tets + bump, 0, (need - bump) * sizeof(Tet), s) != cudaSuccess) return DT_ECUDA;
+    if (grow(h->claim, 2 * bump, 2 * need, s) != cudaSuccess) return DT_ENOMEM;
     // claim words of slots not yet handed out start at zero (below every priority)
-    cudaMemsetAsync(h->claim + 2 * bump, 0, 2 * (need - bump) * sizeof(unsigned long long), h->stream);
+    if (cudaMemsetAsync(h->claim + 2 * bump, 0, 2 * (need - bump) * sizeof(unsigned long long), s) != cudaSuccess)
+      return DT_ECUDA;
+    h->cap_tets = need;
   }
-  if (h->use_subdet) {
+  if (cache) {
     // cache entries of slots not yet handed out read as invalid
-    if (grow(h->subdet, 2 * bump, 2 * need, h->stream) != cudaSuccess) return DT_ENOMEM;
-    cudaMemsetAsync(h->subdet + 2 * bump, 0, 2 * (need - bump) * sizeof(float4), h->stream);
+    if (grow(h->subdet, 2 * bump, 2 * need, s) != cudaSuccess) return DT_ENOMEM;
+    if (cudaMemsetAsync(h->subdet + 2 * bump, 0, 2 * (need - bump) * sizeof(float4), s) != cudaSuccess) return DT_ECUDA;
+    h->cap_subdet = need;
   }
-  // owner words: every slot free (no lock is held between launches)
-  cudaStreamSynchronize(h->stream);
-  cudaFree(h->lock);
-  h->lock = nullptr;
-  h->cap_lock = 0;
-  if (cudaMalloc(&h->lock, need * sizeof(uint32_t)) != cudaSuccess) return DT_ENOMEM;
-  h->cap_lock = need;
-  cudaMemsetAsync(h->lock, 0, need * sizeof(uint32_t), h->stream);
-  // free list: the slots a round frees, plus every warp's private slots that the asynchronous
-  // engine hands back when its launch ends
-  uint64_t nf = std::max<uint64_t>(need / 4 + 4096 + (uint64_t)async_max_warps() * 160, h->cap_free);
-  uint64_t fold = h->has_mesh ? h->st_host->free_avail : 0;
-  if (grow(h->freelist, fold, nf, h->stream) != cudaSuccess) return DT_ENOMEM;
-  cudaFree(h->pending);
-  h->pending = nullptr;
-  if (cudaMalloc(&h->pending, nf * 4) != cudaSuccess) return DT_ENOMEM;
-  h->cap_tets = need;
-  h->cap_free = nf;
-  unsigned long long vals[2] = {need, nf};
-  cudaMemcpyAsync(&h->st->capacity, &vals[0], 8, cudaMemcpyHostToDevice, h->stream);
-  cudaMemcpyAsync(&h->st->free_capacity, &vals[1], 8, cudaMemcpyHostToDevice, h->stream);
-  cudaStreamSynchronize(h->stream);
+  // (the list of a mesh that stays after a failed call uses the words and the pending slots: the old
+  // arrays go only when the new ones are there)
+  cudaStreamSynchronize(s);
+  if (words) {
+    // owner words: every slot free (no lock is held between launches)
+    if (grow(h->lock, 0, need, s) != cudaSuccess) return DT_ENOMEM;
+    if (cudaMemsetAsync(h->lock, 0, need * sizeof(uint32_t), s) != cudaSuccess) return DT_ECUDA;
+    h->cap_lock = need;
+  }
+  if (lists) {
+    const uint64_t fold = h->has_mesh ? h->st_host->free_avail : 0;
+    if (grow(h->freelist, fold, nf, s) != cudaSuccess || grow(h->pending, 0, nf, s) != cudaSuccess) return DT_ENOMEM;
+    h->cap_free = nf;
+  }
+  unsigned long long vals[2] = {h->cap_tets, h->cap_free};
+  cudaMemcpyAsync(&h->st->capacity, &vals[0], 8, cudaMemcpyHostToDevice, s);
+  cudaMemcpyAsync(&h->st->free_capacity, &vals[1], 8, cudaMemcpyHostToDevice, s);
+  cudaStreamSynchronize(s);
   return DT_OK;
 }
 
@@ -1819,8 +1826,9 @@ int insert_impl(dt_handle* h, const double* xyz, uint64_t n, bool exact = false)
     cudaMemsetAsync(h->cell_hint, 0xFF, (size_t)4 << (3 * cb), s);
     cudaMemsetAsync(h->cell_hint2, 0xFF, (size_t)4 << (3 * cbc), s);
     // a new mesh: every slot reads as dead until it is handed out (see reserve_tets)
-    cudaMemsetAsync(h->tets, 0, h->cap_tets * sizeof(Tet), s);
-    if (h->subdet) cudaMemsetAsync(h->subdet, 0, 2 * h->cap_tets * sizeof(float4), s);
+    if (cudaMemsetAsync(h->tets, 0, h->cap_tets * sizeof(Tet), s) != cudaSuccess) return DT_ECUDA;
+    if (h->use_subdet && cudaMemsetAsync(h->subdet, 0, 2 * h->cap_subdet * sizeof(float4), s) != cudaSuccess)
+      return DT_ECUDA;
     DevState z{};
     z.stamp = h->next_stamp;
     z.capacity = h->cap_tets;
@@ -2244,8 +2252,8 @@ int reserve_out(dt_handle* h, uint64_t rows) {
 
 // Memory of the mesh that holds nothing while no insertion runs: the claim words (16 bytes per
 // slot; zero is below every priority), the owner words (4 bytes per slot, zero between
-// launches) and the list of freed slots (a quarter of the slots, empty between launches). A batch
-// has no owner words; its lists of freed and free slots hold an entry per slot and start empty.
+// launches) and the list of freed slots (a quarter of the slots, empty between launches). A batch's
+// lists of freed and free slots hold an entry per slot and start empty.
 CanonScratch canon_scratch(dt_handle* h) {
   uint4* rows = reinterpret_cast<uint4*>(h->claim);
   if (h->batch_mode) return CanonScratch{rows, h->pending, reinterpret_cast<uint2*>(h->freelist)};

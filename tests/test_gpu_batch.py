@@ -167,21 +167,31 @@ def test_repeated_batch_replays_its_graph_on_new_data():
     assert_clouds_match(clouds, [new[int(c3[c]):int(c3[c + 1])] for c in range(30)])
 
 
-def test_insert_after_a_larger_batch_on_the_same_handle():
-    """A batch grows the tetrahedron store without the asynchronous engine's owner words: an
-    insert that follows on the handle has to bring them."""
+@pytest.mark.parametrize("subdet", [False, True])
+def test_insert_after_a_larger_batch_on_the_same_handle(subdet, monkeypatch):
+    """A batch grows the tetrahedron store, its owner words and its free list, but not the
+    sub-determinant cache: an insert that follows on the handle has to bring an entry per slot."""
+    if subdet:
+        monkeypatch.setenv("DT_SUBDET", "1")
     xyz, off = synth.batched_clouds(12, 5, lo=50, hi=3000)
     x = synth.uniform_cube(900, 6)
+    small = synth.uniform_cube(60, 7)
     ref, _ = oracle.delaunay(x)
-    with dt.Triangulation(seed=0) as t:
-        t.batch(torch.from_numpy(xyz).cuda(), off)
-        t.clear()
-        t.insert(torch.from_numpy(x).cuda())
-        assert np.array_equal(t.tets_numpy(), ref)
-        t.batch(torch.from_numpy(xyz).cuda(), off)
-        t.clear()
-        t.insert(torch.from_numpy(x).cuda())
-        assert np.array_equal(t.tets_numpy(), ref)
+    for first in (None, small):  # without a cache yet, and with one shorter than the batch's store
+        with dt.Triangulation(seed=0) as t:
+            if first is not None:
+                t.insert(torch.from_numpy(first).cuda())
+            grown = []
+            for _ in range(2):
+                t.batch(torch.from_numpy(xyz).cuda(), off)
+                before = t.stats()["device_bytes"]
+                t.clear()
+                t.insert(torch.from_numpy(x).cuda())
+                assert np.array_equal(t.tets_numpy(), ref)
+                grown.append(t.stats()["device_bytes"] - before)
+            # an entry of 32 bytes for each of the store's slots (8 a point at least, all but the
+            # 6000 the first insert may have brought)
+            assert not subdet or grown[0] >= 32 * (8 * len(xyz) - 6000) > 0
 
 
 @pytest.mark.parametrize("sizes", [(0, 3, 4, 5, 6), (2047, 2048, 2049), (14336, 14337, 40), (1,), (900, 20001)])
