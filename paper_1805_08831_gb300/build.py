@@ -17,7 +17,7 @@ BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(BUILD, "libdt_gb300.so")
 RUNNER = os.path.join(BUILD, "dt_run")
 SOURCES = ["order.cu", "dt.cu", "async.cu", "batch.cu", "mlp.cu", "refine.cu", "canonical.cu"]
-HEADERS = ["common.cuh", "predicates.cuh", "engine.cuh", "async.cuh", "internal.h"]
+HEADERS = ["common.cuh", "predicates.cuh", "engine.cuh", "async.cuh", "internal.h", "per_device.h"]
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_103a,code=sm_103a",

@@ -9,6 +9,7 @@ constexpr int kADefer = 16;  // aborted points waiting for a retry
 }
 
 #include "async.cuh"
+#include "per_device.h"
 
 namespace dtg {
 namespace {
@@ -96,19 +97,24 @@ __global__ void k_async_close_state(Ctx c, int consumed_q) {
 // kernel with the exact stages: 4, its calls save and restore fewer registers.
 constexpr int kFullBlocks = 8, kFewBlocks = 4, kExactBlocks = 4;
 
-template <int kMinBlocks, bool kCache = false, bool kExact = false>
-int resident_warps() {
-  int dev = 0, sms = 0, per = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_async<kMinBlocks, kCache, kExact>, kAW * 32, 0) != cudaSuccess)
-    per = kMinBlocks;
-  return std::max(1, sms * std::max(per, 1) * kAW);
+int current_device() {
+  int dev = 0;
+  return cudaGetDevice(&dev) == cudaSuccess ? dev : 0;
 }
 
-int async_max_warps_few() {
-  static const int cached = resident_warps<kFewBlocks>();
-  return cached;
+// Warps of the kernel that are resident on the current device at once.
+template <int kMinBlocks, bool kCache = false, bool kExact = false>
+int resident_warps() {
+  static PerDevice kept;
+  const int dev = current_device();
+  return (int)kept.get(dev, [dev] {
+    int sms = 0, per = 0;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_async<kMinBlocks, kCache, kExact>, kAW * 32, 0) !=
+        cudaSuccess)
+      per = kMinBlocks;
+    return std::max(1, sms * std::max(per, 1) * kAW);
+  });
 }
 
 }  // namespace
@@ -124,7 +130,7 @@ int async_launch(const Ctx& c, const AsyncIO& io, uint32_t* lock, const InsertLo
   else if (io.local) k_async_local<false><<<1, io.W * 32, local, s>>>(cc, io, lock, lg);
   else if (io.exact) k_async<kExactBlocks, false, true><<<blocks, kAW * 32, 0, s>>>(cc, io, lock, lg);
   else if (c.subdet) k_async<kFullBlocks, true><<<blocks, kAW * 32, 0, s>>>(cc, io, lock, lg);
-  else if (io.W <= (uint32_t)async_max_warps_few()) k_async<kFewBlocks><<<blocks, kAW * 32, 0, s>>>(cc, io, lock, lg);
+  else if (io.W <= (uint32_t)resident_warps<kFewBlocks>()) k_async<kFewBlocks><<<blocks, kAW * 32, 0, s>>>(cc, io, lock, lg);
   else k_async<kFullBlocks><<<blocks, kAW * 32, 0, s>>>(cc, io, lock, lg);
   k_async_close_copy<<<152, 256, 0, s>>>(cc);
   k_async_close_state<<<1, 1, 0, s>>>(cc, io.carry_n ? io.carry_q : -1);
@@ -149,24 +155,21 @@ int async_launch_big(const Ctx& c, const AsyncIO& io, uint32_t* lock, const Inse
   return cudaPeekAtLastError() == cudaSuccess ? DT_OK : DT_ECUDA;
 }
 
-// Most warps of a launch that runs as one block (AsyncIO::local), 0 if it cannot.
+// Most warps of a launch that runs as one block (AsyncIO::local) on the current device, 0 if it cannot.
 uint32_t async_local_warps() {
-  static const bool ready =
-      cudaFuncSetAttribute(k_async_local<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)(kLocalWarps * sizeof(SmallWST<false, true>))) == cudaSuccess &&
-      cudaFuncSetAttribute(k_async_local<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)(kLocalWarps * sizeof(SmallWST<false, true>))) == cudaSuccess;
-  return ready ? kLocalWarps : 0;
+  static PerDevice kept;
+  return (uint32_t)kept.get(current_device(), [] {
+    const int bytes = (int)(kLocalWarps * sizeof(SmallWST<false, true>));
+    const auto opt_in = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    return cudaFuncSetAttribute(k_async_local<false>, opt_in, bytes) == cudaSuccess &&
+                   cudaFuncSetAttribute(k_async_local<true>, opt_in, bytes) == cudaSuccess
+               ? kLocalWarps
+               : 0u;
+  });
 }
 
-int async_max_warps() {
-  static const int cached = resident_warps<kFullBlocks>();
-  return cached;
-}
+int async_max_warps() { return resident_warps<kFullBlocks>(); }
 
-int async_max_warps_exact() {
-  static const int cached = std::min(resident_warps<kExactBlocks, false, true>(), async_max_warps());
-  return cached;
-}
+int async_max_warps_exact() { return std::min(resident_warps<kExactBlocks, false, true>(), async_max_warps()); }
 
 }  // namespace dtg

@@ -17,6 +17,7 @@
 
 #include "common.cuh"
 #include "internal.h"
+#include "per_device.h"
 
 namespace dtg {
 namespace {
@@ -690,15 +691,16 @@ bool radix_sort_pairs(uint64_t* k, uint32_t* v, uint64_t* ka, uint32_t* va, uint
 }
 
 // The tiled scatter needs more than the default 48 KB of dynamic shared memory: opt in once per
-// process (every device of this library runs the same build).
+// device.
 bool tiled_scatter_ready() {
-  static int state = 0;  // 0 unknown, 1 ready, -1 not available
-  if (state == 0) {
-    if (std::getenv("DT_SORT_SCATTER_PLAIN")) state = -1;
-    else state = cudaFuncSetAttribute(k_radix_scatter_tiled, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)kScatterSmem) == cudaSuccess ? 1 : -1;
-  }
-  return state == 1;
+  static PerDevice kept;
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return false;
+  return kept.get(dev, [] {
+    return !std::getenv("DT_SORT_SCATTER_PLAIN") &&
+           cudaFuncSetAttribute(k_radix_scatter_tiled, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)kScatterSmem) == cudaSuccess;
+  }) != 0;
 }
 
 bool radix_sort_pairs_bits(uint64_t* k, uint32_t* v, uint64_t* ka, uint32_t* va, uint64_t n, int lo_bit,
