@@ -792,6 +792,8 @@ __device__ __forceinline__ int try_insert(const Ctx& c, W& w, uint32_t* lock, ui
       if (nx > 0) pool_give(c, w, w.ex, nx);
       return kALost;
     }
+    // a lane re-reads slots that other lanes locked: the warp first, then each lane's fence
+    __syncwarp();
     fence_mesh<W::kLocal>();
     // 4. re-read under the locks
     bool same = true;
@@ -964,6 +966,9 @@ __device__ __forceinline__ int try_insert(const Ctx& c, W& w, uint32_t* lock, ui
         st_mesh<W::kLocal>(dst + 1, make_uint4(redirect, kNone, kNone, kNone));
       }
     }
+    // a slot's lock is not always released by the lane that wrote its record (dead slots, extra
+    // slots, back-pointers): every lane's writes come before every lane's fence, a vote orders none
+    __syncwarp();
     fence_mesh<W::kLocal>();
     release_all(w, lock, held, heldx, nc, na, nx0);
     if (freed > 0) pool_give(c, w, w.cl + nb, freed);
@@ -981,9 +986,10 @@ __device__ __forceinline__ int try_insert(const Ctx& c, W& w, uint32_t* lock, ui
       w.hint = s0;
       w.bn = W::kTable ? (nb < 32 ? nb : 32) : 0;
     }
-    if (lane < 5) w.cnt[lane] += lane == 0 ? 1 : lane == 3 ? nc : lane == 4 ? nb : 0;
-    __syncwarp();
-    return kAInserted;
+    if (lane == 0) w.cnt[0] += 1;
+    if (lane == 3) w.cnt[3] += nc;
+    if (lane == 4) w.cnt[4] += nb;
+    return kAInserted;  // the caller's next __syncwarp orders these
   }
   return kALost;
 }
@@ -1015,6 +1021,7 @@ __device__ __noinline__ int try_insert_large(const Ctx& c, L* pool, unsigned int
       const uint32_t cand = (me * 0x9E3779B1u + (uint32_t)t * 0x85EBCA6Bu) % n;
       if (atomicCAS(&busy[cand], 0u, 1u) == 0u) k = (int)cand;
     }
+  if (k >= 0) __threadfence();  // after the workspace's last borrower (it fences before its release)
   k = __shfl_sync(kFull, k, 0);
   if (k < 0) return kALost;
   L& b = pool[k];
