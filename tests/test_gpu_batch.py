@@ -268,3 +268,20 @@ def test_no_rows_after_a_refused_batch(earlier):
         again, coff2 = t.tets_batch()
         assert np.array_equal(again, tets) and np.array_equal(coff2, coff)
     assert_clouds_match(split(xyz, off), [tets[int(coff[c]):int(coff[c + 1])] for c in range(6)])
+
+
+@pytest.mark.parametrize("steps", [1, 8])
+def test_batch_of_needles_with_short_walks(steps):
+    """Walks of hundreds of steps (the hint cells of a thin cloud hold whole slices of it): a short
+    max_walk_steps leaves no point behind, and takes no other time than the default."""
+    g = np.random.default_rng(1)
+    clouds = [g.random((n, 3)) * (1.0, thin, thin) for n, thin in ((3000, 1e-3), (3000, 1e-6), (20000, 1e-3))]
+    x = torch.from_numpy(np.concatenate(clouds)).cuda()
+    ms = []
+    for limit in (0, steps):
+        with dt.Triangulation(seed=0, max_walk_steps=limit) as t:
+            t.batch(x, np.array([0, 3000, 6000, 26000]))
+            tets, coff = t.tets_batch()
+            ms.append(t.stats()["ms_insert"])
+        assert_clouds_match(clouds, [tets[int(coff[c]):int(coff[c + 1])] for c in range(3)])
+    assert ms[1] < 5 * ms[0]  # 300 times when every launch stopped the walks
