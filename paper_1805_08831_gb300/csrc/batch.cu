@@ -225,6 +225,7 @@ __global__ void k_batch_prepare(BatchCloud* clouds, const double* __restrict__ c
   __shared__ double s_max[256];
   double m = 0.0;
   for (uint32_t c = threadIdx.x; c < n_clouds; c += blockDim.x) {
+    if (clouds[c].vb == clouds[c].ve) continue;  // its box is (inf, -inf)
     const double* B = cbox + 6ull * c;
     for (int k = 0; k < 6; ++k) m = fmax(m, fabs(B[k]));
     for (int k = 0; k < 3; ++k) {
