@@ -981,6 +981,7 @@ struct dt_handle {
   uint4* bsegs = nullptr;                   // every launch's segments
   uint64_t cap_bsegs = 0;
   std::vector<uint64_t> bplan_key;          // cloud sizes and parameters the segments were made for
+  std::vector<uint32_t> bwarps;             // each cloud's most segments in one launch
   std::vector<std::pair<uint64_t, uint64_t>> bplan;  // each launch's segments: first and number
   float* beta = nullptr;                    // device: the batch's FP32 error term
   cudaStream_t bs = nullptr;                // the handle's own stream for batches (capturable)
@@ -2011,6 +2012,9 @@ int batch_plan(dt_handle* h, const uint64_t* off, uint32_t nc, cudaStream_t s) {
   std::vector<uint4> all;
   h->bplan.clear();
   h->bplan_key.clear();
+  h->bwarps.assign(nc, 0);
+  for (const auto& l : launch)
+    for (const uint4& g : l) h->bwarps[g.x] = std::max(h->bwarps[g.x], g.w >> 16);
   for (const auto& l : launch) {
     h->bplan.emplace_back(all.size(), l.size());
     all.insert(all.end(), l.begin(), l.end());
@@ -2086,9 +2090,19 @@ int batch_impl(dt_handle* h, const double* xyz, const uint64_t* off, uint32_t nc
   } guard{h, h->alpha_async};
   if (const char* e = std::getenv("DT_BATCH_ALPHA")) h->alpha_async = std::max(1e-4, std::atof(e));
   const uint64_t N = off[nc];
+  int rc = DT_OK;
+  if (!h->bs) {
+    if (cudaStreamCreateWithFlags(&h->bs, cudaStreamNonBlocking) != cudaSuccess) return DT_ECUDA;
+    for (auto& e : h->bev)
+      if (cudaEventCreate(&e) != cudaSuccess) return DT_ECUDA;
+    if (cudaMalloc(&h->beta, sizeof(float)) != cudaSuccess) return DT_ENOMEM;
+  }
+  cudaStream_t s = h->bs;
+  if ((rc = batch_plan(h, off, nc, s)) != DT_OK) return rc;
   double f = h->cfg.tet_capacity_factor > 0 ? h->cfg.tet_capacity_factor : 8.0;
   // slots per cloud: f per point, room for the first tetrahedra and ghosts, and the few dozen slots
-  // that each of a launch's warps keeps of its own while it runs
+  // that each of its warps in a launch keeps of its own while it runs (as many warps as the plan
+  // gives it: with those it would have alone the store was 1.45 to 2.2 times the points' share)
   std::vector<BatchCloud> cl(nc);
   // No cloud holds slot 0. A record read while it is first written may still have zero neighbours;
   // with slot 0 in the first cloud, a walk of another cloud went on in that cloud's mesh and
@@ -2096,7 +2110,7 @@ int batch_impl(dt_handle* h, const double* xyz, const uint64_t* off, uint32_t nc
   uint64_t T = 32, hash = 1469598103934665603ull;
   for (uint32_t c = 0; c < nc; ++c) {
     uint64_t n = off[c + 1] - off[c];
-    uint64_t cap = (uint64_t)(f * (double)n) + 64 + 64 * std::min<uint64_t>(async_warps_for(h, n), n);
+    uint64_t cap = (uint64_t)(f * (double)n) + 64 + 64ull * h->bwarps[c];
     cl[c] = BatchCloud{};
     cl[c].vb = (uint32_t)off[c];
     cl[c].ve = (uint32_t)off[c + 1];
@@ -2106,15 +2120,7 @@ int batch_impl(dt_handle* h, const double* xyz, const uint64_t* off, uint32_t nc
     hash = (hash ^ n) * 1099511628211ull;
   }
   if (T > kMaxSlots) return DT_ENOMEM;
-  int rc = batch_reserve(h, N, nc, T);
-  if (rc != DT_OK) return rc;
-  if (!h->bs) {
-    if (cudaStreamCreateWithFlags(&h->bs, cudaStreamNonBlocking) != cudaSuccess) return DT_ECUDA;
-    for (auto& e : h->bev)
-      if (cudaEventCreate(&e) != cudaSuccess) return DT_ECUDA;
-    if (cudaMalloc(&h->beta, sizeof(float)) != cudaSuccess) return DT_ENOMEM;
-  }
-  cudaStream_t s = h->bs;
+  if ((rc = batch_reserve(h, N, nc, T)) != DT_OK) return rc;
   // the batch stream starts after the caller's stream has produced the input
   cudaEventRecord(h->bev[0], h->stream);
   cudaStreamWaitEvent(s, h->bev[0], 0);
@@ -2127,7 +2133,6 @@ int batch_impl(dt_handle* h, const double* xyz, const uint64_t* off, uint32_t nc
   h->n_pts = N;
   h->batch_mode = true;
   unsigned int bad = 0;
-  if ((rc = batch_plan(h, off, nc, s)) != DT_OK) return rc;
   int warps = 4;  // per block; larger blocks are slower and kept for comparison
   if (const char* e = std::getenv("DT_BATCH_WARPS")) warps = std::atoi(e);
   if (const char* e = std::getenv("DT_BATCH_SHAPE")) warps = std::atoi(e) & 255;

@@ -304,3 +304,15 @@ def test_an_empty_cloud_does_not_widen_the_others_error_bounds():
         got = [tets[int(coff[c]):int(coff[c + 1])] for c in range(len(off) - 1) if off[c + 1] > off[c]]
         assert_clouds_match(clouds, got)
     assert best[1] < 1.5 * best[0]
+
+
+def test_many_clouds_take_no_more_memory_than_their_points_need():
+    """The store is 60 bytes for each of 8 slots a point, 64 a cloud, and 64 for each warp that a
+    cloud is planned to have: a hundredth of its points when many clouds fill the device (an eighth
+    more slots, where the warps it would have alone made it 2.2 times the points' share)."""
+    xyz, off = synth.batched_clouds(2000, 4, lo=50, hi=2000)
+    with dt.Triangulation(seed=0) as t:
+        t.batch(torch.from_numpy(xyz).cuda(), off)
+        held = t.stats()["device_bytes"]
+    points = 220 * len(xyz)  # records, order, lists: bytes a point beside the store's
+    assert held < points + 1.5 * 60 * (8 * len(xyz) + 64 * 2000)
