@@ -103,10 +103,11 @@ typedef struct {
   uint64_t max_walk;       /* longest single walk (steps) */
   uint64_t n_clouds_degenerate; /* dt_batch: clouds with fewer than four non-coplanar points */
   uint64_t batch_warps;    /* dt_batch: block shape used (warps per block) */
-  double batch_alpha;      /* dt_batch: most concurrent insertions per mesh vertex */
+  double batch_alpha;      /* dt_batch: concurrent insertions per mesh vertex of a cloud (up to 3
+                              times that below 300, fewer where many clouds fill the device) */
   double ms_batch_tune;    /* dt_batch: 0 (nothing is tuned by timing) */
   uint64_t batch_graph;    /* dt_batch: 1 if the last call replayed its captured CUDA graph */
-  uint64_t batch_min_blocks; /* dt_batch: resident blocks per SM the chosen shape was built for */
+  uint64_t batch_min_blocks; /* dt_batch: resident blocks per SM the largest launch's kernel is built for */
   double ms_async;         /* summed device time of the asynchronous insertion launches
                               (DT_FLAG_PROFILE only) */
   uint64_t n_async;        /* asynchronous insertion launches (one per wave or retry pass) */

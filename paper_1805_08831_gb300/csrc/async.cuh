@@ -1042,7 +1042,10 @@ __device__ __noinline__ int try_insert_large(const Ctx& c, L* pool, unsigned int
     w.cnt[4] += b.cnt[4];
     w.cnt[5] += b.cnt[5];
     w.cnt[6] += b.cnt[6];
-    if (r == kAInserted) w.hint = b.hint;
+    if (r == kAInserted) {
+      w.hint = b.hint;
+      atomicAdd(&c.st->n_big, 1ull);
+    }
     w.bn = 0;
     __threadfence();
     atomicExch(&busy[k], 0u);
@@ -1164,6 +1167,7 @@ __device__ __forceinline__ void run_segment(const Ctx& c, const AsyncIO& io, W& 
     unsigned long long* dst[8] = {&c.st->n_inserted, &c.st->n_conflicts, &c.st->n_attempts, &c.st->sum_cavity,
                                   &c.st->sum_ball, &c.st->sum_walk, &c.st->n_restart, &c.st->n_inserted_async};
     w.cnt[7] = w.cnt[0];
+    if (!W::kTable && w.cnt[0]) atomicAdd(&c.st->n_big, (unsigned long long)w.cnt[0]);
 #pragma unroll 1
     for (int k = 0; k < 8; ++k)
       if (w.cnt[k]) atomicAdd(dst[k], (unsigned long long)w.cnt[k]);

@@ -159,7 +159,8 @@ __global__ void k_batch_finish(BatchMem b, int src) {
     cl->inserted = ok ? (uint32_t)st->n_inserted : 0u;
     const unsigned long long v[kBatchTotals] = {ok ? st->n_inserted : 0ull, st->n_conflicts, st->n_attempts,
                                                 st->sum_cavity, st->sum_ball, st->sum_walk, ok ? st->q[kQLarge] : 0ull,
-                                                ok ? st->q[list_queue(src)] : 0ull, st->n_dups, st->n_exact, st->n_sos};
+                                                ok ? st->q[list_queue(src)] : 0ull, st->n_dups, st->n_exact, st->n_sos,
+                                                st->n_big};
     for (int k = 0; k < kBatchTotals; ++k)
       if (v[k]) atomicAdd(&b.totals[k], v[k]);
   }
@@ -247,7 +248,6 @@ __global__ void k_batch_prepare(BatchCloud* clouds, const double* __restrict__ c
 
 uint32_t batch_hint_fine() { return kBatchFine; }
 uint32_t batch_hint_coarse() { return kBatchCoarse; }
-int batch_cb() { return kBatchCb; }
 size_t batch_big_ws_bytes() { return sizeof(BatchBigWS); }
 
 bool batch_ready() {
@@ -263,13 +263,19 @@ void batch_init(const Ctx& c, const BatchMem& b, cudaStream_t s) {
 // Blocks of 4 warps unless more are asked for: with 128 registers (4 resident blocks per SM) for a
 // launch that fits the chip so, where the length of one insertion counts (64 small clouds: 4.8 ms
 // against 5.3), else with 80 (6 blocks; 512 clouds: 70.6 ms against 74.0).
+int batch_min_blocks(int warps, uint64_t n) {
+  return warps > 4 ? 1 : (n + warps - 1) / warps <= 152u * 4 ? 4 : 6;
+}
+
 int batch_launch(int warps, const Ctx& c, const BatchMem& b, const uint4* segs, uint32_t n, int src, cudaStream_t s) {
   const size_t smem = (size_t)warps * sizeof(SmallWST<false>);
   if (warps < 1 || warps > 32) return DT_EINVAL;
   const unsigned blocks = (n + warps - 1) / warps;
-  if (warps <= 4 && blocks <= 152u * 4) k_batch<128, 4><<<blocks, warps * 32, smem, s>>>(c, b, segs, n, src);
-  else if (warps <= 4) k_batch<128, 6><<<blocks, warps * 32, smem, s>>>(c, b, segs, n, src);
-  else k_batch<1024, 1><<<blocks, warps * 32, smem, s>>>(c, b, segs, n, src);
+  switch (batch_min_blocks(warps, n)) {
+    case 4: k_batch<128, 4><<<blocks, warps * 32, smem, s>>>(c, b, segs, n, src); break;
+    case 6: k_batch<128, 6><<<blocks, warps * 32, smem, s>>>(c, b, segs, n, src); break;
+    default: k_batch<1024, 1><<<blocks, warps * 32, smem, s>>>(c, b, segs, n, src);
+  }
   k_batch_close<<<b.n_clouds, 128, 0, s>>>(c, b, src);
   g_kernel_launches += 2;
   return cudaPeekAtLastError() == cudaSuccess ? DT_OK : DT_ECUDA;

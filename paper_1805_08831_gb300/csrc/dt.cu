@@ -2051,8 +2051,8 @@ int batch_enqueue_insert(dt_handle* h, int warps, uint64_t slots, int* src, cuda
 }
 
 // Points that the planned launches left (large cavities, long walks): one warp per cloud until
-// none is left; as long as some are inserted, or a bounded number of times if not.
-int batch_leftovers(dt_handle* h, int src, unsigned long long* totals, cudaStream_t s) {
+// none is left; as long as some are inserted, or a bounded number of times if not. *launches: how many.
+int batch_leftovers(dt_handle* h, int src, unsigned long long* totals, uint64_t* launches, cudaStream_t s) {
   Ctx c = batch_ctx(h);
   c.max_walk = std::max(c.max_walk, kLongWalkSteps);
   const BatchMem b = batch_mem(h);
@@ -2062,9 +2062,11 @@ int batch_leftovers(dt_handle* h, int src, unsigned long long* totals, cudaStrea
     if (totals[kBBig] > 0) {
       if (!h->bws && !realloc_dev(h->bws, kBatchBigWarps * batch_big_ws_bytes())) return DT_ENOMEM;
       if ((rc = batch_launch_big(c, b, h->bws, kBatchBigWarps, src, s)) != DT_OK) return rc;
+      ++*launches;
     }
     const auto& last = h->bplan.back();
     if ((rc = batch_launch(4, c, b, h->bsegs + last.first, (uint32_t)last.second, src, s)) != DT_OK) return rc;
+    ++*launches;
     src = 1 - src;
     batch_finish(c, b, src, s);
     if (cudaMemcpyAsync(totals, h->bstats, kBatchTotals * 8, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
@@ -2203,7 +2205,13 @@ int batch_impl(dt_handle* h, const double* xyz, const uint64_t* off, uint32_t nc
   cudaMemcpyAsync(st, h->bstats, sizeof(st), cudaMemcpyDeviceToHost, s);
   if (cudaStreamSynchronize(s) != cudaSuccess) return DT_ECUDA;
   if (bad) return DT_EINVAL;
-  if ((rc = batch_leftovers(h, src, st, s)) != DT_OK) return rc;
+  uint64_t launches = 0, most = 0;
+  if ((rc = batch_leftovers(h, src, st, &launches, s)) != DT_OK) return rc;
+  if (launches) cudaEventRecord(h->bev[3], s);  // they are part of the insertion
+  for (const auto& l : h->bplan) {
+    launches += l.second > 0;
+    most = std::max(most, l.second);
+  }
   h->bclouds_host.resize(nc);
   cudaMemcpyAsync(h->bclouds_host.data(), h->bclouds, nc * sizeof(BatchCloud), cudaMemcpyDeviceToHost, s);
   if (cudaStreamSynchronize(s) != cudaSuccess) return DT_ECUDA;
@@ -2230,15 +2238,16 @@ int batch_impl(dt_handle* h, const double* xyz, const uint64_t* off, uint32_t nc
   agg.sum_walk = st[kBWalk];
   agg.n_exact = st[kBExact];
   agg.n_sos = st[kBSos];
+  agg.n_big = st[kBLarge];
   agg.bump = used;
   std::memcpy(h->st_host, &agg, sizeof(agg));
   h->stats.ms_sort = ms_sort;
   h->stats.ms_insert = ms_ins;
-  h->stats.n_rounds = h->bplan.size();
+  h->stats.n_rounds = launches;
   h->stats.n_passes = 0;
   h->stats.n_clouds_degenerate = degenerate;
   h->stats.batch_warps = (uint64_t)warps;
-  h->stats.batch_min_blocks = warps <= 4 ? 4 : 1;
+  h->stats.batch_min_blocks = (uint64_t)batch_min_blocks(warps, most);
   h->stats.batch_alpha = h->alpha_async;
   h->stats.batch_graph = h->bgraph_used ? 1 : 0;
   // DT_EDEGENERATE only when no cloud could be triangulated

@@ -175,11 +175,10 @@ int async_launch_big(const Ctx& c, const AsyncIO& io, uint32_t* lock, const Inse
 // ---------------------------------------------------------------- batch.cu (dt_batch)
 uint32_t batch_hint_fine();     // fine hint cells per cloud
 uint32_t batch_hint_coarse();   // coarse hint cells per cloud
-int batch_cb();                 // bits per axis of a cloud's fine hint grid
 // Totals of a batch: inserted, conflicts, attempts, sum |C|, sum |B|, walk steps, large cavities
-// waiting, points waiting, duplicates met, exact and perturbed predicates.
+// waiting, points waiting, duplicates met, exact and perturbed predicates, large cavities inserted.
 enum BatchTotal { kBInserted, kBConflicts, kBAttempts, kBCavity, kBBall, kBWalk, kBBig, kBLeft, kBDups, kBExact, kBSos,
-                  kBatchTotals };
+                  kBLarge, kBatchTotals };
 // The batch's arrays: clouds and, by cloud, the state (allocator, queues, counters) and hint
 // grids; by vertex, flags and the lists of points carried over and of large cavities (a cloud
 // uses its own range); owner words; borrowed large-cavity workspaces; the FP32 error term.
@@ -202,6 +201,9 @@ struct BatchMem {
 bool batch_ready();  // the kernels' shared memory is set up (call before any capture)
 // A new mesh in every cloud: state, hints and flags, the first tetrahedra.
 void batch_init(const Ctx& c, const BatchMem& b, cudaStream_t s);
+// Resident blocks per SM that the kernel of a launch over n segments in blocks of `warps` warps is
+// built for.
+int batch_min_blocks(int warps, uint64_t n);
 // One launch over the segments segs[0, n) (x: cloud, y..z: vertices, w: index among the cloud's
 // segments | their number << 16), each after its share of the points of list `src`, and the close
 // of every cloud's allocator; what is not inserted goes to list 1 - src.

@@ -1,6 +1,8 @@
 """dt_batch: many independent clouds in one persistent launch, every cloud bit-exact against the
 oracle run on that cloud alone (the perturbed Delaunay triangulation is unique, so batching,
 block shape and round size cannot change it)."""
+import time
+
 import numpy as np
 import pytest
 
@@ -316,3 +318,30 @@ def test_many_clouds_take_no_more_memory_than_their_points_need():
         held = t.stats()["device_bytes"]
     points = 220 * len(xyz)  # records, order, lists: bytes a point beside the store's
     assert held < points + 1.5 * 60 * (8 * len(xyz) + 64 * 2000)
+
+
+def test_statistics_cover_the_launches_after_the_planned_ones():
+    """Cavities of up to 6000 tetrahedra are inserted by launches after the planned sequence: they
+    count as large cavities and as launches, and their time is in ms_insert."""
+    g = np.random.default_rng(5)
+    s = g.normal(size=(6000, 3))
+    shell = np.concatenate([s / np.linalg.norm(s, axis=1, keepdims=True), 0.01 * g.normal(size=(5, 3))])
+    seen = {}
+    for name, x in (("plain", synth.uniform_cube(len(shell), 3)), ("shell", shell)):
+        xd, off = torch.from_numpy(x).cuda(), np.array([0, len(x)])
+        with dt.Triangulation(seed=0) as t:
+            for _ in range(3):
+                torch.cuda.synchronize()
+                begin = time.perf_counter()
+                t.batch(xd, off)
+                wall = 1e3 * (time.perf_counter() - begin)
+            seen[name] = t.stats()
+        assert seen[name]["ms_sort"] + seen[name]["ms_insert"] > 0.6 * wall
+        assert seen[name]["batch_min_blocks"] == 4
+    assert seen["shell"]["n_rounds"] > seen["plain"]["n_rounds"]
+    # one at least: without a cavity beyond the borrowed workspaces there are no such launches
+    assert 1 <= seen["shell"]["n_big"] <= len(shell)
+    xyz, off = synth.batched_clouds(1500, 4, lo=500, hi=5000)  # more than 2432 segments in a launch
+    with dt.Triangulation(seed=0) as t:
+        t.batch(torch.from_numpy(xyz).cuda(), off)
+        assert t.stats()["batch_min_blocks"] == 6
