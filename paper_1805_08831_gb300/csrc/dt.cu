@@ -1677,12 +1677,11 @@ int insert_async(dt_handle* h, uint64_t base, uint64_t n, bool exact) {
     if ((rc = zero_queue(h, q)) != DT_OK) return rc;
   uint64_t given = 0;
   std::vector<uint32_t> cum;
-  std::vector<float> scale;
   for (int r = 0;; ++r) {
     const uint64_t b = r == 0 ? 0 : brio_round_end(r - 1);
     if (b >= n) break;
     const uint64_t e = std::min<uint64_t>(brio_round_end(r), n);
-    if (make_waves(h, (uint32_t)(base + b), (uint32_t)(base + e), r, base, cum, &scale) < 0) return DT_ECUDA;
+    if (make_waves(h, (uint32_t)(base + b), (uint32_t)(base + e), r, base, cum) < 0) return DT_ECUDA;
     uint64_t off = 0;
     for (size_t w = 0; w < cum.size(); ++w) {
       if ((rc = run_pass_async(h, c, h->wlist + off, cum[w] - off, h->queue[cur], h->st_host->q[cur], cur, other,

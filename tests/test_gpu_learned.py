@@ -139,6 +139,30 @@ def test_learned_schedule_gives_the_same_tets(trained, kind, n, seed):
     assert np.array_equal(got, ref)
 
 
+@pytest.mark.parametrize("use", ["defer", "both"])
+def test_deferral_splits_no_launch_of_the_asynchronous_engine(use, monkeypatch):
+    """Putting the points expected to lose after the rest of their wave is the round-based engine's
+    use of the prediction; the asynchronous engine's waves stay one launch each."""
+    x = synth.uniform_cube(60000, 4)
+    xd = torch.from_numpy(x).cuda()
+    params = np.random.default_rng(2).normal(scale=0.5, size=dt.DT_MLP_PARAMS).astype(np.float32)
+    with dt.Triangulation(seed=1, flags=dt.DT_FLAG_LOG) as t:
+        t.insert(xd)
+        f, _, _ = t.features(len(x))
+    logits = dt.mlp_forward(torch.from_numpy(params).cuda(), f)[:, 1]
+    monkeypatch.setenv("DT_RISK_LOGIT", str(float(logits.median())))  # half the points of every wave
+    launches, tets = [], []
+    for u in ("rank", use):
+        monkeypatch.setenv("DT_LEARN_USE", u)
+        with dt.Triangulation(seed=1, schedule=dt.DT_SCHED_LEARNED) as t:
+            t.load_model(params)
+            t.insert(xd)
+            launches.append(t.stats()["n_async"])
+            tets.append(t.tets_numpy())
+    assert np.array_equal(tets[0], tets[1])
+    assert launches[1] <= launches[0] + 6  # a drain's few launches vary from run to run
+
+
 def test_learned_schedule_without_a_model_is_refused():
     with dt.Triangulation(schedule=dt.DT_SCHED_LEARNED) as t:
         with pytest.raises(dt.DTError) as e:
