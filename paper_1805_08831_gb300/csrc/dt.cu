@@ -1092,7 +1092,8 @@ uint64_t device_bytes(const dt_handle* h) {
   if (h->async_borrow_ws) b += (uint64_t)kAsyncBorrow * (async_borrow_ws_bytes() + 4);
   if (h->hugemem) b += carve(nullptr, 4 * h->huge_c, h->huge_c, h->huge_c, 4 * h->huge_c, nullptr);
   b += h->cap_log * 3 + h->cap_feat * (8 + 2) * 4 + h->cap_risky * 2 + h->cap_cells * 4;
-  b += h->cap_bpts * 32 + h->cap_bclouds * sizeof(DevState) + h->cap_bsegs * sizeof(uint4);
+  b += h->cap_bpts * 17 + h->cap_bsegs * sizeof(uint4);             // a batch's cloud ids, flags, lists; segments
+  b += h->cap_bclouds * (sizeof(DevState) + sizeof(BatchCloud) + 8 + 48 + 4 * (batch_hint_fine() + batch_hint_coarse()));
   if (h->bws) b += (uint64_t)kBatchBigWarps * batch_big_ws_bytes();
   return b;
 }
@@ -1188,7 +1189,8 @@ int reserve_tets(dt_handle* h, uint64_t total_pts) {
 // The large-cavity workspaces that the asynchronous kernels' warps borrow.
 int reserve_borrow(dt_handle* h) {
   if (h->async_borrow_ws) return DT_OK;
-  if (cudaMalloc(&h->async_borrow_busy, kAsyncBorrow * sizeof(unsigned int)) != cudaSuccess) return DT_ENOMEM;
+  if (!h->async_borrow_busy && cudaMalloc(&h->async_borrow_busy, kAsyncBorrow * sizeof(unsigned int)) != cudaSuccess)
+    return DT_ENOMEM;
   cudaMemsetAsync(h->async_borrow_busy, 0, kAsyncBorrow * sizeof(unsigned int), h->stream);
   return cudaMalloc(&h->async_borrow_ws, (size_t)kAsyncBorrow * async_borrow_ws_bytes()) == cudaSuccess ? DT_OK
                                                                                                         : DT_ENOMEM;
@@ -1213,32 +1215,36 @@ int reserve_huge(dt_handle* h) {
 }
 
 int reserve_rounds(dt_handle* h, uint64_t qcap) {
-  if (!h->cand_p) {
+  cudaStream_t s = h->stream;
+  if (!h->cand_p) {  // the last of them: without it the next call makes those that are missing
     h->Rmax = 1u << 19;
-    uint64_t R = h->Rmax;
-    if (cudaMalloc(&h->cand_p, R * 4) || cudaMalloc(&h->cand_t, R * 4) || cudaMalloc(&h->cand_status, R * 4) ||
-        cudaMalloc(&h->cand_nc, R * 4) || cudaMalloc(&h->cand_nb, R * 4) ||
-        cudaMalloc(&h->scratch, R * kScratchStride * 4))
-      return DT_ENOMEM;
+    const uint64_t R = h->Rmax;
     h->bigstride = big_stride();
-    if (cudaMalloc(&h->bigmem, h->bigstride * kBigR)) return DT_ENOMEM;
-    if (cudaMalloc(&h->medscratch, (size_t)kBigR * (kMedCN + kMedFN) * 4)) return DT_ENOMEM;
+    h->ctastride = cta_stride();
+    if (grow(h->cand_t, 0, R, s) != cudaSuccess || grow(h->cand_status, 0, R, s) != cudaSuccess ||
+        grow(h->cand_nc, 0, R, s) != cudaSuccess || grow(h->cand_nb, 0, R, s) != cudaSuccess ||
+        grow(h->scratch, 0, R * kScratchStride, s) != cudaSuccess ||
+        grow(h->bigmem, 0, h->bigstride * kBigR, s) != cudaSuccess ||
+        grow(h->medscratch, 0, (uint64_t)kBigR * (kMedCN + kMedFN), s) != cudaSuccess ||
+        grow(h->ctamem, 0, h->ctastride * kCtaWarps, s) != cudaSuccess)
+      return DT_ENOMEM;
     const int msmem = (int)(kMedWarps * med_stride());
     if (cudaFuncSetAttribute(k_cavity<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, msmem) != cudaSuccess ||
         cudaFuncSetAttribute(k_insert<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, msmem) != cudaSuccess)
       return DT_ECUDA;
-    h->ctastride = cta_stride();
-    if (cudaMalloc(&h->ctamem, h->ctastride * kCtaWarps)) return DT_ENOMEM;
+    if (grow(h->cand_p, 0, R, s) != cudaSuccess) return DT_ENOMEM;
   }
   if (!h->wave_cum && cudaMalloc(&h->wave_cum, 256 * 4) != cudaSuccess) return DT_ENOMEM;
   if (!h->wave_hist && cudaMalloc(&h->wave_hist, 512 * 4) != cudaSuccess) return DT_ENOMEM;
   if (qcap > h->cap_w) {
+    h->cap_w = 0;
     cudaFree(h->wlist);
     h->wlist = nullptr;
     if (cudaMalloc(&h->wlist, qcap * 4) != cudaSuccess) return DT_ENOMEM;
     h->cap_w = qcap;
   }
   if (qcap > h->cap_q) {
+    h->cap_q = 0;
     for (auto& qb : h->queue) {
       cudaFree(qb);
       qb = nullptr;
@@ -1879,6 +1885,7 @@ int batch_reserve(dt_handle* h, uint64_t N, uint32_t nc, uint64_t T) {
   if (reserve_points(h, N) != DT_OK) return DT_ENOMEM;
   if (order_ws_reserve(h->ows, N) != cudaSuccess) return DT_ENOMEM;
   if (N > h->cap_bpts) {
+    h->cap_bpts = 0;
     if (!realloc_dev(h->bcid, N) || !realloc_dev(h->bdup, N) || !realloc_dev(h->blist_a, N) ||
         !realloc_dev(h->blist_b, N) || !realloc_dev(h->blist_big, N))
       return DT_ENOMEM;
