@@ -188,12 +188,31 @@ def test_slab_bit_exact():
     assert_same(got, ref)
 
 
-def test_schedule_does_not_change_tets():
-    x = synth.uniform_cube(20000, 8)
+@pytest.mark.parametrize("kind", ["uniform", "degenerate"])
+def test_schedule_does_not_change_tets(kind, monkeypatch):
+    """Other schedules, the same set: the round-based engine's segments per round, the asynchronous
+    engine's warps, wave sizes and starts, and the order that another seed gives."""
+    x = synth.make(kind, 20000, 8)
     ref, _ = oracle.delaunay(x, seed=1)
-    for seg in (1, 7, 64, 4096):
-        got, _ = gpu_tets(x, seed=1, segments=seg)
+    rounds = set()
+    for warps, gamma, ball in ((1, 2.0, 1), (7, 2.0, 1), (64, 0.3, 1), (4096, 2.0, 0), (4096, 8.0, 1)):
+        monkeypatch.setenv("DT_ASYNC_WARPS", str(warps))
+        monkeypatch.setenv("DT_GAMMA_ASYNC", str(gamma))
+        monkeypatch.setenv("DT_ASYNC_BALL_START", str(ball))
+        got, st = gpu_tets(x, seed=1)
         assert_same(got, ref)
+        assert st["n_inserted_async"] > 0
+        if warps == 1:
+            assert st["n_conflicts"] == 0
+    for name in ("DT_ASYNC_WARPS", "DT_GAMMA_ASYNC", "DT_ASYNC_BALL_START"):
+        monkeypatch.delenv(name)
+    monkeypatch.setenv("DT_ASYNC", "0")
+    for seg in (1, 7, 64, 4096):
+        got, st = gpu_tets(x, seed=1, segments=seg)
+        assert_same(got, ref)
+        rounds.add(st["n_rounds"])
+    assert len(rounds) == 4  # each a schedule of its own
+    monkeypatch.delenv("DT_ASYNC")
     got, _ = gpu_tets(x, seed=12345)
     assert_same(got, ref)
 
