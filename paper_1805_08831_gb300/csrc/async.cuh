@@ -117,8 +117,8 @@ struct AWS : AWSTail<kHashN, kFMaxN, kEdgeSlots> {
 };
 
 // Shared-memory workspace of the main kernel (cavities of up to 64 tetrahedra and 60 boundary
-// facets), the global-memory one a warp borrows for a larger cavity (145 KB), and that of the
-// large-cavity kernel (1.6 MB: the sphere's empty interior, a surface's first inner points).
+// facets), the global-memory one a warp borrows for a larger cavity (135 KB), and that of the
+// large-cavity kernel (1.14 MB: the sphere's empty interior, a surface's first inner points).
 template <bool kCache, bool kLocal = false>
 using SmallWST = AWS<256, 64, 64, 60, 0, kCache, kLocal>;
 template <bool kCache, bool kLocal = false>

@@ -1661,9 +1661,9 @@ int run_brio_round(dt_handle* h, uint32_t vbegin, uint32_t vend, int round, uint
 // 3 % of the points it was given (and more than a few), the kernels with the exact stages do the
 // rest of the call. They hold twice the registers, so half the warps are resident; but a point
 // handed on is searched for twice, and the list of them, inserted at once, loses often (a
-// degenerate mix hands on 5 to 10 % of each wave). 1e6 points of it take 118 ms with the line at
-// a tenth, 95 at 5 %, 88 at 3 %, 89 at 1.5 % and 86 at 0.7 %; a slab of 1e6, which hands on 0.6 %,
-// takes 29.4 ms down to 1.5 % and 32.7 at 0.7 %; uniform clouds hand on 0.2 %.
+// degenerate mix hands on 5 to 10 % of each wave). 1e6 points of it take 80 ms with the line at a
+// tenth, 75 at 5 % and at 3 %, 73 at 1.5 % and at 0.7 %; a slab of 1e6, which hands on 0.6 %, takes
+// 28 ms down to 1.5 % and 31 at 0.7 %; uniform clouds hand on 0.2 %.
 bool handoffs_decide(dt_handle* h, uint64_t given) {
   const uint64_t ne = h->st_host->q[kQExact];
   return ne >= h->async_handoff_min && (double)ne > h->async_handoff_frac * (double)given;

@@ -211,10 +211,10 @@ static __device__ __noinline__ int ex_det3(const Ex2* r0, const Ex2* r1, const E
 // What bounds it is the fetch of its instructions, run by few lanes of a warp and seldom enough to
 // be evicted in between: so the code is short (loops over the terms, the determinant of three rows
 // and the scaling out of line, one copy for both predicates), without branches on signs or zeros.
-// The degenerate mix of 1e6 points takes 73 ms, the box surface of 48 intervals with its
-// refinement 74; the same arithmetic unrolled, with shared 2 x 2 minors, 88 and 79 (an insphere
-// took 58,000 cycles); terms formed one by one as sign and magnitude about 100 and 89. Run before
-// the FP64 filter it takes 70 and 82.
+// Measured one after the other on one device: the degenerate mix of 1e6 points took 73 ms and the box
+// surface of 48 intervals with its refinement 74 so, 88 and 79 with the same arithmetic unrolled and
+// shared 2 x 2 minors (an insphere took 58,000 cycles), about 100 and 89 with terms formed one by one
+// as sign and magnitude, and 70 and 82 with this stage ahead of the FP64 filter.
 using u128 = unsigned __int128;
 using s128 = __int128;
 
