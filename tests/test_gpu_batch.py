@@ -1,4 +1,4 @@
-"""dt_batch: many independent clouds in one persistent launch, every cloud bit-exact against the
+"""dt_batch: many independent clouds in one sequence of launches, every cloud bit-exact against the
 oracle run on that cloud alone (the perturbed Delaunay triangulation is unique, so batching,
 block shape and round size cannot change it)."""
 import time
